@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "hgmm_internal.cuh"
+#include "hgmm_levels.cuh"
 
 using namespace hgmm;
 
@@ -33,7 +34,7 @@ void clear_prof(hgmm_tree* t) {
 }
 
 const char* const kKernelNames[HGMM_PROF_KERNELS] = {
-    "root_partial", "root_final", "init_children", "make_items", "fill_items", "estep",
+    "root_partial", "build_levels", "init_children", "make_items", "fill_items", "estep",
     "mstep", "assign", "child_offsets", "scatter", "finalize", "reg_init", "register",
     "reg_mstep", "copy_T", "labels"};
 
@@ -47,7 +48,7 @@ void free_tree(hgmm_tree* t) {
     if (t->cap_stream) cudaStreamDestroy(t->cap_stream);
     void* ptrs[] = {t->est, t->stat, t->seg_start, t->seg_count, t->pts[0], t->pts[1],
                     t->codes, t->items, t->item_range, t->meta, t->partials, t->item_cnt,
-                    t->item_off, t->slice_tot, t->root, t->root_part, t->root_counter, t->em_cnt, t->mslices, t->mcnt, t->status, t->reg_acc, t->reg_acc2, t->reg_part,
+                    t->item_off, t->slice_tot, t->root, t->root_part, t->root_counter, t->em_cnt, t->mslices, t->mcnt, t->lv_part, t->lv_slices, t->lv_cnt, t->status, t->reg_acc, t->reg_acc2, t->reg_part,
                     t->reg_bar, t->reg_T, t->reg_Rt, t->reg_dbg, t->reg_obj, t->rnode, t->trace, t->stage_tgt,
                     t->stage_src, t->stage_T};
     for (void* p : ptrs)
@@ -159,6 +160,16 @@ int hgmm_tree_create(int64_t max_points, int32_t max_depth, hgmm_tree** out) {
     good &= dalloc(&t->em_cnt, level_size(std::max(0, max_depth - 1)) + 1);
     good &= dalloc(&t->mslices, int64_t(MSTEP_SLICED_PARENTS) * MSTEP_SLICES * NPART);
     good &= dalloc(&t->mcnt, MSTEP_SLICED_PARENTS);
+    // the one-launch build takes clouds of up to a few hundred thousand
+    // points, also in a tree made for more
+    t->levels_ok = levels_smem_attr();
+    if (!t->levels_ok) cudaGetLastError();  // the level-wide launches then build every cloud
+    if (t->levels_ok) {
+        t->lv_slots = levels_slots(std::min<int64_t>(max_points, int64_t(4 * TILE) * t->est_grid));
+        good &= dalloc(&t->lv_part, 2 * t->lv_slots * NPART);
+        good &= dalloc(&t->lv_slices, 2 * (t->lv_slots / 8 + 1) * NPART);
+        good &= dalloc(&t->lv_cnt, levels_counters());
+    }
     good &= dalloc(&t->status, 1);
     good &= dalloc(&t->reg_acc, 4 * ACC_REPLICAS * t->max_nodes);
     good &= dalloc(&t->reg_acc2, 6 * t->max_nodes);

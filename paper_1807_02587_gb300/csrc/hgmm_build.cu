@@ -26,6 +26,7 @@
 
 #include "hgmm_dev.cuh"
 #include "hgmm_async.cuh"
+#include "hgmm_levels.cuh"
 
 namespace hgmm {
 
@@ -571,11 +572,6 @@ using namespace hgmm;
         }                                                     \
     } while (0)
 
-// levels with at least this many parents, of at most LOCAL_EM_POINTS points
-// on average, run their EM parent-locally (one CTA per parent)
-constexpr int LOCAL_EM_PARENTS = 256;
-constexpr int64_t LOCAL_EM_POINTS = 2048;
-
 // Whether est_grid CTAs of the cooperative EM kernel fit on the device at
 // once (a cooperative launch needs them co-resident).
 // k_estep's dynamic shared memory plus its static part exceeds the 48 KB
@@ -603,16 +599,51 @@ int hgmm_build_impl(hgmm_tree* t, const float4* pts, int64_t n64, int depth,
                     const hgmm_params& p, cudaStream_t s) {
     const int n = int(n64);
     const int G = t->est_grid;
-    {
+    const float4* cur = pts;
+    const int* perm_prev = nullptr;
+    const bool comp = p.precision == 0;
+    // clouds whose points fit the CTAs' shared memory: the first levels (all
+    // of them up to depth 4) in one launch
+    const int taken = comp && t->levels_ok ? levels_taken(n64, depth, G) : 0;
+    if (taken > 0) {
+        LevelsArgs a;
+        a.pts = pts;
+        a.n = n;
+        a.levels = taken;
+        a.em_iters = p.em_iters;
+        a.stop_level = p.debug_stop_level;
+        a.stop_iters = p.debug_stop_iters;
+        a.n_min = p.n_min;
+        a.lam_c = p.lam_c;
+        a.eps_rel = p.eps_rel;
+        a.est = t->est;
+        a.stat = t->stat;
+        a.rnode = t->rnode;
+        a.seg_start = t->seg_start;
+        a.seg_count = t->seg_count;
+        a.root = t->root;
+        a.root_part = t->root_part;
+        for (int k = 0; k < 2; ++k) a.buf[k] = t->pts[k];
+        for (int k = 0; k < HGMM_MAX_DEPTH; ++k) a.perm[k] = t->perm[k];
+        a.part = t->lv_part;
+        a.part_stride = t->lv_slots * NPART;
+        a.slices = t->lv_slices;
+        a.slice_stride = (t->lv_slots / 8 + 1) * NPART;
+        a.item_cnt = t->item_cnt;
+        a.cnt = t->lv_cnt;
+        a.status = t->status;
+        ProfScope ps_(t, K_LEVELS, s);
+        if (int rc = levels_launch(a, G, s)) return rc;
+        if (taken == depth || (p.debug_stop_level > 0 && p.debug_stop_level <= taken)) return HGMM_OK;
+        cur = t->pts[(taken - 1) & 1];
+        perm_prev = t->perm[taken - 1];
+    } else {
         ProfScope ps_(t, K_ROOT_PARTIAL, s);
         k_root<<<G, 256, 0, s>>>(pts, n, p.eps_rel, t->root_part, t->root_counter, t->root,
                                  t->status);
     }
     HGMM_LAUNCH_CHECK();
-    const float4* cur = pts;
-    const int* perm_prev = nullptr;
-    const bool comp = p.precision == 0;
-    for (int l = 0; l < depth; ++l) {
+    for (int l = taken; l < depth; ++l) {
         const int n_par = l == 0 ? 1 : int(level_size(l - 1));
         const int64_t off = level_offset(l);
         NodeEst* est_lvl = t->est + off;

@@ -48,6 +48,7 @@ __device__ __forceinline__ void root_identity(float* f) {
 struct RootSmem {
     float sm[8][25];
     float gs[16][25];
+    float tot[25];
 };
 
 // CTA `cta` of `ncta` sums its share of the points into out[0..24].
@@ -110,74 +111,148 @@ __device__ __forceinline__ void root_partial_cta(const float4* __restrict__ pts,
 }
 
 // One CTA (>= 256 threads) reduces the `nparts` partials (stride 32 floats)
-// in a fixed order -- 16 half-warp groups, then one thread -- and writes the
-// FP64 root record with its eigen-decomposition.
-__device__ __forceinline__ void root_final_cta(const float* __restrict__ part, int nparts,
-                                               const float4* __restrict__ pts, int n, float eps_rel,
-                                               RootDev* __restrict__ root, int* __restrict__ status,
-                                               RootSmem& rs) {
+// in a fixed order -- 16 half-warp groups, then one thread per value -- and
+// its first warp writes the FP64 root record with its eigen-decomposition.
+// Latency alone bounds it (one CTA, dependent FP64 chains), so the group
+// sums, the conversions and the moments take one lane per value: an FP64 warp
+// instruction costs the same whatever its active lanes.  On 93k points the
+// root statistics took 48.8 us with one thread doing all of it and take 25 us
+// (20 of them here, most of it the eigen-decomposition).  `root` may be
+// shared memory.
+__device__ __forceinline__ void root_final_cta(const float* part, int nparts, const float4* pts, int n,
+                                               float eps_rel, RootDev* root, int* status, RootSmem& rs) {
     if (threadIdx.x < 256) {
         const int grp = threadIdx.x >> 4, it = threadIdx.x & 15;
         float a = 0.f, b = 0.f;
         if (it >= 9 && it < 12) a = CUDART_INF_F;
         if (it >= 12 && it < 15) a = -CUDART_INF_F;
         int cntb = 0;
-#pragma unroll 4
-        for (int blk = grp; blk < nparts; blk += 16) {
-            const float* o = part + 32 * blk;
-            if (it < 9) pair_add(a, b, __ldcg(o + 2 * it), __ldcg(o + 2 * it + 1));
-            else if (it < 12) a = fminf(a, __ldcg(o + 18 + it - 9));
-            else if (it < 15) a = fmaxf(a, __ldcg(o + 21 + it - 12));
-            else cntb += __float_as_int(__ldcg(o + 24));
+        // this value's word(s) of a partial; a one-word value reads it twice
+        const int o0 = it < 9 ? 2 * it : it + 9, o1 = it < 9 ? o0 + 1 : o0;
+        for (int b0 = grp; b0 < nparts; b0 += 16 * 8) {
+            float x[8], y[8];  // eight partials in flight
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int blk = min(b0 + 16 * u, nparts - 1);
+                x[u] = __ldcg(part + 32 * blk + o0);
+                y[u] = __ldcg(part + 32 * blk + o1);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (b0 + 16 * u >= nparts) break;
+                if (it < 9) pair_add(a, b, x[u], y[u]);
+                else if (it < 12) a = fminf(a, x[u]);
+                else if (it < 15) a = fmaxf(a, x[u]);
+                else cntb += __float_as_int(x[u]);
+            }
         }
         if (it < 9) { rs.gs[grp][2 * it] = a; rs.gs[grp][2 * it + 1] = b; }
-        else if (it < 12) rs.gs[grp][18 + it - 9] = a;
-        else if (it < 15) rs.gs[grp][21 + it - 12] = a;
+        else if (it < 15) rs.gs[grp][it + 9] = a;
         else rs.gs[grp][24] = __int_as_float(cntb);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float F[25];
-        root_identity(F);
-        for (int w = 0; w < 16; ++w) root_combine(F, rs.gs[w]);
-        if (__float_as_int(F[24]) > 0) atomicOr(status, ST_NONFINITE);
+    if (threadIdx.x < 16) {
+        const int it = threadIdx.x;
+        if (it < 9) {
+            float a = 0.f, b = 0.f;
+#pragma unroll
+            for (int w = 0; w < 16; ++w) pair_add(a, b, rs.gs[w][2 * it], rs.gs[w][2 * it + 1]);
+            rs.tot[2 * it] = a;
+            rs.tot[2 * it + 1] = b;
+        } else if (it < 15) {
+            float a = rs.gs[0][it + 9];
+#pragma unroll
+            for (int w = 1; w < 16; ++w) a = it < 12 ? fminf(a, rs.gs[w][it + 9]) : fmaxf(a, rs.gs[w][it + 9]);
+            rs.tot[it + 9] = a;
+        } else {
+            int c = 0;
+#pragma unroll
+            for (int w = 0; w < 16; ++w) c += __float_as_int(rs.gs[w][24]);
+            rs.tot[24] = __int_as_float(c);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        if (lane == 0 && status && __float_as_int(rs.tot[24]) > 0) atomicOr(status, ST_NONFINITE);
         const float4 z0 = pts[0];
         const double nn = double(n);
         const double rn = rcp_f64(nn);  // one reciprocal instead of nine divisions
-        double m1[3], m2[6];
-        for (int a = 0; a < 3; ++a) m1[a] = (double(F[2 * a]) + double(F[2 * a + 1])) * rn;
-        for (int v = 0; v < 6; ++v) m2[v] = (double(F[6 + 2 * v]) + double(F[7 + 2 * v])) * rn;
-        root->n = nn;
-        root->mu[0] = double(z0.x) + m1[0];
-        root->mu[1] = double(z0.y) + m1[1];
-        root->mu[2] = double(z0.z) + m1[2];
+        // lane v < 9: moment v about the first point over n
+        const int v = lane < 9 ? lane : 8;
+        const double m = (double(rs.tot[2 * v]) + double(rs.tot[2 * v + 1])) * rn;
+        // lane v < 6: covariance entry v (xx xy xz yy yz zz)
+        const int r = lane < 3 ? 0 : (lane < 5 ? 1 : 2);
+        const int c = lane < 3 ? lane : (lane == 3 ? 1 : 2);
+        const double m2 = __shfl_sync(FULL, m, 3 + (lane < 6 ? lane : 5));
+        const double mr = __shfl_sync(FULL, m, r), mc = __shfl_sync(FULL, m, c);
+        const double e = m2 - mr * mc;
+        if (lane < 3) root->mu[lane] = double(lane == 0 ? z0.x : (lane == 1 ? z0.y : z0.z)) + m;
+        if (lane < 6) root->S[lane] = e;
+        const int a = lane < 3 ? lane : 2;
+        const double d = double(rs.tot[21 + a]) - double(rs.tot[18 + a]);
+        const double dx = __shfl_sync(FULL, d, 0), dy = __shfl_sync(FULL, d, 1), dz = __shfl_sync(FULL, d, 2);
         double S[6];
-        S[0] = m2[0] - m1[0] * m1[0];
-        S[1] = m2[1] - m1[0] * m1[1];
-        S[2] = m2[2] - m1[0] * m1[2];
-        S[3] = m2[3] - m1[1] * m1[1];
-        S[4] = m2[4] - m1[1] * m1[2];
-        S[5] = m2[5] - m1[2] * m1[2];
-        for (int v = 0; v < 6; ++v) root->S[v] = S[v];
-        double e2 = 0.0;
-        for (int a = 0; a < 3; ++a) {
-            const double d = double(F[21 + a]) - double(F[18 + a]);
-            e2 += d * d;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) S[k] = __shfl_sync(FULL, e, k);
+        if (lane == 0) {
+            root->n = nn;
+            double e2 = 0.0;
+            e2 += dx * dx;
+            e2 += dy * dy;
+            e2 += dz * dz;
+            root->extent = sqrt(e2);
+            const double q = double(eps_rel) * root->extent;
+            root->eps = q * q;
+            eig3(S, root->lam, root->V);
         }
-        root->extent = sqrt(e2);
-        const double e = double(eps_rel) * root->extent;
-        root->eps = e * e;
-        eig3(S, root->lam, root->V);
     }
     __syncthreads();
 }
 
 // ===================================================================== init
-// PCA-octant initial child c of parent p (level-0 parent = the root): mean
-// mu_p + 1/2 sum_a s_a sqrt(lambda_a) v_a (s_a = +1 iff bit a of c), covariance
-// Sigma_p / 4 + eps I, weight 1/8.  Children of a parent that is dead or
-// holds no points are dead.  The parent's eigen-decomposition was computed
-// when it was finalised.
+// PCA-octant initial child c of a parent with Gaussian (mu_p, S_p) and
+// eigen-decomposition (lam, V): mean mu_p + 1/2 sum_a s_a sqrt(lambda_a) v_a
+// (s_a = +1 iff bit a of c), covariance Sigma_p / 4 + eps I, weight 1/8; dead
+// if the parent is dead or holds no points (`alive` false).  The FP32
+// constants go to ce, the FP64 record to cs (if not null).
+__device__ __forceinline__ void init_child_of(bool alive, const double (&mu_p)[3], const double (&S_p)[6],
+                                              const double (&lam)[3], const double (&V)[9], double eps, int c,
+                                              NodeStat* cs, NodeEst& ce, int* status) {
+    if (!alive) {
+        if (cs) {
+            cs->live = 0;
+            cs->pi = 0.0;
+            for (int a = 0; a < 3; ++a) cs->mu[a] = mu_p[a];
+            for (int v = 0; v < 6; ++v) cs->S[v] = 0.0;
+        }
+        dead_est(mu_p, ce);
+        return;
+    }
+    double mu[3];
+    for (int a = 0; a < 3; ++a) {
+        double acc = mu_p[a];
+        for (int b = 0; b < 3; ++b) {
+            const double sgn = ((c >> b) & 1) ? 1.0 : -1.0;
+            const double lb = fmax(lam[b], 0.0);
+            acc += sgn * 0.5 * (lb > 0.0 ? lb * rsqrt_f64(lb) : 0.0) * V[a * 3 + b];
+        }
+        mu[a] = acc;
+    }
+    double S[6];
+    for (int v = 0; v < 6; ++v) S[v] = S_p[v] * 0.25;
+    S[0] += eps; S[3] += eps; S[5] += eps;
+    if (cs) {
+        cs->live = 1;
+        cs->pi = 0.125;
+        for (int a = 0; a < 3; ++a) cs->mu[a] = mu[a];
+        for (int v = 0; v < 6; ++v) cs->S[v] = S[v];
+    }
+    if (!pack_est(0.125, mu, S, eps, 0.f, ce)) atomicOr(status, ST_CHOL);
+}
+
+// Initial child c of parent p of a level (level-0 parent = the root).  The
+// parent's eigen-decomposition was computed when it was finalised.
 __device__ __forceinline__ void init_child(int level, int p, int c, const RootDev* __restrict__ root,
                                            NodeStat* __restrict__ stat, NodeEst* __restrict__ est,
                                            const int* __restrict__ seg_count,
@@ -198,35 +273,7 @@ __device__ __forceinline__ void init_child(int level, int p, int c, const RootDe
         alive = ps.live && seg_count[g] > 0;
     }
     const int64_t gc = d_level_offset(level) + 8 * int64_t(p) + c;
-    NodeStat& cs = stat[gc];
-    NodeEst& ce = est[gc];
-    if (!alive) {
-        cs.live = 0;
-        cs.pi = 0.0;
-        for (int a = 0; a < 3; ++a) cs.mu[a] = mu_p[a];
-        for (int v = 0; v < 6; ++v) cs.S[v] = 0.0;
-        dead_est(mu_p, ce);
-        return;
-    }
-    const double eps = root->eps;
-    double mu[3];
-    for (int a = 0; a < 3; ++a) {
-        double acc = mu_p[a];
-        for (int b = 0; b < 3; ++b) {
-            const double sgn = ((c >> b) & 1) ? 1.0 : -1.0;
-            const double lb = fmax(lam[b], 0.0);
-            acc += sgn * 0.5 * (lb > 0.0 ? lb * rsqrt_f64(lb) : 0.0) * V[a * 3 + b];
-        }
-        mu[a] = acc;
-    }
-    double S[6];
-    for (int v = 0; v < 6; ++v) S[v] = S_p[v] * 0.25;
-    S[0] += eps; S[3] += eps; S[5] += eps;
-    cs.live = 1;
-    cs.pi = 0.125;
-    for (int a = 0; a < 3; ++a) cs.mu[a] = mu[a];
-    for (int v = 0; v < 6; ++v) cs.S[v] = S[v];
-    if (!pack_est(0.125, mu, S, eps, 0.f, ce)) atomicOr(status, ST_CHOL);
+    init_child_of(alive, mu_p, S_p, lam, V, root->eps, c, &stat[gc], est[gc], status);
 }
 
 // ==================================================================== items
@@ -711,34 +758,40 @@ __device__ __forceinline__ void estep_items_warp(const float4* __restrict__ pts,
 // S2/S0 - d d^T + eps I with d = S1/S0 (moments about the child's FP32
 // mean); pi = S0 / n_p.  mom: 80 doubles (child c's ten at c * NMOM), shared
 // or global.  All 32 lanes of the warp call it.
-__device__ __forceinline__ void child_mstep_quad(int level, int n, int p, const double* mom,
-                                                 const int* __restrict__ seg_count,
-                                                 const RootDev* __restrict__ root, float n_min,
-                                                 NodeStat* __restrict__ stat, NodeEst* __restrict__ est,
-                                                 int* __restrict__ status) {
+// est8: the children's FP32 constants (read for the current means, then
+// rewritten); was_live: whether this quad's child was live; stat8 (FP64
+// records) and copy8 (a second place for the constants) may be null.
+// Returns whether the quad's child is live.
+__device__ __forceinline__ bool child_mstep_at(double n_p, const double* mom, double eps, float n_min,
+                                               bool was_live, NodeEst* est8, NodeStat* stat8, NodeEst* copy8,
+                                               int* status) {
     const int lane = threadIdx.x & 31, c = lane >> 2, r = lane & 3, q0 = lane & ~3;
     const unsigned qm = 0xFu << q0;
-    const int64_t g = d_level_offset(level) + 8 * int64_t(p) + c;
-    NodeStat& cs = stat[g];
-    NodeEst& ce = est[g];
+    NodeEst& ce = est8[c];
     const double* m = mom + c * NMOM;
     const double S0 = m[0];
-    const double n_p = level == 0 ? double(n) : double(seg_count[d_level_offset(level - 1) + p]);
     // a child below n_min expected points dies; if all eight die the parent
     // stays a leaf (its points keep zero posteriors from then on)
-    const bool live = cs.live && S0 >= double(n_min) && S0 > 0.0;  // the same on the quad
+    const bool live = was_live && S0 >= double(n_min) && S0 > 0.0;  // the same on the quad
     if (!live) {
         if (r == 0) {
-            cs.live = 0;
-            cs.pi = 0.0;
+            if (stat8) {
+                stat8[c].live = 0;
+                stat8[c].pi = 0.0;
+            }
             ce.a.w = -CUDART_INF_F;
             ce.b = make_float4(0.f, 0.f, 0.f, 0.f);
             ce.c.x = 0.f;
             ce.c.y = 0.f;
+            if (copy8) {
+                copy8[c].a.w = -CUDART_INF_F;
+                copy8[c].b = make_float4(0.f, 0.f, 0.f, 0.f);
+                copy8[c].c.x = 0.f;
+                copy8[c].c.y = 0.f;
+            }
         }
-        return;
+        return false;
     }
-    const double eps = root->eps;
     const double rx = rcp_f64(r == 1 ? n_p : S0);
     const double inv = __shfl_sync(qm, rx, q0);
     const double rnp = __shfl_sync(qm, rx, q0 | 1);
@@ -765,10 +818,13 @@ __device__ __forceinline__ void child_mstep_quad(int level, int n, int p, const 
     S[4] = __shfl_sync(qm, e1, q0);
     S[5] = __shfl_sync(qm, e1, q0 | 1);
     const double pi = S0 * rnp;
-    if (r == 0) cs.pi = pi;
-    if (r < 3) cs.mu[r] = mua;
-    cs.S[r] = e0;
-    if (r < 2) cs.S[r + 4] = e1;
+    if (stat8) {
+        NodeStat& cs = stat8[c];
+        if (r == 0) cs.pi = pi;
+        if (r < 3) cs.mu[r] = mua;
+        cs.S[r] = e0;
+        if (r < 2) cs.S[r + 4] = e1;
+    }
     // Cholesky of Sigma (every lane of the quad), with the diagonal loading
     // of pack_est when it is not positive definite
     double L[6], R[3];
@@ -812,7 +868,25 @@ __device__ __forceinline__ void child_mstep_quad(int level, int n, int p, const 
         ce.a = make_float4(mx, my, mz, C);
         ce.b = make_float4(w00, w10, w11, w20);
         ce.c = make_float4(w21, w22, 0.f, 0.f);
+        if (copy8) {
+            copy8[c].a = make_float4(mx, my, mz, C);
+            copy8[c].b = make_float4(w00, w10, w11, w20);
+            copy8[c].c = make_float4(w21, w22, 0.f, 0.f);
+        }
     }
+    return true;
+}
+
+// child_mstep_at of parent p's children in the tree's own arrays.
+__device__ __forceinline__ void child_mstep_quad(int level, int n, int p, const double* mom,
+                                                 const int* __restrict__ seg_count,
+                                                 const RootDev* __restrict__ root, float n_min,
+                                                 NodeStat* __restrict__ stat, NodeEst* __restrict__ est,
+                                                 int* __restrict__ status) {
+    const int64_t g0 = d_level_offset(level) + 8 * int64_t(p);
+    const double n_p = level == 0 ? double(n) : double(seg_count[d_level_offset(level - 1) + p]);
+    child_mstep_at(n_p, mom, root->eps, n_min, stat[g0 + ((threadIdx.x & 31) >> 2)].live != 0, est + g0, stat + g0,
+                   nullptr, status);
 }
 
 struct MstepSmem {

@@ -97,7 +97,7 @@ struct RootDev {
 };
 
 enum KernelId {
-    K_ROOT_PARTIAL, K_ROOT_FINAL, K_INIT, K_MAKE_ITEMS, K_FILL_ITEMS, K_ESTEP, K_MSTEP,
+    K_ROOT_PARTIAL, K_LEVELS, K_INIT, K_MAKE_ITEMS, K_FILL_ITEMS, K_ESTEP, K_MSTEP,
     K_ASSIGN, K_OFFSETS, K_SCATTER, K_FINALIZE, K_REG_INIT, K_DESCEND, K_REG_MSTEP, K_COPY_T,
     K_LABELS, K_COUNT
 };
@@ -143,6 +143,7 @@ struct hgmm_tree {
     int64_t max_nodes = 0;
     int est_grid = 0;   // CTAs of the persistent build E-step
     int em_coop_grid = 0;  // co-resident CTAs of the cooperative per-level EM kernel (0: unavailable)
+    bool levels_ok = false;  // the one-launch build of the levels fits on the device
     int reg_grid = 0;       // CTAs of the registration kernel, two per SM
     int reg_grid_wide = 0;  // three per SM, for large sources (0: not co-resident)
     // last build
@@ -173,6 +174,11 @@ struct hgmm_tree {
     unsigned* em_cnt = nullptr;  // cooperative EM: per-parent arrivals + done counter
     float2* mslices = nullptr;   // M-step slice sums (sliced levels: parents x slices x NPART)
     unsigned* mcnt = nullptr;    // M-step slice arrivals per parent (zero between launches)
+    // one-launch build of the levels (hgmm_levels.cu)
+    float2* lv_part = nullptr;   // 2 x lv_slots x NPART
+    float2* lv_slices = nullptr; // 2 x (lv_slots / 8 + 1) x NPART
+    int64_t lv_slots = 0;
+    unsigned* lv_cnt = nullptr;
     int* status = nullptr;
     // registration
     unsigned long long* reg_acc = nullptr;  // nodes x ACC_REPLICAS x 4 fixed point
