@@ -7,13 +7,11 @@
 //   H1 = relu(x W1^T + b1)      tcgen05, N = 256, K = 1280, bias+ReLU epilogue -> BF16
 //   H2 = relu(H1 W2^T + b2)     tcgen05, N = 256, K = 256
 //   Y  = H2 W3^T + b3           tcgen05, N = 16 (rows 9..15 of W3 are zero), FP32 out
-// Backward (dY from the loss kernel, BF16 for the tensor cores, FP32 kept):
-//   dW3^T = H2^T dY             M = 256 hidden, N = 16, K = batch (both read transposed)
-//   dZ2 = (dY W3) * [H2 > 0]    N = 256, K = 16, mask epilogue -> BF16
-//   dW2 = dZ2^T H1              M = 256, N = 256, K = batch
-//   dZ1 = (dZ2 W2) * [H1 > 0]
-//   dW1 = dZ1^T x               M = 256, N = 1280, K = batch
+// Backward (hgmm_train.cuh; dY from the loss kernel, BF16 for the tensor cores, FP32 kept):
+//   dZ2 = (dY W3) * [H2 > 0], dZ1 = (dZ2 W2) * [H1 > 0]   one launch per 128-row block
+//   dW3^T = H2^T dY, dW2 = dZ2^T H1, dW1 = dZ1^T x        one launch, operands read transposed
 //   db = column sums of dZ1, dZ2, dY (two-pass, fixed order: deterministic)
+//   K slices summed in order, with Adam in the same pass
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 #include <mutex>
@@ -27,6 +25,7 @@
 #include "../../include/hgmm_proposal.h"
 #include "hgmm_feat.cuh"
 #include "hgmm_internal.cuh"
+#include "hgmm_math.cuh"
 #include "hgmm_tc.cuh"
 
 namespace hgmm {
@@ -94,139 +93,6 @@ __device__ __forceinline__ void gram_schmidt(const double* a1, const double* a2,
     const double i2 = *n2 > 0.0 ? 1.0 / *n2 : 0.0;
     for (int i = 0; i < 3; ++i) b2[i] = u[i] * i2;
     cross3(b1, b2, b3);
-}
-
-// Loss of every row and dL/dy (mean over the batch); one CTA of 256
-// threads, fixed-order block reduction of the loss.
-__global__ void __launch_bounds__(256) k_loss(const float* __restrict__ Y, const float* __restrict__ L,
-                                              int batch, float w_t, bf16* __restrict__ dY,
-                                              float* __restrict__ dYf, float* __restrict__ loss) {
-    __shared__ double red[256];
-    double acc = 0.0;
-    const double inv_b = 1.0 / double(batch);
-    for (int r = threadIdx.x; r < batch; r += blockDim.x) {
-        const float* y = Y + int64_t(r) * OUT;
-        const float* l = L + int64_t(r) * HGMM_LABEL_FLOATS;
-        double a1[3], a2[3], b1[3], b2[3], b3[3], n1, dd, n2;
-        for (int i = 0; i < 3; ++i) {
-            a1[i] = y[i];
-            a2[i] = y[3 + i];
-        }
-        gram_schmidt(a1, a2, b1, b2, b3, &n1, &dd, &n2);
-        double G1[3], G2[3], G3[3], e = 0.0;
-        for (int i = 0; i < 3; ++i) {
-            // label R' row-major: column k entry i at l[3 i + k]
-            const double r0 = b1[i] - l[3 * i + 0], r1 = b2[i] - l[3 * i + 1], r2 = b3[i] - l[3 * i + 2];
-            e += r0 * r0 + r1 * r1 + r2 * r2;
-            G1[i] = 2.0 * r0;
-            G2[i] = 2.0 * r1;
-            G3[i] = 2.0 * r2;
-        }
-        double gt[3];
-        for (int i = 0; i < 3; ++i) {
-            const double d = double(y[6 + i]) - l[9 + i];
-            e += double(w_t) * d * d;
-            gt[i] = 2.0 * double(w_t) * d;
-        }
-        acc += e;
-        // back through b3 = b1 x b2, b2 = u / |u|, u = a2 - (b1.a2) b1, b1 = a1 / |a1|
-        double gb1[3], gb2[3], c[3];
-        cross3(b2, G3, c);
-        for (int i = 0; i < 3; ++i) gb1[i] = G1[i] + c[i];
-        cross3(G3, b1, c);
-        for (int i = 0; i < 3; ++i) gb2[i] = G2[i] + c[i];
-        const double i2 = n2 > 0.0 ? 1.0 / n2 : 0.0, i1 = n1 > 0.0 ? 1.0 / n1 : 0.0;
-        const double p2 = dot3(gb2, b2);
-        double gu[3];
-        for (int i = 0; i < 3; ++i) gu[i] = (gb2[i] - p2 * b2[i]) * i2;
-        const double q = dot3(gu, b1);
-        double ga2[3];
-        for (int i = 0; i < 3; ++i) {
-            ga2[i] = gu[i] - q * b1[i];
-            gb1[i] += -q * a2[i] - dd * gu[i];
-        }
-        const double p1 = dot3(gb1, b1);
-        double g[OUTP];
-        for (int i = 0; i < 3; ++i) {
-            g[i] = (gb1[i] - p1 * b1[i]) * i1 * inv_b;
-            g[3 + i] = ga2[i] * inv_b;
-            g[6 + i] = gt[i] * inv_b;
-        }
-        for (int i = OUT; i < OUTP; ++i) g[i] = 0.0;
-        for (int i = 0; i < OUTP; ++i) {
-            dYf[int64_t(r) * OUTP + i] = float(g[i]);
-            dY[int64_t(r) * OUTP + i] = __double2bfloat16(g[i]);
-        }
-    }
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int st = 128; st > 0; st >>= 1) {
-        if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && loss) *loss = float(red[0] * inv_b);
-}
-
-// Column sums for the bias gradients, pass 1: block (chunk, matrix) sums
-// COLSUM_ROWS rows of one column per thread.  matrix 0: dZ1, 1: dZ2 (BF16,
-// 256 columns), 2: dY (FP32, 16 columns).
-__global__ void __launch_bounds__(256) k_colsum_partial(const bf16* __restrict__ dZ1,
-                                                        const bf16* __restrict__ dZ2,
-                                                        const float* __restrict__ dYf, int batch,
-                                                        float* __restrict__ part) {
-    const int chunk = blockIdx.x, mat = blockIdx.y, j = threadIdx.x;
-    const int r0 = chunk * COLSUM_ROWS, r1 = min(batch, r0 + COLSUM_ROWS);
-    float s = 0.f;
-    if (mat < 2) {
-        const bf16* Z = mat == 0 ? dZ1 : dZ2;
-        for (int r = r0; r < r1; ++r) s += __bfloat162float(Z[int64_t(r) * HID + j]);
-    } else if (j < OUTP) {
-        for (int r = r0; r < r1; ++r) s += dYf[int64_t(r) * OUTP + j];
-    }
-    part[(int64_t(chunk) * 3 + mat) * HID + j] = s;
-}
-
-// pass 2: fixed-order sum over the chunks into the bias gradients.
-__global__ void __launch_bounds__(256) k_colsum_final(const float* __restrict__ part, int nchunks,
-                                                      float* __restrict__ grads) {
-    const int mat = blockIdx.x, j = threadIdx.x;
-    double s = 0.0;
-    for (int c = 0; c < nchunks; ++c) s += part[(int64_t(c) * 3 + mat) * HID + j];
-    if (mat == 0) grads[OFF_B1 + j] = float(s);
-    else if (mat == 1) grads[OFF_B2 + j] = float(s);
-    else if (j < OUT) grads[OFF_B3 + j] = float(s);
-}
-
-// BF16 copies of the weights the tensor cores read; W3 padded to 16 rows.
-__device__ __forceinline__ void store_bf16_copy(int64_t i, float p, bf16* W1, bf16* W2, bf16* W3,
-                                                float* b3p) {
-    if (i < OFF_B1) W1[i - OFF_W1] = __float2bfloat16_rn(p);
-    else if (i >= OFF_W2 && i < OFF_B2) W2[i - OFF_W2] = __float2bfloat16_rn(p);
-    else if (i >= OFF_W3 && i < OFF_B3) W3[i - OFF_W3] = __float2bfloat16_rn(p);
-    else if (i >= OFF_B3) b3p[i - OFF_B3] = p;
-}
-
-__global__ void k_refresh(const float* __restrict__ P, bf16* W1, bf16* W2, bf16* W3, float* b3p) {
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < N_PARAMS;
-         i += int64_t(gridDim.x) * blockDim.x)
-        store_bf16_copy(i, P[i], W1, W2, W3, b3p);
-}
-
-__global__ void k_adam(float* __restrict__ P, const float* __restrict__ G, float* __restrict__ Mo,
-                       float* __restrict__ Vo, float lr, float c1, float c2, bf16* W1, bf16* W2,
-                       bf16* W3, float* b3p) {
-    const float beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < N_PARAMS;
-         i += int64_t(gridDim.x) * blockDim.x) {
-        const float g = G[i];
-        const float m = beta1 * Mo[i] + (1.f - beta1) * g;
-        const float v = beta2 * Vo[i] + (1.f - beta2) * g * g;
-        Mo[i] = m;
-        Vo[i] = v;
-        const float p = P[i] - lr * (m * c1) / (sqrtf(v * c2) + eps);
-        P[i] = p;
-        store_bf16_copy(i, p, W1, W2, W3, b3p);
-    }
 }
 
 __device__ __forceinline__ void load_frame(const double* f, double* c, double& s, double* V) {
@@ -558,6 +424,8 @@ k_mlp_forward(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
 }  // namespace
 }  // namespace hgmm
 
+#include "hgmm_train.cuh"
+
 using namespace hgmm;
 using hgmm::tc::GemmArgs;
 
@@ -574,19 +442,23 @@ struct hgmm_mlp {
     bf16* W2 = nullptr;
     bf16* W3 = nullptr;   // 16 x 256, rows >= 9 zero
     float* b3p = nullptr; // 16
+    bf16* W2T = nullptr;  // W2 transposed (the backward pass)
+    bf16* W3T = nullptr;  // W3 transposed, 256 x 64, columns >= 9 zero
     bf16* Xg = nullptr;   // gathered batch
     float* Lg = nullptr;
     bf16* H1 = nullptr;
     bf16* H2 = nullptr;
     float* Y = nullptr;   // batch x 9
-    bf16* dY = nullptr;   // batch x 16
+    bf16* dY = nullptr;   // batch x 64, columns >= 9 zero
     float* dYf = nullptr;
     bf16* dZ2 = nullptr;
     bf16* dZ1 = nullptr;
     float* part = nullptr;
     float* loss = nullptr;
+    double* loss_part = nullptr;  // per CTA of the loss
+    unsigned* loss_cnt = nullptr;
     int* err = nullptr;
-    float* ws = nullptr;      // K-slice partials of the weight-gradient products
+    float* ws = nullptr;      // K-slice partials of the weight gradients
     long long ws_cap = 0;     // floats
     bf16* prop_x = nullptr;   // hgmm_propose: one pair's input (1280)
     double* prop_fr = nullptr;  // ... its frames (source, target: 32)
@@ -772,12 +644,73 @@ bool set_gemm_smem() {
                                 tc::tma_smem_bytes(128)) == cudaSuccess &&
            cudaFuncSetAttribute(tc::k_gemm_tma<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 tc::tma_smem_bytes(16)) == cudaSuccess &&
-           cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, FW_SMEM) == cudaSuccess;
+           cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, FW_SMEM) == cudaSuccess &&
+           cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, BW_SMEM) == cudaSuccess &&
+           cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM) == cudaSuccess;
 }
 
 int check_dev(const hgmm_mlp* m) {
     int cur = -1;
     return (cudaGetDevice(&cur) == cudaSuccess && cur == m->device) ? HGMM_OK : HGMM_EINVAL;
+}
+
+WeightCopies copies(const hgmm_mlp* m) { return WeightCopies{m->W1, m->W2, m->W3, m->W2T, m->W3T, m->b3p}; }
+
+// Adam's bias corrections of step t.
+void adam_scales(int t, float* c1, float* c2) {
+    *c1 = float(1.0 / (1.0 - std::pow(0.9, t)));
+    *c2 = float(1.0 / (1.0 - std::pow(0.999, t)));
+}
+
+// Loss, gradients and (lr not null) the Adam step of one batch.
+int gradients_impl(hgmm_mlp* m, const uint16_t* d_x, const float* d_labels, const int32_t* d_index, int32_t batch,
+                   int32_t n_rows, float w_t, float* d_loss, const float* lr, void* stream) {
+    if (!m || !d_x || !d_labels || batch < 1 || batch > m->max_batch || !a16(d_x) || !(w_t >= 0.f))
+        return HGMM_EINVAL;
+    if (d_index && n_rows < 1) return HGMM_EINVAL;
+    if (int rc = check_dev(m)) return rc;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const bf16* X = reinterpret_cast<const bf16*>(d_x);
+    const float* L = d_labels;
+    // tensor maps of the backward pass: K-major operands and the dZ tiles
+    // (128-row boxes), and the weight gradients' operands (64-row boxes)
+    CUtensorMap bdy, bw3, bw2, bz2, bz1, gz1, gx, gz2, gh1, gh2, gdy;
+    const bf16* Xb = d_index ? m->Xg : X;
+    if (!encode_operand(&bdy, m->dY, DY_STRIDE, batch, DY_STRIDE, 128) ||
+        !encode_operand(&bw3, m->W3T, DY_STRIDE, HID, DY_STRIDE, HID) ||
+        !encode_operand(&bw2, m->W2T, HID, HID, HID, HID) || !encode_operand(&bz2, m->dZ2, HID, batch, HID, 128) ||
+        !encode_operand(&bz1, m->dZ1, HID, batch, HID, 128) || !encode_operand(&gz1, m->dZ1, HID, batch, HID, 64) ||
+        !encode_operand(&gx, Xb, IN, batch, IN, 64) || !encode_operand(&gz2, m->dZ2, HID, batch, HID, 64) ||
+        !encode_operand(&gh1, m->H1, HID, batch, HID, 64) || !encode_operand(&gh2, m->H2, HID, batch, HID, 64) ||
+        !encode_operand(&gdy, m->dY, DY_STRIDE, batch, DY_STRIDE, 64))
+        return HGMM_ECUDA;
+    if (d_index) {
+        k_gather<<<batch, 160, 0, s>>>(X, d_labels, d_index, n_rows, m->Xg, m->Lg, m->err);
+        X = m->Xg;
+        L = m->Lg;
+    }
+    if (int rc = forward_impl(m, X, batch, m->Y, s)) return rc;
+    k_loss<<<(batch + LOSS_ROWS - 1) / LOSS_ROWS, LOSS_THREADS, 0, s>>>(m->Y, L, batch, w_t, m->dY, m->dYf,
+                                                                       m->loss_part, m->loss_cnt,
+                                                                       d_loss ? d_loss : m->loss);
+    k_mlp_backward<<<(batch + 127) / 128, BW_THREADS, BW_SMEM, s>>>(bdy, bw3, bw2, bz2, bz1, m->H1, m->H2, batch,
+                                                                   m->err);
+    const int slices = wg_slices(batch), nchunks = (batch + COLSUM_ROWS - 1) / COLSUM_ROWS;
+    k_mlp_wgrad<<<WG_TILES * slices + nchunks, WG_THREADS, WG_SMEM, s>>>(gz1, gx, gz2, gh1, gh2, gdy, batch, slices,
+                                                                        wg_chunks(batch), m->dZ1, m->dZ2, m->dYf,
+                                                                        m->ws, m->part, m->err);
+    const int ug = int((N_PARAMS + 511) / 512);
+    if (lr) {
+        m->step += 1;
+        float c1, c2;
+        adam_scales(m->step, &c1, &c2);
+        k_grad_update<true><<<ug, 128, 0, s>>>(m->ws, slices, m->part, nchunks, m->G, m->P, m->Mo, m->Vo, *lr, c1,
+                                               c2, copies(m));
+    } else {
+        k_grad_update<false><<<ug, 128, 0, s>>>(m->ws, slices, m->part, nchunks, m->G, m->P, m->Mo, m->Vo, 0.f, 0.f,
+                                                0.f, copies(m));
+    }
+    return cudaGetLastError() == cudaSuccess ? HGMM_OK : HGMM_ECUDA;
 }
 
 }  // namespace
@@ -802,13 +735,15 @@ int hgmm_mlp_create(int32_t max_batch, hgmm_mlp** out) {
                 malloc_into(m, &m->W3, size_t(OUTP) * HID) && malloc_into(m, &m->b3p, OUTP) &&
                 malloc_into(m, &m->Xg, B * IN) && malloc_into(m, &m->Lg, B * HGMM_LABEL_FLOATS) &&
                 malloc_into(m, &m->H1, B * HID) && malloc_into(m, &m->H2, B * HID) &&
-                malloc_into(m, &m->Y, B * OUT) && malloc_into(m, &m->dY, B * OUTP) &&
+                malloc_into(m, &m->Y, B * OUT) && malloc_into(m, &m->dY, B * DY_STRIDE) &&
                 malloc_into(m, &m->dYf, B * OUTP) && malloc_into(m, &m->dZ2, B * HID) &&
                 malloc_into(m, &m->dZ1, B * HID) && malloc_into(m, &m->part, size_t(nchunks) * 3 * HID) &&
-                malloc_into(m, &m->loss, 1) && malloc_into(m, &m->err, 1) &&
+                malloc_into(m, &m->loss, 1) &&
+                malloc_into(m, &m->W2T, size_t(HID) * HID) && malloc_into(m, &m->W3T, size_t(HID) * DY_STRIDE) &&
+                malloc_into(m, &m->loss_part, (B + LOSS_ROWS - 1) / LOSS_ROWS) && malloc_into(m, &m->loss_cnt, 1) && malloc_into(m, &m->err, 1) &&
                 malloc_into(m, &m->prop_x, IN) && malloc_into(m, &m->prop_fr, 2 * HGMM_FRAME_DOUBLES) &&
                 malloc_into(m, &m->prop_y, 16);
-    m->ws_cap = (long long)MAX_SLICES * HID * IN;
+    m->ws_cap = (long long)WG_MAX_SLICES * WS_STRIDE;
     good = good && malloc_into(m, &m->ws, size_t(m->ws_cap));
     good = good && set_gemm_smem();
     if (!good) {
@@ -837,7 +772,7 @@ int hgmm_mlp_set_params(hgmm_mlp* m, const float* h_params, int64_t count) {
                 cudaMemset(m->Mo, 0, bytes) == cudaSuccess && cudaMemset(m->Vo, 0, bytes) == cudaSuccess &&
                 cudaMemset(m->G, 0, bytes) == cudaSuccess;
     if (!good) return HGMM_ECUDA;
-    k_refresh<<<512, 256>>>(m->P, m->W1, m->W2, m->W3, m->b3p);
+    k_refresh<<<512, 256>>>(m->P, copies(m));
     m->step = 0;
     return cudaDeviceSynchronize() == cudaSuccess ? HGMM_OK : HGMM_ECUDA;
 }
@@ -867,77 +802,23 @@ int hgmm_mlp_forward(hgmm_mlp* m, const uint16_t* d_x, int32_t batch, float* d_y
 
 int hgmm_mlp_gradients(hgmm_mlp* m, const uint16_t* d_x, const float* d_labels, const int32_t* d_index,
                        int32_t batch, int32_t n_rows, float w_t, float* d_loss, void* stream) {
-    if (!m || !d_x || !d_labels || batch < 1 || batch > m->max_batch || !a16(d_x) || !(w_t >= 0.f))
-        return HGMM_EINVAL;
-    if (d_index && n_rows < 1) return HGMM_EINVAL;
-    if (int rc = check_dev(m)) return rc;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const bf16* X = reinterpret_cast<const bf16*>(d_x);
-    const float* L = d_labels;
-    if (d_index) {
-        k_gather<<<batch, 160, 0, s>>>(X, d_labels, d_index, n_rows, m->Xg, m->Lg, m->err);
-        X = m->Xg;
-        L = m->Lg;
-    }
-    if (int rc = forward_impl(m, X, batch, m->Y, s)) return rc;
-    k_loss<<<1, 256, 0, s>>>(m->Y, L, batch, w_t, m->dY, m->dYf, d_loss ? d_loss : m->loss);
-    // dW3^T[h][o] = sum_r H2[r][h] dY[r][o]: A = H2^T, B = dY^T (both read along rows)
-    GemmArgs g = gargs(m->H2, 1, HID, m->dY, 1, OUTP, HID, OUTP, batch, tc::EPI_F32, m->err);
-    g.out_f32 = m->G + OFF_W3;
-    g.o_m = 1;
-    g.o_n = HID;
-    g.n_store = OUT;
-    if (int rc = gemm(g, s, m->ws, m->ws_cap)) return rc;
-    // dZ2 = (dY W3) * [H2 > 0]: B[n = h][k = o] = W3[o][h]
-    g = gargs(m->dY, OUTP, 1, m->W3, 1, HID, batch, HID, OUTP, tc::EPI_MASK_BF16, m->err);
-    g.mask = m->H2;
-    g.mask_m = HID;
-    g.out_bf16 = m->dZ2;
-    g.o_m = HID;
-    g.o_n = 1;
-    if (int rc = gemm(g, s, m->ws, m->ws_cap)) return rc;
-    // dW2 = dZ2^T H1
-    g = gargs(m->dZ2, 1, HID, m->H1, 1, HID, HID, HID, batch, tc::EPI_F32, m->err);
-    g.out_f32 = m->G + OFF_W2;
-    g.o_m = HID;
-    g.o_n = 1;
-    if (int rc = gemm(g, s, m->ws, m->ws_cap)) return rc;
-    // dZ1 = (dZ2 W2) * [H1 > 0]
-    g = gargs(m->dZ2, HID, 1, m->W2, 1, HID, batch, HID, HID, tc::EPI_MASK_BF16, m->err);
-    g.mask = m->H1;
-    g.mask_m = HID;
-    g.out_bf16 = m->dZ1;
-    g.o_m = HID;
-    g.o_n = 1;
-    if (int rc = gemm(g, s, m->ws, m->ws_cap)) return rc;
-    // dW1 = dZ1^T x
-    g = gargs(m->dZ1, 1, HID, X, 1, IN, HID, IN, batch, tc::EPI_F32, m->err);
-    g.out_f32 = m->G + OFF_W1;
-    g.o_m = IN;
-    g.o_n = 1;
-    if (int rc = gemm(g, s, m->ws, m->ws_cap)) return rc;
-    const int nchunks = (batch + COLSUM_ROWS - 1) / COLSUM_ROWS;
-    k_colsum_partial<<<dim3(nchunks, 3), 256, 0, s>>>(m->dZ1, m->dZ2, m->dYf, batch, m->part);
-    k_colsum_final<<<3, 256, 0, s>>>(m->part, nchunks, m->G);
-    return cudaGetLastError() == cudaSuccess ? HGMM_OK : HGMM_ECUDA;
+    return gradients_impl(m, d_x, d_labels, d_index, batch, n_rows, w_t, d_loss, nullptr, stream);
 }
 
 int hgmm_mlp_adam(hgmm_mlp* m, float lr, void* stream) {
     if (!m || !(lr >= 0.f)) return HGMM_EINVAL;
     if (int rc = check_dev(m)) return rc;
     m->step += 1;
-    const double c1 = 1.0 / (1.0 - std::pow(0.9, m->step));
-    const double c2 = 1.0 / (1.0 - std::pow(0.999, m->step));
-    k_adam<<<608, 256, 0, static_cast<cudaStream_t>(stream)>>>(m->P, m->G, m->Mo, m->Vo, lr, float(c1),
-                                                              float(c2), m->W1, m->W2, m->W3, m->b3p);
+    float c1, c2;
+    adam_scales(m->step, &c1, &c2);
+    k_adam<<<608, 256, 0, static_cast<cudaStream_t>(stream)>>>(m->P, m->G, m->Mo, m->Vo, lr, c1, c2, copies(m));
     return cudaGetLastError() == cudaSuccess ? HGMM_OK : HGMM_ECUDA;
 }
 
 int hgmm_mlp_train_step(hgmm_mlp* m, const uint16_t* d_x, const float* d_labels, const int32_t* d_index,
                         int32_t batch, int32_t n_rows, float w_t, float lr, float* d_loss, void* stream) {
-    if (int rc = hgmm_mlp_gradients(m, d_x, d_labels, d_index, batch, n_rows, w_t, d_loss, stream))
-        return rc;
-    return hgmm_mlp_adam(m, lr, stream);
+    if (!(lr >= 0.f)) return HGMM_EINVAL;
+    return gradients_impl(m, d_x, d_labels, d_index, batch, n_rows, w_t, d_loss, &lr, stream);
 }
 
 int hgmm_mlp_sync(hgmm_mlp* m, void* stream) {

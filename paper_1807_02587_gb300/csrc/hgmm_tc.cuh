@@ -158,7 +158,6 @@ enum Epilogue : int {
     EPI_F32 = 0,             // out_f32[m, n] = acc
     EPI_BIAS_F32 = 1,        // out_f32[m, n] = acc + bias[n]
     EPI_BIAS_RELU_BF16 = 2,  // out_bf16[m, n] = bf16(max(acc + bias[n], 0))
-    EPI_MASK_BF16 = 3,       // out_bf16[m, n] = bf16(mask[m, n] > 0 ? acc : 0)
 };
 
 struct GemmArgs {
@@ -172,8 +171,6 @@ struct GemmArgs {
     int n_store;          // columns n >= n_store are not written
     int epi;
     const float* bias;
-    const __nv_bfloat16* mask;
-    long long mask_m;
     float* out_f32;
     __nv_bfloat16* out_bf16;
     long long o_m, o_n;   // out[m * o_m + n * o_n]
@@ -251,14 +248,9 @@ __device__ __forceinline__ void epilogue16(const GemmArgs& g, float* outf, int m
         switch (g.epi) {
             case EPI_F32: outf[o] = x; break;
             case EPI_BIAS_F32: outf[o] = x + g.bias[n]; break;
-            case EPI_BIAS_RELU_BF16:
+            default:
                 x += g.bias[n];
                 g.out_bf16[o] = __float2bfloat16_rn(x > 0.f ? x : 0.f);
-                break;
-            default: {
-                const float mk = __bfloat162float(g.mask[m * g.mask_m + n]);
-                g.out_bf16[o] = __float2bfloat16_rn(mk > 0.f ? x : 0.f);
-            }
         }
     }
 }
@@ -269,10 +261,10 @@ __device__ __forceinline__ void epilogue16(const GemmArgs& g, float* outf, int m
 // and reads the bias as float4; otherwise element by element.
 __device__ __forceinline__ void epilogue32(const GemmArgs& g, float* outf, int m, int n0c, const float (&v)[32]) {
     if (m >= g.M) return;
-    const bool bf = g.epi == EPI_BIAS_RELU_BF16 || g.epi == EPI_MASK_BF16;
+    const bool bf = g.epi == EPI_BIAS_RELU_BF16;
     const int lim = min(g.N, g.n_store);
     const long long o = m * g.o_m + n0c;
-    const bool vec = n0c + 32 <= lim && g.o_n == 1 && g.epi != EPI_MASK_BF16 &&
+    const bool vec = n0c + 32 <= lim && g.o_n == 1 &&
                      ((bf ? reinterpret_cast<uintptr_t>(g.out_bf16 + o) : reinterpret_cast<uintptr_t>(outf + o)) &
                       15u) == 0 &&
                      (g.epi == EPI_F32 || (reinterpret_cast<uintptr_t>(g.bias + n0c) & 15u) == 0);
