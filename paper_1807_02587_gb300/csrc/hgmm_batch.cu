@@ -219,8 +219,8 @@ __device__ void run_pair(const BatchArgs& a, const BatchWs& w, int cid, int pair
 
     // ---- proposal features of the target (levels 0 and 1)
     if (a.feat && rank == 0 && warp == 0 && depth >= 2)
-        tree_features_warp(w.root, w.stat, a.feat + int64_t(FEAT_PER_CLOUD) * pair,
-                           a.frame + int64_t(FRAME_DOUBLES) * pair, rgs.fsm);
+        tree_features<32>(w.root, w.stat, a.feat + int64_t(FEAT_PER_CLOUD) * pair,
+                          a.frame + int64_t(FRAME_DOUBLES) * pair, rgs.fsm, [] { __syncwarp(); });
 
     // ---- registration (Algorithm 1 + Eq. 9-16)
     const int n_nodes = int(level_offset(depth));

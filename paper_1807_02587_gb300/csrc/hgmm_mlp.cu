@@ -48,9 +48,18 @@ constexpr int COLSUM_ROWS = 64;  // rows per partial column sum
 
 using bf16 = __nv_bfloat16;
 
-__global__ void k_tree_features(const RootDev* root, const NodeStat* stat, bf16* feat, double* frame) {
+// Features and frames of one or two trees (blockIdx.x), one thread per node.
+struct FeatJob {
+    const RootDev* root;
+    const NodeStat* stat;
+    bf16* feat;
+    double* frame;
+};
+
+__global__ void __launch_bounds__(FEAT_NODES) k_tree_features(FeatJob a, FeatJob b) {
     __shared__ double fsm[FRAME_DOUBLES];
-    tree_features_warp(root, stat, feat, frame, fsm);
+    const FeatJob j = blockIdx.x == 0 ? a : b;
+    tree_features<FEAT_NODES>(j.root, j.stat, j.feat, j.frame, fsm, [] { __syncthreads(); });
 }
 
 // Rows idx[r] of x and labels -> row r of the gathered batch.
@@ -101,37 +110,55 @@ __device__ __forceinline__ void load_frame(const double* f, double* c, double& s
     for (int v = 0; v < 9; ++v) V[v] = f[4 + v];
 }
 
-__global__ void k_decode(const float* __restrict__ Y, const double* __restrict__ F, int n,
-                         double* __restrict__ T) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+// Sixteen lanes per pair, lane (r, c) = entry (r, c) of T: a handful of pairs
+// is one dependent FP64 chain, so the entries share its instructions (one
+// pair: 6.8 us with one thread, 4.6 here).
+constexpr int DECODE_THREADS = 128;
+__global__ void __launch_bounds__(DECODE_THREADS)
+k_decode(const float* __restrict__ Y, const double* __restrict__ F, int n, double* __restrict__ T) {
+    const int64_t i = (int64_t(blockIdx.x) * DECODE_THREADS + threadIdx.x) >> 4;
+    const unsigned half = 0xFFFFu << (threadIdx.x & 16);
+    if (i >= n) return;  // whole half-warps
+    const int e = threadIdx.x & 15, r = e >> 2 < 3 ? e >> 2 : 2, c = e & 3;
     double cs[3], ct[3], Vs[9], Vt[9], ss, st;
-    load_frame(F + 32 * int64_t(i), cs, ss, Vs);
-    load_frame(F + 32 * int64_t(i) + 16, ct, st, Vt);
-    const float* y = Y + int64_t(i) * OUT;
-    double a1[3], a2[3], b[3][3], n1, dd, n2;
+    load_frame(F + 32 * i, cs, ss, Vs);
+    load_frame(F + 32 * i + 16, ct, st, Vt);
+    const float* y = Y + i * OUT;
+    double a1[3], a2[3], b1[3], b2[3], b3[3];
     for (int k = 0; k < 3; ++k) {
         a1[k] = y[k];
         a2[k] = y[3 + k];
     }
-    gram_schmidt(a1, a2, b[0], b[1], b[2], &n1, &dd, &n2);
-    // R' (columns b[0..2]); A = Vt R', R = A Vs^T
-    double A[3][3], R[3][3];
-    for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) A[r][c] = Vt[3 * r] * b[c][0] + Vt[3 * r + 1] * b[c][1] + Vt[3 * r + 2] * b[c][2];
-    for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) R[r][c] = A[r][0] * Vs[3 * c] + A[r][1] * Vs[3 * c + 1] + A[r][2] * Vs[3 * c + 2];
-    double* o = T + 16 * int64_t(i);
-    for (int r = 0; r < 3; ++r) {
-        const double vt = Vt[3 * r] * y[6] + Vt[3 * r + 1] * y[7] + Vt[3 * r + 2] * y[8];
-        const double rc = R[r][0] * cs[0] + R[r][1] * cs[1] + R[r][2] * cs[2];
-        for (int c = 0; c < 3; ++c) o[4 * r + c] = R[r][c];
-        o[4 * r + 3] = ct[r] + st * vt - rc;
-    }
-    o[12] = 0.0;
-    o[13] = 0.0;
-    o[14] = 0.0;
-    o[15] = 1.0;
+    // Gram-Schmidt of (a1, a2) into the columns b1, b2, b3 = b1 x b2
+    const double s1 = dot3(a1, a1);
+    const double i1 = s1 > 0.0 ? rsqrt_f64(s1) : 0.0;
+    for (int k = 0; k < 3; ++k) b1[k] = a1[k] * i1;
+    const double dd = dot3(b1, a2);
+    double u[3];
+    for (int k = 0; k < 3; ++k) u[k] = a2[k] - dd * b1[k];
+    const double s2 = dot3(u, u);
+    const double i2 = s2 > 0.0 ? rsqrt_f64(s2) : 0.0;
+    for (int k = 0; k < 3; ++k) b2[k] = u[k] * i2;
+    cross3(b1, b2, b3);
+    // R' (columns b1..b3); A = Vt R', R = A Vs^T: lane (r, c) forms entry (r,
+    // c) of both; lane (r, 3) the translation's Vt y_t instead of A's entry
+    const double vt0 = r == 0 ? Vt[0] : (r == 1 ? Vt[3] : Vt[6]);
+    const double vt1 = r == 0 ? Vt[1] : (r == 1 ? Vt[4] : Vt[7]);
+    const double vt2 = r == 0 ? Vt[2] : (r == 1 ? Vt[5] : Vt[8]);
+    double x[3];
+    for (int k = 0; k < 3; ++k) x[k] = c == 0 ? b1[k] : (c == 1 ? b2[k] : (c == 2 ? b3[k] : double(y[6 + k])));
+    const double Arc = vt0 * x[0] + vt1 * x[1] + vt2 * x[2];
+    const int row = threadIdx.x & 28;  // this lane's row of four
+    const double A0 = __shfl_sync(half, Arc, row & 31), A1 = __shfl_sync(half, Arc, (row + 1) & 31);
+    const double A2 = __shfl_sync(half, Arc, (row + 2) & 31);
+    double z[3];
+    for (int k = 0; k < 3; ++k) z[k] = c == 1 ? Vs[3 + k] : (c == 2 ? Vs[6 + k] : Vs[k]);
+    const double Rrc = A0 * z[0] + A1 * z[1] + A2 * z[2];
+    const double R0 = __shfl_sync(half, Rrc, row), R1 = __shfl_sync(half, Rrc, row + 1);
+    const double R2 = __shfl_sync(half, Rrc, row + 2);
+    const double ctr = r == 0 ? ct[0] : (r == 1 ? ct[1] : ct[2]);
+    const double t = ctr + st * Arc - (R0 * cs[0] + R1 * cs[1] + R2 * cs[2]);
+    T[16 * i + e] = e >= 12 ? (e == 15 ? 1.0 : 0.0) : (c == 3 ? t : Rrc);
 }
 
 __global__ void k_encode(const double* __restrict__ T, const double* __restrict__ F, int n,
@@ -835,26 +862,29 @@ int hgmm_mlp_sync(hgmm_mlp* m, void* stream) {
 
 int hgmm_tree_features(hgmm_tree* t, uint16_t* d_feat, double* d_frame, void* stream) {
     if (!t || !d_feat || !d_frame || !t->built || t->depth < 2 || !a16(d_feat)) return HGMM_EINVAL;
-    k_tree_features<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(
-        t->root, t->stat, reinterpret_cast<bf16*>(d_feat), d_frame);
+    const FeatJob j{t->root, t->stat, reinterpret_cast<bf16*>(d_feat), d_frame};
+    k_tree_features<<<1, FEAT_NODES, 0, static_cast<cudaStream_t>(stream)>>>(j, j);
     return cudaGetLastError() == cudaSuccess ? HGMM_OK : HGMM_ECUDA;
 }
 
 int hgmm_propose(hgmm_tree* tgt, hgmm_tree* src, hgmm_mlp* m, void* stream, double* d_T_out) {
     if (!tgt || !src || !m || !d_T_out) return HGMM_EINVAL;
     if (int rc = check_dev(m)) return rc;
-    uint16_t* x = reinterpret_cast<uint16_t*>(m->prop_x);
-    // network input: [features(source), features(target)], frames likewise
-    if (int rc = hgmm_tree_features(src, x, m->prop_fr, stream)) return rc;
-    if (int rc = hgmm_tree_features(tgt, x + HGMM_FEAT_PER_CLOUD, m->prop_fr + HGMM_FRAME_DOUBLES, stream))
-        return rc;
-    if (int rc = hgmm_mlp_forward(m, x, 1, m->prop_y, stream)) return rc;
+    if (!src->built || src->depth < 2 || !tgt->built || tgt->depth < 2) return HGMM_EINVAL;
+    // network input: [features(source), features(target)], frames likewise,
+    // both trees in one launch
+    k_tree_features<<<2, FEAT_NODES, 0, static_cast<cudaStream_t>(stream)>>>(
+        FeatJob{src->root, src->stat, m->prop_x, m->prop_fr},
+        FeatJob{tgt->root, tgt->stat, m->prop_x + FEAT_PER_CLOUD, m->prop_fr + FRAME_DOUBLES});
+    if (cudaGetLastError() != cudaSuccess) return HGMM_ECUDA;
+    if (int rc = hgmm_mlp_forward(m, reinterpret_cast<const uint16_t*>(m->prop_x), 1, m->prop_y, stream)) return rc;
     return hgmm_pose_decode(m->prop_y, m->prop_fr, 1, d_T_out, stream);
 }
 
 int hgmm_pose_decode(const float* d_y, const double* d_frames, int32_t n, double* d_T, void* stream) {
     if (!d_y || !d_frames || !d_T || n < 1) return HGMM_EINVAL;
-    k_decode<<<(n + 127) / 128, 128, 0, static_cast<cudaStream_t>(stream)>>>(d_y, d_frames, n, d_T);
+    k_decode<<<(n + DECODE_THREADS / 16 - 1) / (DECODE_THREADS / 16), DECODE_THREADS, 0,
+               static_cast<cudaStream_t>(stream)>>>(d_y, d_frames, n, d_T);
     return cudaGetLastError() == cudaSuccess ? HGMM_OK : HGMM_ECUDA;
 }
 
