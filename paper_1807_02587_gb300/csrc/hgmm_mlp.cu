@@ -217,20 +217,30 @@ __global__ void k_compose(int n, const double* __restrict__ A, const double* __r
 // tcgen05 with TMEM accumulators and TMA operand streams):
 //   layer 1: acc1 (TMEM columns 0..255) = X[128 x 1280] W1^T, 20 K-steps of
 //            TMA-fed 128 x 64 / 256 x 64 tiles in a 4-stage ring;
-//   epilogue warps: h1 = relu(acc1 + b1) as BF16 to H1 (global, for the
-//            backward pass; skipped when H1 is null) and into shared memory
-//            in the 128-byte-swizzled K-major layout that TMA would write,
-//            as layer 2's A operand;
+//   epilogue warps: h1 = relu(acc1 + b1) as BF16 into shared memory in the
+//            128-byte-swizzled K-major layout that TMA would write, as layer 2's
+//            A operand, one 64-column chunk after the other: layer 2's products
+//            of a chunk start when it is there;
 //   layer 2: acc2 (columns 256..511) = h1 W2^T, W2 tiles streamed by TMA;
-//   epilogue: h2 likewise (H2 if not null, and shared memory over h1);
+//   epilogue: h2 likewise (over h1);
 //   layer 3: acc3 (columns 0..15) = h2 W3^T (W3 padded to 16 rows);
 //   epilogue: Y = acc3 + b3 (9 columns, FP32).
-// Warps 0-3 are the epilogue (warp w owns TMEM lanes 32w..32w+31, i.e.
-// rows), one thread of warp 4 issues the TMA loads, one thread of warp 5
-// the MMAs.  Every wait is bounded; on a timeout the kernel records the
-// error, lets every role run out (commits and arrivals still happen) and
-// drains its loads in flight before it frees TMEM.
-constexpr int FW_THREADS = 192;
+// For the backward pass the chunks also go to H1 and H2 by TMA stores.
+// Warps 0-7 are the epilogue (warp w owns TMEM lanes 32 (w mod 4)..., i.e.
+// rows, and half w / 4 of a chunk's columns), one thread of warp 8 issues the
+// TMA loads, warp 9 the MMAs.  Every wait is bounded; on a timeout the kernel
+// records the error, lets every role run out (commits and arrivals still
+// happen) and drains its loads in flight before it frees TMEM.
+// A block is a chain on one SM: 20 K steps of four 128 x 256 x 16 MMAs at the
+// tensor pipe's own rate (0.385 us each, 7.7 us in all), then two epilogues and
+// layers: 18.9 us per call from 1 to 9,728 rows with four epilogue warps and
+// whole-layer hand-overs, 15.7 to 16.5 now; 16,384 rows (128 blocks) 20.7 against
+// 16.8.  Splitting a block's columns over a cluster of two or
+// four CTAs does not shorten it: an MMA of 128 or 64 columns takes 0.075 us
+// against 0.096 for 256, and handing the hidden layers round through
+// distributed shared memory costs more than the shorter epilogues save (20.9 us
+// against 18.9 per call at 8192 rows, 17.3 against 18.8 at one row).
+constexpr int FW_THREADS = 320;
 constexpr int FW_S1 = 4;                          // layer-1 stages
 constexpr int FW_A = 128 * 128;                   // 128 rows x 64 BF16
 constexpr int FW_B = 256 * 128;                   // 256 rows x 64 BF16
@@ -247,34 +257,51 @@ __device__ __forceinline__ uint32_t sw128_offset(int r, int u) {
     return uint32_t(r * 128 + ((u ^ (r & 7)) << 4));
 }
 
-// Epilogue of one hidden layer: relu(acc + bias) for this thread's row (all
-// 256 columns) to the global row (16-byte stores, if grow is not null) and
-// to the shared h buffer.
-__device__ __forceinline__ void fw_hidden_epilogue(uint32_t tacc, const float* __restrict__ bias,
-                                                   bf16* __restrict__ grow, uint32_t hbuf, int r) {
-#pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-        float v[64];
-        tc::tmem_ld64(tacc + uint32_t(c * 64), v);
-        const float4* b4 = reinterpret_cast<const float4*>(bias + c * 64);
+// relu(acc + bias) of this thread's row and one half (32 columns) of a
+// 64-column chunk, as BF16 into the chunk's swizzled tile.
+__device__ __forceinline__ void fw_hidden_epilogue(uint32_t tacc, const float* __restrict__ bias, uint32_t chunk,
+                                                   int r, int half) {
+    float v[32];
+    tc::tmem_ld32(tacc, v);
+    const float4* b4 = reinterpret_cast<const float4*>(bias);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const float4 ba = __ldg(b4 + 2 * u), bb = __ldg(b4 + 2 * u + 1);
-            const float x[8] = {v[8 * u] + ba.x, v[8 * u + 1] + ba.y, v[8 * u + 2] + ba.z, v[8 * u + 3] + ba.w,
-                                v[8 * u + 4] + bb.x, v[8 * u + 5] + bb.y, v[8 * u + 6] + bb.z, v[8 * u + 7] + bb.w};
-            uint32_t w[4];
+    for (int u = 0; u < 4; ++u) {
+        const float4 ba = __ldg(b4 + 2 * u), bb = __ldg(b4 + 2 * u + 1);
+        const float x[8] = {v[8 * u] + ba.x, v[8 * u + 1] + ba.y, v[8 * u + 2] + ba.z, v[8 * u + 3] + ba.w,
+                            v[8 * u + 4] + bb.x, v[8 * u + 5] + bb.y, v[8 * u + 6] + bb.z, v[8 * u + 7] + bb.w};
+        uint32_t w[4];
 #pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                const __nv_bfloat162 p2 = __floats2bfloat162_rn(fmaxf(x[2 * h], 0.f), fmaxf(x[2 * h + 1], 0.f));
-                w[h] = *reinterpret_cast<const uint32_t*>(&p2);
-            }
-            if (grow) reinterpret_cast<uint4*>(grow + c * 64)[u] = make_uint4(w[0], w[1], w[2], w[3]);
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
-                         :: "r"(hbuf + uint32_t(c * FW_A) + sw128_offset(r, u)), "r"(w[0]), "r"(w[1]), "r"(w[2]),
-                            "r"(w[3]) : "memory");
+        for (int h = 0; h < 4; ++h) {
+            const __nv_bfloat162 p2 = __floats2bfloat162_rn(fmaxf(x[2 * h], 0.f), fmaxf(x[2 * h + 1], 0.f));
+            w[h] = *reinterpret_cast<const uint32_t*>(&p2);
         }
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                     :: "r"(chunk + sw128_offset(r, 4 * half + u)), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                     : "memory");
     }
 }
+
+// The four K = 16 steps of a 64-wide K chunk by a converged warp (32 bytes
+// along the swizzled row per step: the descriptors' address field counts 16
+// bytes), and a commit on bar if it is not null.
+__device__ __forceinline__ void mma_k64(bool lead, uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc,
+                                        bool accumulate, uint64_t* bar) {
+    if (lead) {
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+            tc::mma_bf16(tmem, da + 2 * kk, db + 2 * kk, idesc, accumulate || kk != 0 ? 1u : 0u);
+        if (bar) tc::mma_commit(bar);
+    }
+    __syncwarp();
+}
+
+__device__ __forceinline__ void tma_store_2d(const void* tmap, int x, int y, uint32_t src) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
+                 :: "l"(tmap), "r"(x), "r"(y), "r"(src) : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 __device__ __forceinline__ bool fw_wait(uint64_t* bar, uint32_t parity, int* fail) {
     if (*(volatile int*)fail) return false;
@@ -286,12 +313,12 @@ __device__ __forceinline__ bool fw_wait(uint64_t* bar, uint32_t parity, int* fai
 __global__ void __launch_bounds__(FW_THREADS, 1)
 k_mlp_forward(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW1,
               const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmW3,
+              const __grid_constant__ CUtensorMap tmH1, const __grid_constant__ CUtensorMap tmH2,
               const float* __restrict__ b1, const float* __restrict__ b2, const float* __restrict__ b3p,
-              bf16* __restrict__ H1, bf16* __restrict__ H2, float* __restrict__ Y, int batch,
-              int* __restrict__ err) {
+              bool keep_hidden, float* __restrict__ Y, int batch, int* __restrict__ err) {
     extern __shared__ unsigned char fw_raw[];
     __shared__ __align__(8) uint64_t full1[FW_S1], empty1[FW_S1], full2[2], empty2[2];
-    __shared__ __align__(8) uint64_t full3, done1, done2, done3, h1_ready, h2_ready;
+    __shared__ __align__(8) uint64_t full3, done1, done2, done3, h1_ready[4], h2_ready[4];
     __shared__ uint32_t tmem_slot;
     __shared__ int fail;
     const uint32_t base = (tc::smem_u32(fw_raw) + 1023u) & ~1023u;
@@ -299,11 +326,11 @@ k_mlp_forward(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     const int m0 = blockIdx.x * 128;
     constexpr int NK1 = IN / 64, NK2 = HID / 64;
     constexpr uint32_t ID1 = tc::idesc_bf16_f32(128, HID), ID3 = tc::idesc_bf16_f32(128, OUTP);
-    if (warp == 4) {
+    if (warp == 8) {
         tc::tmem_alloc(&tmem_slot, 512);
         tc::tmem_relinquish();
     }
-    if (threadIdx.x == 160) {
+    if (threadIdx.x == 288) {
         for (int i = 0; i < FW_S1; ++i) {
             tc::mbar_init(&full1[i], 1);
             tc::mbar_init(&empty1[i], 1);
@@ -316,8 +343,10 @@ k_mlp_forward(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
         tc::mbar_init(&done1, 1);
         tc::mbar_init(&done2, 1);
         tc::mbar_init(&done3, 1);
-        tc::mbar_init(&h1_ready, 128);
-        tc::mbar_init(&h2_ready, 128);
+        for (int i = 0; i < 4; ++i) {
+            tc::mbar_init(&h1_ready[i], 256);
+            tc::mbar_init(&h2_ready[i], 256);
+        }
         fail = 0;
         tc::fence_mbar_init();
         tc::prefetch_tmap(&tmX);
@@ -332,7 +361,7 @@ k_mlp_forward(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
     const uint32_t hbuf = base;
     int issued1 = 0, issued2 = 0;
     bool issued3 = false;
-    if (threadIdx.x == 128) {
+    if (threadIdx.x == 256) {
         // ---- producer
         for (int kt = 0; kt < NK1; ++kt) {
             const int st = kt % FW_S1;
@@ -357,82 +386,89 @@ k_mlp_forward(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
                 issued2 = kt + 1;
             }
         }
-    } else if (threadIdx.x == 160) {
-        // ---- MMA issuer
+    } else if (warp == 9) {
+        // ---- MMA issuer: the warp runs converged, one lane issues (the
+        // descriptors are then warp-uniform values)
+        const bool lead = tc::elect_one();
         bool ok = true;
         for (int kt = 0; kt < NK1 && ok; ++kt) {
             const int st = kt % FW_S1;
-            ok = fw_wait(&full1[st], (kt / FW_S1) & 1, &fail);
+            ok = __all_sync(0xffffffffu, fw_wait(&full1[st], (kt / FW_S1) & 1, &fail));
             if (!ok) break;
             tc::fence_after_sync();
             const uint32_t sa = base + st * FW_STAGE1;
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                tc::mma_bf16(tmem, tc::smem_desc_sw128(sa + kk * 32), tc::smem_desc_sw128(sa + FW_A + kk * 32), ID1,
-                             (kt | kk) != 0 ? 1u : 0u);
-            tc::mma_commit(&empty1[st]);
+            mma_k64(lead, tmem, tc::smem_desc_sw128(sa), tc::smem_desc_sw128(sa + FW_A), ID1, kt != 0, &empty1[st]);
         }
-        tc::mma_commit(&done1);
-        ok = ok && fw_wait(&h1_ready, 0, &fail);
+        if (lead) tc::mma_commit(&done1);
         for (int kt = 0; kt < NK2 && ok; ++kt) {
             const int st = kt & 1;
-            ok = fw_wait(&full2[st], (kt >> 1) & 1, &fail);
+            ok = __all_sync(0xffffffffu, fw_wait(&h1_ready[kt], 0, &fail) && fw_wait(&full2[st], (kt >> 1) & 1, &fail));
             if (!ok) break;
             tc::fence_after_sync();
-            const uint32_t sb = base + FW_W2_OFF + st * FW_B;
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                tc::mma_bf16(tmem + 256u, tc::smem_desc_sw128(hbuf + kt * FW_A + kk * 32),
-                             tc::smem_desc_sw128(sb + kk * 32), ID1, (kt | kk) != 0 ? 1u : 0u);
-            tc::mma_commit(&empty2[st]);
+            mma_k64(lead, tmem + 256u, tc::smem_desc_sw128(hbuf + kt * FW_A),
+                    tc::smem_desc_sw128(base + FW_W2_OFF + st * FW_B), ID1, kt != 0, &empty2[st]);
+            if (lead && keep_hidden) {
+                tma_store_2d(&tmH1, kt * 64, m0, hbuf + kt * FW_A);
+                bulk_commit();
+            }
         }
-        tc::mma_commit(&done2);
-        ok = ok && fw_wait(&h2_ready, 0, &fail) && fw_wait(&full3, 0, &fail);
-        if (ok) {
+        if (lead) {
+            bulk_wait_read();  // h1 has left the buffer that h2 takes after done2
+            tc::mma_commit(&done2);
+        }
+        ok = ok && __all_sync(0xffffffffu, fw_wait(&full3, 0, &fail));
+        for (int kt = 0; kt < NK2 && ok; ++kt) {
+            ok = __all_sync(0xffffffffu, fw_wait(&h2_ready[kt], 0, &fail));
+            if (!ok) break;
             tc::fence_after_sync();
-            for (int kt = 0; kt < NK2; ++kt)
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    tc::mma_bf16(tmem, tc::smem_desc_sw128(hbuf + kt * FW_A + kk * 32),
-                                 tc::smem_desc_sw128(base + FW_W3_OFF + kt * FW_W3_TILE + kk * 32), ID3,
-                                 (kt | kk) != 0 ? 1u : 0u);
+            mma_k64(lead, tmem, tc::smem_desc_sw128(hbuf + kt * FW_A),
+                    tc::smem_desc_sw128(base + FW_W3_OFF + kt * FW_W3_TILE), ID3, kt != 0, nullptr);
+            if (lead && keep_hidden) {
+                tma_store_2d(&tmH2, kt * 64, m0, hbuf + kt * FW_A);
+                bulk_commit();
+            }
         }
-        tc::mma_commit(&done3);
-    } else if (warp < 4) {
-        // ---- epilogue: thread = tile row
-        const int r = warp * 32 + lane;
+        if (lead) {
+            tc::mma_commit(&done3);
+            bulk_wait();
+        }
+    } else if (warp < 8) {
+        // ---- epilogue: thread = tile row and half of every chunk
+        const int r = (warp & 3) * 32 + lane, half = warp >> 2;
         const int m = m0 + r;
-        const bool row_ok = m < batch;
-        const uint32_t lanes = uint32_t(warp * 32) << 16;
-        // warp-uniform decisions: the TMEM loads below are warp-collective
+        const uint32_t lanes = uint32_t((warp & 3) * 32) << 16;
+        auto hidden = [&](bool ok, uint32_t acc, const float* bias, uint64_t* ready) {
+            if (ok) tc::fence_after_sync();
+#pragma unroll 1
+            for (int c = 0; c < NK2; ++c) {
+                if (ok) {
+                    fw_hidden_epilogue(tmem + lanes + acc + uint32_t(64 * c + 32 * half), bias + 64 * c + 32 * half,
+                                       hbuf + uint32_t(c * FW_A), r, half);
+                    tc::fence_before_sync();
+                }
+                tc::fence_proxy_async();  // the chunk, written here, is read by the tensor core and by TMA
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tc::smem_u32(ready + c)) : "memory");
+            }
+        };
+        // warp-uniform decisions: the TMEM loads are warp-collective
         const bool ok1 = __all_sync(0xffffffffu, fw_wait(&done1, 0, &fail));
-        if (ok1) {
-            tc::fence_after_sync();
-            fw_hidden_epilogue(tmem + lanes, b1, (H1 && row_ok) ? H1 + int64_t(m) * HID : nullptr, hbuf, r);
-            tc::fence_before_sync();
-        }
-        tc::fence_proxy_async();  // the h buffer, written here, is read by the tensor core
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tc::smem_u32(&h1_ready)) : "memory");
+        hidden(ok1, 0u, b1, h1_ready);
         const bool ok2 = __all_sync(0xffffffffu, ok1 && fw_wait(&done2, 0, &fail));
-        if (ok2) {
-            tc::fence_after_sync();
-            fw_hidden_epilogue(tmem + lanes + 256u, b2, (H2 && row_ok) ? H2 + int64_t(m) * HID : nullptr, hbuf, r);
-            tc::fence_before_sync();
-        }
-        tc::fence_proxy_async();
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tc::smem_u32(&h2_ready)) : "memory");
-        const bool ok3 = __all_sync(0xffffffffu, ok2 && fw_wait(&done3, 0, &fail));
-        if (ok3) {
-            tc::fence_after_sync();
-            float v[16];
-            tc::tmem_ld16(tmem + lanes, v);
-            if (row_ok)
+        hidden(ok2, 256u, b2, h2_ready);
+        if (warp < 4) {
+            const bool ok3 = __all_sync(0xffffffffu, ok2 && fw_wait(&done3, 0, &fail));
+            if (ok3) {
+                tc::fence_after_sync();
+                float v[16];
+                tc::tmem_ld16(tmem + lanes, v);
+                if (m < batch)
 #pragma unroll
-                for (int j = 0; j < OUT; ++j) Y[int64_t(m) * OUT + j] = v[j] + b3p[j];
+                    for (int j = 0; j < OUT; ++j) Y[int64_t(m) * OUT + j] = v[j] + b3p[j];
+            }
         }
     }
     __syncwarp();
-    if (threadIdx.x == 128) {
+    if (threadIdx.x == 256) {
         // loads issued but never consumed: let them land before the CTA exits
         for (int kt = max(0, issued1 - FW_S1); kt < issued1; ++kt)
             tc::mbar_wait_bounded(&full1[kt % FW_S1], (kt / FW_S1) & 1, tc::MBAR_SPIN_LIMIT);
@@ -440,12 +476,12 @@ k_mlp_forward(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
             tc::mbar_wait_bounded(&full2[kt & 1], (kt >> 1) & 1, tc::MBAR_SPIN_LIMIT);
         if (issued3) tc::mbar_wait_bounded(&full3, 0, tc::MBAR_SPIN_LIMIT);
     }
-    if (threadIdx.x == 160) tc::mbar_wait_bounded(&done3, 0, tc::MBAR_SPIN_LIMIT);  // MMAs in flight
+    if (threadIdx.x == 288) tc::mbar_wait_bounded(&done3, 0, tc::MBAR_SPIN_LIMIT);  // MMAs in flight
     __syncthreads();
     if (threadIdx.x == 0 && *(volatile int*)&fail) atomicOr(err, ERR_TIMEOUT);
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 4) tc::tmem_dealloc(tmem, 512);
+    if (warp == 8) tc::tmem_dealloc(tmem, 512);
 }
 
 }  // namespace
@@ -629,13 +665,15 @@ GemmArgs gargs(const bf16* A, long long a_m, long long a_k, const bf16* B, long 
 // to m->H1 / m->H2 only when the backward pass needs them), or HGMM_ECUDA if
 // its tensor maps cannot be encoded (the caller then runs the three GEMMs).
 int forward_fused(hgmm_mlp* m, const bf16* X, int batch, float* Y, cudaStream_t s, bool keep_hidden) {
-    CUtensorMap tx, t1, t2, t3;
+    CUtensorMap tx, t1, t2, t3, h1 = {}, h2 = {};
     if (!encode_operand(&tx, X, IN, batch, IN, 128) || !encode_operand(&t1, m->W1, IN, HID, IN, HID) ||
-        !encode_operand(&t2, m->W2, HID, HID, HID, HID) || !encode_operand(&t3, m->W3, HID, OUTP, HID, OUTP))
+        !encode_operand(&t2, m->W2, HID, HID, HID, HID) || !encode_operand(&t3, m->W3, HID, OUTP, HID, OUTP) ||
+        (keep_hidden && (!encode_operand(&h1, m->H1, HID, batch, HID, 128) ||
+                         !encode_operand(&h2, m->H2, HID, batch, HID, 128))))
         return HGMM_ECUDA;
-    k_mlp_forward<<<(batch + 127) / 128, FW_THREADS, FW_SMEM, s>>>(tx, t1, t2, t3, m->P + OFF_B1, m->P + OFF_B2,
-                                                                 m->b3p, keep_hidden ? m->H1 : nullptr,
-                                                                 keep_hidden ? m->H2 : nullptr, Y, batch, m->err);
+    k_mlp_forward<<<(batch + 127) / 128, FW_THREADS, FW_SMEM, s>>>(tx, t1, t2, t3, h1, h2, m->P + OFF_B1,
+                                                                 m->P + OFF_B2, m->b3p, keep_hidden, Y, batch,
+                                                                 m->err);
     return cudaGetLastError() == cudaSuccess ? HGMM_OK : HGMM_ECUDA;
 }
 
@@ -726,15 +764,15 @@ int gradients_impl(hgmm_mlp* m, const uint16_t* d_x, const float* d_labels, cons
     k_mlp_wgrad<<<WG_TILES * slices + nchunks, WG_THREADS, WG_SMEM, s>>>(gz1, gx, gz2, gh1, gh2, gdy, batch, slices,
                                                                         wg_chunks(batch), m->dZ1, m->dZ2, m->dYf,
                                                                         m->ws, m->part, m->err);
-    const int ug = int((N_PARAMS + 511) / 512);
+    constexpr int ug = UPDATE_CTAS + UPDATE_BIAS_CTAS;
     if (lr) {
         m->step += 1;
         float c1, c2;
         adam_scales(m->step, &c1, &c2);
-        k_grad_update<true><<<ug, 128, 0, s>>>(m->ws, slices, m->part, nchunks, m->G, m->P, m->Mo, m->Vo, *lr, c1,
+        k_grad_update<true><<<ug, UPDATE_THREADS, 0, s>>>(m->ws, slices, m->part, nchunks, m->G, m->P, m->Mo, m->Vo, *lr, c1,
                                                c2, copies(m));
     } else {
-        k_grad_update<false><<<ug, 128, 0, s>>>(m->ws, slices, m->part, nchunks, m->G, m->P, m->Mo, m->Vo, 0.f, 0.f,
+        k_grad_update<false><<<ug, UPDATE_THREADS, 0, s>>>(m->ws, slices, m->part, nchunks, m->G, m->P, m->Mo, m->Vo, 0.f, 0.f,
                                                 0.f, copies(m));
     }
     return cudaGetLastError() == cudaSuccess ? HGMM_OK : HGMM_ECUDA;

@@ -84,6 +84,15 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t da, uint64_t 
         :: "r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate));
 }
 
+// One lane of a converged warp.  The MMA-issuing warp runs its loop converged
+// and elects a lane only around the issue itself: the descriptors are then
+// warp-uniform values.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(e));
+    return e != 0;
+}
+
 // Arrive once on the mbarrier when every tcgen05.mma this thread issued so
 // far has completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {

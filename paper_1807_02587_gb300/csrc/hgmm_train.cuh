@@ -119,19 +119,11 @@ k_loss(const float* __restrict__ Y, const float* __restrict__ L, int batch, floa
     }
 }
 
-// --------------------------------------------------- TMA stores and MN-major operands
-__device__ __forceinline__ void tma_store_2d(const void* tmap, int x, int y, uint32_t src) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
-                 :: "l"(tmap), "r"(x), "r"(y), "r"(src) : "memory");
-}
+// --------------------------------------------------- bulk stores and MN-major operands
 __device__ __forceinline__ void bulk_s2g(void* dst, uint32_t src, uint32_t bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" :: "l"(dst), "r"(src), "r"(bytes)
                  : "memory");
 }
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 // Descriptor of an operand stored with M (or N) contiguous, in the 128-byte
 // swizzled layout of a TMA box of 64 columns: K rows of 128 bytes, groups of
 // eight rows 1024 bytes apart (stride byte offset), the next 64 columns one
@@ -228,24 +220,26 @@ k_mlp_backward(const __grid_constant__ CUtensorMap tmDY, const __grid_constant__
             tc::tma_load_2d(w2_tile(kt), &tmW2T, kt * 64, 0, &full2[kt]);
             issued2 = kt + 1;
         }
-    } else if (threadIdx.x == 288) {
-        bool ok = fw_wait(&full1, 0, &fail);
-        if (ok) {
-            tc::fence_after_sync();
-            tc::mma_bf16(tmem, tc::smem_desc_sw128(base + BW_DY), tc::smem_desc_sw128(base + BW_W3), ID, 0u);
+    } else if (warp == 9) {
+        const bool lead = tc::elect_one();
+        bool ok = __all_sync(0xffffffffu, fw_wait(&full1, 0, &fail));
+        if (lead) {
+            if (ok) {
+                tc::fence_after_sync();
+                tc::mma_bf16(tmem, tc::smem_desc_sw128(base + BW_DY), tc::smem_desc_sw128(base + BW_W3), ID, 0u);
+            }
+            tc::mma_commit(&done1);
         }
-        tc::mma_commit(&done1);
-        ok = ok && fw_wait(&z_ready, 0, &fail);
+        __syncwarp();
+        ok = ok && __all_sync(0xffffffffu, fw_wait(&z_ready, 0, &fail));
         for (int kt = 0; kt < NK2 && ok; ++kt) {
-            ok = fw_wait(&full2[kt], 0, &fail);
+            ok = __all_sync(0xffffffffu, fw_wait(&full2[kt], 0, &fail));
             if (!ok) break;
             tc::fence_after_sync();
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                tc::mma_bf16(tmem + 256u, tc::smem_desc_sw128(base + kt * FW_A + kk * 32),
-                             tc::smem_desc_sw128(w2_tile(kt) + kk * 32), ID, (kt | kk) != 0 ? 1u : 0u);
+            mma_k64(lead, tmem + 256u, tc::smem_desc_sw128(base + kt * FW_A), tc::smem_desc_sw128(w2_tile(kt)), ID,
+                    kt != 0, nullptr);
         }
-        tc::mma_commit(&done2);
+        if (lead) tc::mma_commit(&done2);
     } else if (warp < 8) {
         const int r = (warp & 3) * 32 + lane, half = warp >> 2, m = m0 + r;
         const uint32_t lanes = uint32_t((warp & 3) * 32) << 16;
@@ -308,6 +302,8 @@ constexpr int WG_BOX = 64 * 128;             // 64 rows x 64 BF16
 constexpr int WG_STAGE = 6 * WG_BOX;         // two A boxes, up to four B boxes
 constexpr int WG_ROW = 1040;
 constexpr int WG_SMEM = WG_STAGES * WG_STAGE + 1024;
+static_assert(OFF_B1 % 4 == 0 && OFF_W2 % 4 == 0 && OFF_B2 % 4 == 0 && OFF_W3 % 4 == 0 && OFF_B3 % 4 == 0,
+              "whole vectors of weights");
 static_assert(128 * WG_ROW <= WG_STAGES * WG_STAGE, "staging inside the ring");
 constexpr int WG_TILES = 2 * (IN / 256) + 2 + 2;
 constexpr int WG_MAX_SLICES = 8;
@@ -398,19 +394,23 @@ k_mlp_wgrad(const __grid_constant__ CUtensorMap tmZ1, const __grid_constant__ CU
             for (int b = 0; b < nb; ++b) tc::tma_load_2d(sa + (2 + b) * WG_BOX, tb, n0 + 64 * b, row, &full[st]);
             issued = kt + 1;
         }
-    } else if (threadIdx.x == 160) {
+    } else if (warp == 5) {
+        const bool lead = tc::elect_one();
         for (int kt = 0; kt < nk; ++kt) {
             const int st = kt % WG_STAGES;
-            if (!fw_wait(&full[st], (kt / WG_STAGES) & 1, &fail)) break;
+            if (!__all_sync(0xffffffffu, fw_wait(&full[st], (kt / WG_STAGES) & 1, &fail))) break;
             tc::fence_after_sync();
             const uint32_t sa = base + st * WG_STAGE;
+            const uint64_t da = smem_desc_mn(sa, WG_BOX), db = smem_desc_mn(sa + 2 * WG_BOX, WG_BOX);
+            if (lead) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)  // 16 rows of 128 bytes
-                tc::mma_bf16(tmem, smem_desc_mn(sa + kk * 2048, WG_BOX), smem_desc_mn(sa + 2 * WG_BOX + kk * 2048, WG_BOX),
-                             idesc, (kt | kk) != 0 ? 1u : 0u);
-            tc::mma_commit(&empty[st]);
+                for (int kk = 0; kk < 4; ++kk)  // 16 rows of 128 bytes
+                    tc::mma_bf16(tmem, da + 128 * kk, db + 128 * kk, idesc, (kt | kk) != 0 ? 1u : 0u);
+                tc::mma_commit(&empty[st]);
+            }
+            __syncwarp();
         }
-        tc::mma_commit(&done);
+        if (lead) tc::mma_commit(&done);
     } else if (warp < 4) {
         const int r = warp * 32 + lane, m = m0 + r;
         const uint32_t tacc = tmem + (uint32_t(warp * 32) << 16);
@@ -489,69 +489,75 @@ __device__ __forceinline__ void adam_one(float g, float& p, float& m, float& v, 
 }
 
 // Gradients from the slices' partials (in slice order) and the column sums
-// (in chunk order), and with ADAM the update in the same pass.
+// (in chunk order), and with ADAM the update in the same pass.  Four weights
+// per thread; the biases, whose column sums add up in FP64, one per thread of
+// the last UPDATE_BIAS_CTAS CTAs (an FP64 warp instruction takes about 64 cycles
+// whatever its lanes do: four per thread made them the slowest of the launch).
+constexpr int UPDATE_THREADS = 128;
+constexpr int UPDATE_BIASES = 2 * HID + OUT;
+constexpr int UPDATE_CTAS = int((N_PARAMS + 4 * UPDATE_THREADS - 1) / (4 * UPDATE_THREADS));
+constexpr int UPDATE_BIAS_CTAS = (UPDATE_BIASES + UPDATE_THREADS - 1) / UPDATE_THREADS;
+
 template <bool ADAM>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(UPDATE_THREADS)
 k_grad_update(const float* __restrict__ ws, int slices, const float* __restrict__ part, int nchunks,
               float* __restrict__ G, float* __restrict__ P, float* __restrict__ Mo, float* __restrict__ Vo, float lr,
               float c1, float c2, WeightCopies w) {
-    const int64_t i0 = 4 * (int64_t(blockIdx.x) * 128 + threadIdx.x);
-    if (i0 >= N_PARAMS) return;
-    const bool whole = i0 + 4 <= N_PARAMS;  // all but the last parameter's thread
-    float pv[4] = {}, mv[4] = {}, vv[4] = {}, g[4];
-    auto load = [&](const float* src, float (&x)[4]) {
-        if (whole) {
-            const float4 t = *reinterpret_cast<const float4*>(src + i0);
-            x[0] = t.x;
-            x[1] = t.y;
-            x[2] = t.z;
-            x[3] = t.w;
-        } else {
-            for (int k = 0; i0 + k < N_PARAMS; ++k) x[k] = src[i0 + k];
+    if (blockIdx.x >= UPDATE_CTAS) {
+        const int b = (int(blockIdx.x) - UPDATE_CTAS) * UPDATE_THREADS + threadIdx.x;
+        if (b >= UPDATE_BIASES) return;
+        const int mat = b / HID, j = b % HID;
+        const int64_t i = (mat == 0 ? OFF_B1 : (mat == 1 ? OFF_B2 : OFF_B3)) + j;
+        double s = 0.0;
+#pragma unroll 8
+        for (int c = 0; c < nchunks; ++c) s += part[(int64_t(c) * 3 + mat) * HID + j];
+        const float g = float(s);
+        G[i] = g;
+        if (ADAM) {
+            float p = P[i], m = Mo[i], v = Vo[i];
+            adam_one(g, p, m, v, lr, c1, c2);
+            Mo[i] = m;
+            Vo[i] = v;
+            P[i] = p;
+            store_copies(i, p, w);
         }
+        return;
+    }
+    const int64_t i0 = 4 * (int64_t(blockIdx.x) * UPDATE_THREADS + threadIdx.x);
+    // the biases' ranges start and end on multiples of four
+    if (i0 >= OFF_B3 || (i0 >= OFF_B1 && i0 < OFF_W2) || (i0 >= OFF_B2 && i0 < OFF_W3)) return;
+    float pv[4], mv[4], vv[4], g[4];
+    auto load = [&](const float* src, float (&x)[4]) {
+        const float4 t = *reinterpret_cast<const float4*>(src + i0);
+        x[0] = t.x;
+        x[1] = t.y;
+        x[2] = t.z;
+        x[3] = t.w;
     };
     auto store = [&](float* dst, const float (&x)[4]) {
-        if (whole) *reinterpret_cast<float4*>(dst + i0) = make_float4(x[0], x[1], x[2], x[3]);
-        else
-            for (int k = 0; i0 + k < N_PARAMS; ++k) dst[i0 + k] = x[k];
+        *reinterpret_cast<float4*>(dst + i0) = make_float4(x[0], x[1], x[2], x[3]);
     };
     if (ADAM) {  // in flight with the partials
         load(P, pv);
         load(Mo, mv);
         load(Vo, vv);
     }
-    const int mat = i0 >= OFF_B3 ? 2 : (i0 >= OFF_B2 && i0 < OFF_W3 ? 1 : (i0 >= OFF_B1 && i0 < OFF_W2 ? 0 : -1));
-    if (mat >= 0) {
-        const int j0 = int(i0 - (mat == 0 ? OFF_B1 : (mat == 1 ? OFF_B2 : OFF_B3)));
-        double s[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll 4
-        for (int c = 0; c < nchunks; ++c) {
-            const float4 x = *reinterpret_cast<const float4*>(part + (int64_t(c) * 3 + mat) * HID + j0);
-            s[0] += x.x;
-            s[1] += x.y;
-            s[2] += x.z;
-            s[3] += x.w;
+    float4 x[WG_MAX_SLICES];
+#pragma unroll
+    for (int z = 0; z < WG_MAX_SLICES; ++z)
+        if (z < slices) x[z] = __ldcg(reinterpret_cast<const float4*>(ws + z * WS_STRIDE + i0));
+    g[0] = x[0].x;
+    g[1] = x[0].y;
+    g[2] = x[0].z;
+    g[3] = x[0].w;
+#pragma unroll
+    for (int z = 1; z < WG_MAX_SLICES; ++z)
+        if (z < slices) {
+            g[0] += x[z].x;
+            g[1] += x[z].y;
+            g[2] += x[z].z;
+            g[3] += x[z].w;
         }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) g[k] = float(s[k]);
-    } else {
-        float4 x[WG_MAX_SLICES];
-#pragma unroll
-        for (int z = 0; z < WG_MAX_SLICES; ++z)
-            if (z < slices) x[z] = __ldcg(reinterpret_cast<const float4*>(ws + z * WS_STRIDE + i0));
-        g[0] = x[0].x;
-        g[1] = x[0].y;
-        g[2] = x[0].z;
-        g[3] = x[0].w;
-#pragma unroll
-        for (int z = 1; z < WG_MAX_SLICES; ++z)
-            if (z < slices) {
-                g[0] += x[z].x;
-                g[1] += x[z].y;
-                g[2] += x[z].z;
-                g[3] += x[z].w;
-            }
-    }
     store(G, g);
     if (ADAM) {
 #pragma unroll
@@ -565,8 +571,7 @@ k_grad_update(const float* __restrict__ ws, int slices, const float* __restrict_
                 make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
         } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (i0 + k < N_PARAMS) store_copies(i0 + k, pv[k], w);
+            for (int k = 0; k < 4; ++k) store_copies(i0 + k, pv[k], w);
         }
     }
 }

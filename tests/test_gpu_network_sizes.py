@@ -1,0 +1,56 @@
+"""The proposal network at the batch sizes where its split of the work changes
+(128-row blocks, 64-row slices of the weight gradients, CTA clusters of four,
+two and one per block) against the FP64 oracle with the same BF16 storage
+points, at the tolerances of tests/test_gpu_proposal.py."""
+import numpy as np
+import pytest
+
+from oracle import mlp_oracle as M
+from tests.test_gpu_proposal import _batch, _bf16, _params, _rel
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [1, 64, 127, 129, 4864, 4865, 9728, 9729])
+def test_forward(n):
+    import torch
+    from paper_1807_02587_gb300 import binding as B
+    p = _params(1)
+    rng = np.random.default_rng(n)
+    X = M.bf16(rng.normal(size=(n, 1280)).astype(np.float32))
+    net = B.Mlp(n)
+    B.hgmm_mlp_set_params(net.handle, p)
+    y = torch.full((n + 1, 9), 7.0, dtype=torch.float32, device="cuda")
+    B.hgmm_mlp_forward(net.handle, _bf16(torch, X), y)
+    B.hgmm_mlp_sync(net.handle)
+    emu, _ = M.forward(p.astype(np.float64), X, act_bf16=True)
+    got = y.cpu().numpy()
+    assert np.all(got[n] == 7.0)  # nothing past the batch
+    assert _rel(got[:n], emu) < 1e-3
+
+
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 129, 513, 1100, 4900])
+def test_gradients_and_update(n):
+    import torch
+    from paper_1807_02587_gb300 import binding as B
+    p = _params(3)
+    X, L = _batch(4, n)
+    x, lab = _bf16(torch, X), torch.from_numpy(L).cuda()
+    net = B.Mlp(n)
+    B.hgmm_mlp_set_params(net.handle, p)
+    loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+    B.hgmm_mlp_gradients(net.handle, x, lab, n, w_t=2.0, loss=loss)
+    B.hgmm_mlp_sync(net.handle)
+    g = B.hgmm_mlp_read_grads(net.handle)
+    emu_loss, emu, _ = M.backward(p.astype(np.float64), X, L.astype(np.float64), 2.0, act_bf16=True)
+    assert abs(loss.item() - emu_loss) < 1e-4 * emu_loss
+    G, E = M.unpack(g.astype(np.float64)), M.unpack(emu)
+    for name, _ in M.SHAPES:
+        assert _rel(G[name], E[name]) < 2e-3, name
+    # the step that updates in the same pass: the same gradients, Adam's first update
+    B.hgmm_mlp_train_step(net.handle, x, lab, n, w_t=2.0, lr=1e-3, loss=loss)
+    B.hgmm_mlp_sync(net.handle)
+    assert np.array_equal(B.hgmm_mlp_read_grads(net.handle), g)
+    w, _, _ = M.adam_step(p.astype(np.float64), g.astype(np.float64), 0.0, 0.0, 1, 1e-3)
+    got = B.hgmm_mlp_get_params(net.handle).astype(np.float64)
+    assert np.max(np.abs(got - w)) < 1e-6 * (1 + np.abs(w)).max()
