@@ -376,16 +376,75 @@ k_em_coop(int level, int n, int n_par, int K, int n_chunks, const float4* __rest
     }
 }
 
-__global__ void __launch_bounds__(EST_THREADS) k_assign(const float4* __restrict__ pts,
-                                                        const Item* __restrict__ items,
-                                                        const int* __restrict__ meta,
-                                                        const NodeEst* __restrict__ est_lvl,
-                                                        uint32_t* __restrict__ codes,
-                                                        int* __restrict__ item_cnt) {
-    __shared__ AssignSmem as;
+// Argmax hand-off, one warp per item (at most TILE points) and one lane per
+// point: the eight children's constants sit in registers (reloaded when the
+// warp's parent changes: its items are consecutive), a point's rank among the
+// item's points of its child is a running count per child (lane c holds child
+// c's) plus the ballot's bits below the lane, and no CTA barrier is needed.
+// The labels, ranks and counts are those of assign_item (same scores, ties to
+// the lowest index).  A quad of lanes per point, eight ballots per eight points
+// and a barrier per item took 521 us per level of 16.8M points (2,085 us of the
+// build), this 168 us.
+constexpr int ASSIGN_THREADS = 256;
+__global__ void __launch_bounds__(ASSIGN_THREADS, 2)
+k_assign(const float4* __restrict__ pts, const Item* __restrict__ items, const int* __restrict__ meta,
+         const NodeEst* __restrict__ est_lvl, uint32_t* __restrict__ codes, int* __restrict__ item_cnt) {
+    constexpr int STEPS = TILE / 32, AHEAD = 4;
     const int n_items = meta[0];
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x)
-        assign_item(pts, items[it], it, est_lvl, codes, item_cnt, as);
+    const int lane = threadIdx.x & 31;
+    const int64_t gw = blockIdx.x * (ASSIGN_THREADS / 32) + (threadIdx.x >> 5);
+    const int64_t warps = int64_t(gridDim.x) * (ASSIGN_THREADS / 32);
+    const int ib = int(gw * n_items / warps), ie = int((gw + 1) * n_items / warps);
+    const unsigned lt = (1u << lane) - 1u;
+    ChildPair cp[4];
+    int cur = -1;
+    for (int it = ib; it < ie; ++it) {
+        const Item w = items[it];
+        float4 z[AHEAD];
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k) z[k] = pts[w.start + min(32 * k + lane, w.count - 1)];
+        if (w.parent != cur) {
+            cur = w.parent;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) load_child_pair(est_lvl + 8 * cur + 2 * k, cp[k]);
+        }
+        int count = 0;  // of child `lane` (lanes 0..7) in the steps before
+#pragma unroll
+        for (int st = 0; st < STEPS; ++st) {
+            if (32 * st >= w.count) break;
+            const float4 p = z[st % AHEAD];
+            if (st + AHEAD < STEPS) z[st % AHEAD] = pts[w.start + min(32 * (st + AHEAD) + lane, w.count - 1)];
+            int lab = 0;
+            float best = 0.f;  // of the negated scores
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float2 ex, ey, ez;
+                const float2 u = neg_score_pair(cp[k], p.x, p.y, p.z, ex, ey, ez);
+                if (k == 0 || u.x < best) {
+                    best = u.x;
+                    lab = 2 * k;
+                }
+                if (u.y < best) {
+                    best = u.y;
+                    lab = 2 * k + 1;
+                }
+            }
+            const int i = 32 * st + lane;
+            const bool valid = i < w.count;
+            unsigned mine = 0;
+            int add = 0;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const unsigned m = __ballot_sync(FULL, valid && lab == c);
+                if (lab == c) mine = m;
+                if (lane == c) add = __popc(m);
+            }
+            const int rank = __shfl_sync(FULL, count, lab) + __popc(mine & lt);
+            count += add;
+            if (valid) codes[w.start + i] = uint32_t(lab) | (uint32_t(rank) << 3);
+        }
+        if (lane < 8) item_cnt[8 * it + lane] = count;
+    }
 }
 
 // Slice j of the nsl slices of a parent's items [i0, i1).
@@ -466,6 +525,11 @@ __global__ void __launch_bounds__(256) k_child_offsets(int level, int n,
     child_offsets_scan(a, b, item_cnt, item_off, os);
 }
 
+// Stable 8-way partition of every parent's segment, one warp per item: all of
+// an item's loads are in flight before its stores (one CTA per item, a point
+// per thread and one load chain each took 227 us per level of 16.8M points,
+// this 134; reading and writing the points, codes and permutation is
+// 740 MB, 109 us at the copy rate).
 __global__ void __launch_bounds__(256) k_scatter(const float4* __restrict__ pts_in,
                                                  const int* __restrict__ perm_in,
                                                  const Item* __restrict__ items,
@@ -474,10 +538,31 @@ __global__ void __launch_bounds__(256) k_scatter(const float4* __restrict__ pts_
                                                  const int* __restrict__ item_off,
                                                  float4* __restrict__ pts_out,
                                                  int* __restrict__ perm_out) {
+    constexpr int STEPS = TILE / 32;
     const int n_items = meta[0];
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x)
-        scatter_item(pts_in, perm_in, items[it], it, codes, item_off, pts_out, perm_out,
-                     threadIdx.x, blockDim.x);
+    const int lane = threadIdx.x & 31;
+    for (int it = blockIdx.x * 8 + (threadIdx.x >> 5); it < n_items; it += gridDim.x * 8) {
+        const Item w = items[it];
+        const int off = item_off[8 * it + (lane & 7)];
+        uint32_t code[STEPS];
+        float4 z[STEPS];
+        int from[STEPS];
+#pragma unroll
+        for (int k = 0; k < STEPS; ++k) {
+            const int pos = w.start + min(32 * k + lane, w.count - 1);
+            code[k] = codes[pos];
+            z[k] = pts_in[pos];
+            from[k] = perm_in ? perm_in[pos] : pos;
+        }
+#pragma unroll
+        for (int k = 0; k < STEPS; ++k) {
+            const int dst = __shfl_sync(FULL, off, code[k] & 7u) + int(code[k] >> 3);
+            if (32 * k + lane < w.count) {
+                pts_out[dst] = z[k];
+                perm_out[dst] = from[k];
+            }
+        }
+    }
 }
 
 __global__ void k_finalize(int level, float lam_c, const RootDev* __restrict__ root,
@@ -713,7 +798,7 @@ int hgmm_build_impl(hgmm_tree* t, const float4* pts, int64_t n64, int depth,
         if (stop_here) return HGMM_OK;  // checking aid: parameters after em_iters
         {
             ProfScope ps_(t, K_ASSIGN, s);
-            k_assign<<<t->n_sm * 4, EST_THREADS, 0, s>>>(cur, t->items, t->meta, est_lvl, t->codes, t->item_cnt);
+            k_assign<<<t->n_sm * 2, ASSIGN_THREADS, 0, s>>>(cur, t->items, t->meta, est_lvl, t->codes, t->item_cnt);
         }
         {
             ProfScope ps_(t, K_OFFSETS, s);
@@ -731,7 +816,7 @@ int hgmm_build_impl(hgmm_tree* t, const float4* pts, int64_t n64, int depth,
         float4* out = t->pts[l & 1];
         {
             ProfScope ps_(t, K_SCATTER, s);
-            k_scatter<<<G, 256, 0, s>>>(cur, perm_prev, t->items, t->meta, t->codes, t->item_off,
+            k_scatter<<<t->n_sm * 4, 256, 0, s>>>(cur, perm_prev, t->items, t->meta, t->codes, t->item_off,
                                         out, t->perm[l]);
         }
         const int m = int(level_size(l));

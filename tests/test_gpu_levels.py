@@ -40,15 +40,18 @@ def test_em_iterations_of_every_level(kind, n, depth):
         assert r["mu"] < 1e-5 and r["S"] < 1e-5 and r["pi"] < 1e-5, r
 
 
-@pytest.mark.parametrize("kind,n,depth", [("scene", 300, 3), ("scene", 256 * CHUNKS + 1, 3), ("blob", 60000, 4),
-                                          ("scene", 20000, 5)])
-def test_segments_partition_the_points(kind, n, depth):
+@pytest.mark.parametrize("precision", [0, 1])  # 1: the level-wide launches at every size
+@pytest.mark.parametrize("kind,n,depth", [("scene", 8, 2), ("scene", 300, 3), ("scene", 256 * CHUNKS + 1, 3),
+                                          ("blob", 60000, 4), ("scene", 20000, 5), ("scene", 409601, 2)])
+def test_segments_partition_the_points(kind, n, depth, precision):
     """After every hand-off each node's segment holds exactly the points
-    labelled with it, children inside their parent, and two builds agree."""
+    labelled with it, children inside their parent, every point with its best
+    child under the level's parameters (near-ties aside), and two builds agree."""
     from paper_1807_02587_gb300 import binding as B
     dev, Z = PT.device_cloud(_cloud(kind, n))
+    prm = B.params(precision=precision)
     tree = B.Tree(n, depth)
-    tree.build(dev, depth)
+    tree.build(dev, depth, prm)
     tree.sync()
     prev = np.zeros(n, np.int64)
     first = []
@@ -57,9 +60,12 @@ def test_segments_partition_the_points(kind, n, depth):
         assert np.array_equal(lab // 8, prev), l
         g = tree.export(l)
         assert np.array_equal(np.bincount(lab, minlength=8 ** (l + 1)), g["count"]), l
+        if n <= 100000:
+            ref, margin = PT.handoff_check(Z, prev, g)
+            assert not np.any((lab != ref) & (margin >= PT.TIE_MARGIN)), l
         first.append((lab, g))
         prev = lab
-    tree.build(dev, depth)
+    tree.build(dev, depth, prm)
     tree.sync()
     for l in range(depth):
         assert np.array_equal(tree.labels(l), first[l][0])
