@@ -1957,7 +1957,7 @@ __device__ __forceinline__ bool warp_solve_update(const double* tot, double* T, 
 // takes partials w, w + 8, ...; then the eight group sums in order), the
 // objective to *obj, and the FP64 solve and pose update by warp 0.  A
 // singular system records ST_DEGENERATE and keeps T (also in T_hist).
-__device__ inline void sum_terms_and_solve(const float2* __restrict__ tpart, int nb, int it, double* T,
+__device__ inline void sum_terms_and_solve(const float2* tpart, int nb, int it, double* T,
                                            float* Rt, double* T_hist, double* obj, int* status) {
     __shared__ float2 fin[8][32];
     __shared__ double tot[NTERM];
@@ -1965,8 +1965,9 @@ __device__ inline void sum_terms_and_solve(const float2* __restrict__ tpart, int
     if (warp < 8) {
         float S = 0.f, C = 0.f;
         if (lane < NTERM)
+#pragma unroll 4
             for (int b = warp; b < nb; b += 8) {
-                const float2 x = tpart[NTERM * b + lane];
+                const float2 x = __ldcg(tpart + NTERM * b + lane);  // perhaps written in this launch
                 pair_add(S, C, x.x, x.y);
             }
         fin[warp][lane] = make_float2(S, C);

@@ -608,12 +608,18 @@ __device__ __forceinline__ void scatter_terms(const float (&P)[3][3], const floa
 // a warp reduce-scatter per 32 nodes, the CTA's eight warp sums in order);
 // the accumulators are cleared for the next round.  FULL adds the scatter
 // terms of the full Eq. 7 from the second moments.
+// The last CTA to finish sums the CTAs' partials in a fixed order, solves and
+// updates the pose (a launch of its own for that took 6.6 us a round, most of it
+// its start and its first loads).
 template <bool FULL>
 __global__ void __launch_bounds__(VAR_THREADS)
 k_var_terms(int n_nodes, int n, const NodeEst* __restrict__ est, const float4* __restrict__ rnode,
             const RootDev* __restrict__ root, unsigned long long* __restrict__ acc,
-            unsigned long long* __restrict__ acc2, float2* __restrict__ part, double* __restrict__ dbg) {
+            unsigned long long* __restrict__ acc2, float2* __restrict__ part, double* __restrict__ dbg,
+            unsigned* __restrict__ arrived, int it, double* T, float* Rt, double* T_hist, double* obj,
+            int* status) {
     __shared__ float2 sm[VAR_THREADS / 32][NTERM];
+    __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = blockIdx.x * VAR_THREADS + threadIdx.x;
     __shared__ float s_scale[2];
@@ -684,12 +690,17 @@ k_var_terms(int n_nodes, int n, const NodeEst* __restrict__ est, const float4* _
         for (int k = 0; k < VAR_THREADS / 32; ++k) pair_add(S, C, sm[k][threadIdx.x].x, sm[k][threadIdx.x].y);
         part[NTERM * blockIdx.x + threadIdx.x] = make_float2(S, C);
     }
-}
-
-__global__ void __launch_bounds__(VAR_THREADS)
-k_var_solve(const float2* __restrict__ part, int nb, int it, double* __restrict__ T, float* __restrict__ Rt,
-            double* __restrict__ T_hist, double* __restrict__ obj, int* __restrict__ status) {
-    sum_terms_and_solve(part, nb, it, T, Rt, T_hist, obj, status);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(arrived, 1u) == gridDim.x - 1;
+        if (last) {
+            *arrived = 0u;  // ready for the next round
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    if (last) sum_terms_and_solve(part, gridDim.x, it, T, Rt, T_hist, obj, status);
 }
 
 }  // namespace
@@ -817,12 +828,12 @@ int hgmm_register_descent_impl(hgmm_tree* t, const float4* src, int64_t n64, con
 #undef HGMM_DESCEND
         if (full)
             k_var_terms<true><<<tgrid, VAR_THREADS, 0, s>>>(n_nodes, n, t->est, t->rnode, t->root, t->reg_acc,
-                                                            t->reg_acc2, t->reg_part, t->reg_dbg);
+                                                            t->reg_acc2, t->reg_part, t->reg_dbg, t->reg_bar + 6,
+                                                            it, t->reg_T, t->reg_Rt, T_hist, t->reg_obj, t->status);
         else
             k_var_terms<false><<<tgrid, VAR_THREADS, 0, s>>>(n_nodes, n, t->est, t->rnode, t->root, t->reg_acc,
-                                                             t->reg_acc2, t->reg_part, t->reg_dbg);
-        k_var_solve<<<1, VAR_THREADS, 0, s>>>(t->reg_part, tgrid, it, t->reg_T, t->reg_Rt, T_hist, t->reg_obj,
-                                              t->status);
+                                                             t->reg_acc2, t->reg_part, t->reg_dbg, t->reg_bar + 6,
+                                                             it, t->reg_T, t->reg_Rt, T_hist, t->reg_obj, t->status);
     }
     if (T_out) k_copy_T<<<1, 32, 0, s>>>(t->reg_T, T_out);
     const cudaError_t e = cudaGetLastError();
