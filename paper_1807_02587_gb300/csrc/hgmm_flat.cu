@@ -3,7 +3,7 @@
 // of Eq. 8 over every (point, component) pair, and the tree's M-step
 // (Eq. 9-16) and pose update.
 //
-// One round is four launches:
+// One round is three launches:
 //   k_flat_lse      four lanes per two points (each lane every fourth
 //                   component), components staged in shared memory:
 //                   log2 sum_j pi_j N(z'|Theta_j) of every point (chunks of
@@ -19,9 +19,9 @@
 //   k_flat_terms    32 components per CTA, eight warps splitting the
 //                   slices: fixed-order sums, then per component the Eq. 12-16
 //                   normal-equation and objective terms (node_terms) and a
-//                   warp reduce-scatter to one partial per CTA.
-//   k_flat_solve    fixed-order sum of the CTA partials, FP64 solve and
-//                   T <- dT T by one warp (warp_solve_update).
+//                   warp reduce-scatter to one partial per CTA; the last CTA
+//                   sums those in a fixed order and one of its warps solves in
+//                   FP64 and updates T <- dT T (warp_solve_update).
 // Every sum has a fixed order, so a registration is bit-reproducible.
 #include <cstdio>
 #include <cstring>
@@ -51,40 +51,44 @@ constexpr int LSE_PPT = 2;       // points per thread
 constexpr int LSE_SPLIT = 4;     // lanes sharing one point group (each takes every 4th component)
 constexpr int LSE_POINTS = LSE_THREADS / LSE_SPLIT * LSE_PPT;  // points per CTA
 constexpr int LSE_TILE = 512;    // components staged per pass
+constexpr int GROUP = 8 * LSE_SPLIT;  // components of one chunk of a point group's lanes, and of a warp of moments
+static_assert(GROUP == 32 && LSE_TILE % GROUP == 0, "whole groups");
+constexpr size_t GMAX_KEPT = size_t(1) << 30;  // largest table of group maxima (4 GB)
 constexpr int MOM_THREADS = 256; // one component per thread
-constexpr int MOM_STAGE = 256;   // points staged per pass
+constexpr int MOM_STAGE = 2048;  // points staged per pass (a slice of an ordinary cloud)
 constexpr int NMOM_MAX = 10;
 
 // ------------------------------------------------------------ from the tree
 // One CTA.  Candidates are the nodes of levels 0..L-1 (global id order);
 // thread t takes a contiguous run of them, so the block scan of the run
-// counts gives the components in (level, index) order.
+// counts gives the components in (level, index) order.  slot[g] = component
+// of node g (-1: none), wt[g] = its path product, wtot = the products' sum.
 __global__ void __launch_bounds__(FROM_TREE_THREADS)
-k_flat_from_tree(const NodeStat* __restrict__ st, const RootDev* __restrict__ root, int L, int n_cand,
-                 FlatComp* __restrict__ comp, NodeEst* __restrict__ est, float4* __restrict__ rterm,
-                 int* __restrict__ meta, double* __restrict__ eps_out, int* __restrict__ status) {
+k_flat_select(const NodeStat* __restrict__ st, const RootDev* __restrict__ root, int L, int n_cand,
+              int* __restrict__ slot, double* __restrict__ wt, double* __restrict__ wtot, int* __restrict__ meta,
+              double* __restrict__ eps_out, int* __restrict__ status) {
     __shared__ int wcount[FROM_TREE_THREADS / 32];
     __shared__ double wsum[FROM_TREE_THREADS / 32];
-    __shared__ double total_sh;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int per = (n_cand + FROM_TREE_THREADS - 1) / FROM_TREE_THREADS;
     const int g0 = min(n_cand, t * per), g1 = min(n_cand, g0 + per);
-    // pass 1: flags, weights, counts
     int cnt = 0;
     double wsum_t = 0.0;
     for (int g = g0; g < g1; ++g) {
         int l = 0;
         while (l + 1 < L && g >= d_level_offset(l + 1)) ++l;
         const int64_t i = g - d_level_offset(l);
-        if (!st[g].live) continue;
-        bool child = false;
+        bool leaf = st[g].live != 0;
         if (l + 1 < L) {
             const int64_t c0 = d_level_offset(l + 1) + 8 * i;
-            for (int c = 0; c < 8; ++c) child = child || st[c0 + c].live;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) leaf = leaf && !st[c0 + c].live;
         }
-        if (child) continue;
+        slot[g] = leaf ? cnt : -1;  // within the thread's run for now
+        if (!leaf) continue;
         double w = 1.0;
         for (int k = 0; k <= l; ++k) w = st[d_level_offset(k) + (i >> (3 * (l - k)))].pi * w;
+        wt[g] = w;
         wsum_t += w;
         ++cnt;
     }
@@ -108,48 +112,49 @@ k_flat_from_tree(const NodeStat* __restrict__ st, const RootDev* __restrict__ ro
             run += c;
             tot += wsum[w];
         }
-        total_sh = tot;
+        *wtot = tot;
         meta[0] = run;
         *eps_out = root->eps;
         if (!(tot > 0.0)) atomicOr(status, ST_DEGENERATE);
     }
     __syncthreads();
-    const double inv_total = total_sh > 0.0 ? 1.0 / total_sh : 0.0;
-    const double eps = root->eps;
-    int j = wcount[warp] + incl - cnt;
-    // pass 2: write the components
-    for (int g = g0; g < g1; ++g) {
-        int l = 0;
-        while (l + 1 < L && g >= d_level_offset(l + 1)) ++l;
-        const int64_t i = g - d_level_offset(l);
-        const NodeStat& s = st[g];
-        if (!s.live) continue;
-        bool child = false;
-        if (l + 1 < L) {
-            const int64_t c0 = d_level_offset(l + 1) + 8 * i;
-            for (int c = 0; c < 8; ++c) child = child || st[c0 + c].live;
-        }
-        if (child) continue;
-        double w = 1.0;
-        for (int k = 0; k <= l; ++k) w = st[d_level_offset(k) + (i >> (3 * (l - k)))].pi * w;
-        FlatComp& f = comp[j];
-        f.pi = w * inv_total;
-        for (int a = 0; a < 3; ++a) f.mu[a] = s.mu[a];
-        for (int v = 0; v < 6; ++v) f.S[v] = s.S[v];
-        for (int a = 0; a < 3; ++a) f.lam[a] = s.lam[a];
-        for (int v = 0; v < 9; ++v) f.V[v] = s.V[v];
-        for (int v = 0; v < 6; ++v) f.P[v] = s.P[v];
-        f.live = 1;
-        f.level = l;
-        f.index = int(i);
-        if (!pack_est(f.pi, f.mu, f.S, eps, 0.f, est[j])) atomicOr(status, ST_CHOL);
-        const float4 a = est[j].a;
-        rterm[3 * j] = make_float4(float(s.P[0]), float(s.P[1]), float(s.P[2]), float(s.P[3]));
-        rterm[3 * j + 1] = make_float4(float(s.P[4]), float(s.P[5]), 0.f, 0.f);
-        rterm[3 * j + 2] = make_float4(float(s.mu[0] - double(a.x)), float(s.mu[1] - double(a.y)),
-                                       float(s.mu[2] - double(a.z)), 0.f);
-        ++j;
-    }
+    const int first = wcount[warp] + incl - cnt;
+    for (int g = g0; g < g1; ++g)
+        if (slot[g] >= 0) slot[g] += first;
+}
+
+// The components, one thread per candidate (one CTA doing the selection and
+// the FP64 Cholesky factors of all of them took 170 us for 4,680 candidates;
+// the two launches 39).
+__global__ void __launch_bounds__(64)
+k_flat_write(const NodeStat* __restrict__ st, int n_cand, const int* __restrict__ slot,
+             const double* __restrict__ wt, const double* __restrict__ wtot, const double* __restrict__ eps_in,
+             FlatComp* __restrict__ comp, NodeEst* __restrict__ est, float4* __restrict__ rterm,
+             int* __restrict__ status) {
+    const int g = blockIdx.x * 64 + threadIdx.x;
+    if (g >= n_cand) return;
+    const int j = slot[g];
+    if (j < 0) return;
+    int l = 0;
+    while (g >= d_level_offset(l + 1)) ++l;
+    const NodeStat& s = st[g];
+    const double total = *wtot;
+    FlatComp& f = comp[j];
+    f.pi = wt[g] * (total > 0.0 ? 1.0 / total : 0.0);
+    for (int a = 0; a < 3; ++a) f.mu[a] = s.mu[a];
+    for (int v = 0; v < 6; ++v) f.S[v] = s.S[v];
+    for (int a = 0; a < 3; ++a) f.lam[a] = s.lam[a];
+    for (int v = 0; v < 9; ++v) f.V[v] = s.V[v];
+    for (int v = 0; v < 6; ++v) f.P[v] = s.P[v];
+    f.live = 1;
+    f.level = l;
+    f.index = int(g - d_level_offset(l));
+    if (!pack_est(f.pi, f.mu, f.S, *eps_in, 0.f, est[j])) atomicOr(status, ST_CHOL);
+    const float4 a = est[j].a;
+    rterm[3 * j] = make_float4(float(s.P[0]), float(s.P[1]), float(s.P[2]), float(s.P[3]));
+    rterm[3 * j + 1] = make_float4(float(s.P[4]), float(s.P[5]), 0.f, 0.f);
+    rterm[3 * j + 2] = make_float4(float(s.mu[0] - double(a.x)), float(s.mu[1] - double(a.y)),
+                                   float(s.mu[2] - double(a.z)), 0.f);
 }
 
 // ------------------------------------------------------------- E-step parts
@@ -189,13 +194,19 @@ __device__ __forceinline__ void comp_from_smem(const float4* sc, int c, ChildReg
     r.w21 = d.x; r.w22 = d.y;
 }
 
-// Running log2-sum-exp2 of one point over a chunk of K scores: one rescale
-// of the running sum per chunk.  -inf scores (dead components) add nothing.
 template <int K>
-__device__ __forceinline__ void lse_chunk(const float (&s)[K], float& m, float& sum) {
+__device__ __forceinline__ float chunk_max(const float (&s)[K]) {
     float cm = s[0];
 #pragma unroll
     for (int k = 1; k < K; ++k) cm = fmaxf(cm, s[k]);
+    return cm;
+}
+
+// Running log2-sum-exp2 of one point over a chunk of K scores with maximum cm:
+// one rescale of the running sum per chunk.  -inf scores (dead components) add
+// nothing.
+template <int K>
+__device__ __forceinline__ void lse_chunk(const float (&s)[K], float cm, float& m, float& sum) {
     const float nm = fmaxf(m, cm);
     const float ref = nm == -CUDART_INF_F ? 0.f : nm;
     float acc = sum * exp2f(m - ref);
@@ -205,11 +216,15 @@ __device__ __forceinline__ void lse_chunk(const float (&s)[K], float& m, float& 
     m = nm;
 }
 
+// A posterior 2^(score - lse) below 2^-126 flushes to zero: a score further
+// than this below lse (or below any score of the point) contributes nothing.
+constexpr float SKIP = 127.f;
+
 template <bool XF>
 __global__ void __launch_bounds__(LSE_THREADS)
 k_flat_lse(const float4* __restrict__ pts, int n, const float* __restrict__ Rt,
            const NodeEst* __restrict__ est, const int* __restrict__ meta, float* __restrict__ lse,
-           int* __restrict__ status) {
+           float* __restrict__ gmax, int64_t gstride, int* __restrict__ status) {
     __shared__ float4 sc[3 * LSE_TILE];
     const int J = meta[0];
     // lane = 4 * (point group within the warp) + phase; the four lanes of a
@@ -229,6 +244,26 @@ k_flat_lse(const float4* __restrict__ pts, int n, const float* __restrict__ Rt,
         m[k] = -CUDART_INF_F;
         sum[k] = 0.f;
     }
+    // the largest score of each point over a group of components (its four
+    // lanes'), kept for the moments' skipping; returns whether the group can
+    // matter to any of the warp's points, given the scores so far
+    float top[LSE_PPT];
+#pragma unroll
+    for (int k = 0; k < LSE_PPT; ++k) top[k] = -CUDART_INF_F;
+    auto group_matters = [&](int group, float (&hi)[LSE_PPT]) {
+        bool far = true;
+#pragma unroll
+        for (int k = 0; k < LSE_PPT; ++k) {
+            hi[k] = fmaxf(hi[k], __shfl_xor_sync(FULL, hi[k], 1));
+            hi[k] = fmaxf(hi[k], __shfl_xor_sync(FULL, hi[k], 2));
+            far = far && hi[k] < top[k] - SKIP;
+            top[k] = fmaxf(top[k], hi[k]);
+        }
+        const int i = blockIdx.x * LSE_POINTS + phase * GROUPS + grp;
+        if (gmax && phase < LSE_PPT && i < n) gmax[group * gstride + i] = phase == 0 ? hi[0] : hi[LSE_PPT - 1];
+        return !__all_sync(FULL, far);
+    };
+    static_assert(LSE_PPT == 2 && LSE_SPLIT == 4, "two points a lane");
     for (int j0 = 0; j0 < J; j0 += LSE_TILE) {
         const int cnt = min(LSE_TILE, J - j0);
         __syncthreads();
@@ -236,7 +271,7 @@ k_flat_lse(const float4* __restrict__ pts, int n, const float* __restrict__ Rt,
         for (int q = threadIdx.x; q < 3 * cnt; q += LSE_THREADS) sc[q] = src[q];
         __syncthreads();
         int c = phase;
-        for (; c + 7 * LSE_SPLIT < cnt; c += 8 * LSE_SPLIT) {
+        for (; c - phase + GROUP <= cnt; c += GROUP) {
             float s[LSE_PPT][8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -248,18 +283,31 @@ k_flat_lse(const float4* __restrict__ pts, int n, const float* __restrict__ Rt,
                     s[k][u] = child_score(cr, zx[k], zy[k], zz[k], ex, ey, ez);
                 }
             }
+            float cm[LSE_PPT], hi[LSE_PPT];
 #pragma unroll
-            for (int k = 0; k < LSE_PPT; ++k) lse_chunk<8>(s[k], m[k], sum[k]);
-        }
-        for (; c < cnt; c += LSE_SPLIT) {
-            ChildRegs cr;
-            comp_from_smem(sc, c, cr);
+            for (int k = 0; k < LSE_PPT; ++k) cm[k] = hi[k] = chunk_max<8>(s[k]);
+            if (group_matters((j0 + c) / GROUP, hi)) {
 #pragma unroll
-            for (int k = 0; k < LSE_PPT; ++k) {
-                float ex, ey, ez;
-                float s1[1] = {child_score(cr, zx[k], zy[k], zz[k], ex, ey, ez)};
-                lse_chunk<1>(s1, m[k], sum[k]);
+                for (int k = 0; k < LSE_PPT; ++k) lse_chunk<8>(s[k], cm[k], m[k], sum[k]);
             }
+        }
+        if (c - phase < cnt) {  // a last, partial group
+            const int group = (j0 + c) / GROUP;
+            float hi[LSE_PPT];
+#pragma unroll
+            for (int k = 0; k < LSE_PPT; ++k) hi[k] = -CUDART_INF_F;
+            for (; c < cnt; c += LSE_SPLIT) {
+                ChildRegs cr;
+                comp_from_smem(sc, c, cr);
+#pragma unroll
+                for (int k = 0; k < LSE_PPT; ++k) {
+                    float ex, ey, ez;
+                    const float s1[1] = {child_score(cr, zx[k], zy[k], zz[k], ex, ey, ez)};
+                    hi[k] = fmaxf(hi[k], s1[0]);
+                    lse_chunk<1>(s1, s1[0], m[k], sum[k]);
+                }
+            }
+            group_matters(group, hi);
         }
     }
     // combine the four partial (max, sum) pairs of each point group
@@ -311,20 +359,33 @@ __device__ __forceinline__ void fold_mom(float (&in)[NM], float (&s)[NM], float 
     }
 }
 
-// Partial moments of components [tile*256, tile*256 + 256) over the points
-// of one slice; NM = 4 (gamma, gamma e) or 10 (and gamma e e^T), e = z' - mu32.
+// Partial moments of a tile of 256 components over the points of one slice; NM = 4 (gamma, gamma e) or 10 (and gamma e e^T), e = z' - mu32.
+// Issue bounds it (22 instructions per 32 pairs at 79 % of the issue slots;
+// packing two components or points into FP32x2 instructions halves their
+// number and leaves the time as it was: 159 against 162 us), so the pairs
+// have to become fewer.  Most posteriors are exactly zero: 2^(score - lse) below
+// 2^-126 flushes to zero, which 92 % of the (point, component) pairs of a
+// 93k-point LiDAR cloud and its 2,200 components do (all 32 components of a warp for
+// three quarters of the points), and adding zeros changes no sum.  So each warp
+// runs over the points whose largest score in its group of components, as
+// k_flat_lse recorded it, lies within SKIP of lse, in their order and with the
+// same folds (162 -> 95 us).
 template <int NM, bool XF>
 __global__ void __launch_bounds__(MOM_THREADS)
 k_flat_moments(const float4* __restrict__ pts, int n, const float* __restrict__ Rt,
                const float* __restrict__ lse, const NodeEst* __restrict__ est,
-               const int* __restrict__ meta, int max_ctas, float2* __restrict__ part) {
+               const int* __restrict__ meta, int max_ctas, const float* __restrict__ gmax, int64_t gstride,
+               float2* __restrict__ part) {
     __shared__ float4 sp[MOM_STAGE];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int J = meta[0];
     const FlatPlan pl = flat_plan(J, n, max_ctas);
     const int tile = blockIdx.x % pl.tiles, slice = blockIdx.x / pl.tiles;
     if (slice >= pl.slices) return;  // uniform over the CTA
     const int slice_len = pl.slice_len, jpad = pl.jpad;
-    const int j = tile * MOM_THREADS + threadIdx.x;
+    // the tiles deal the groups of components out in turn: the wide components
+    // of a tree's shallow leaves, which few points skip, lie side by side
+    const int group = tile + pl.tiles * warp, j = group * GROUP + lane;
     const bool own = j < J;
     ChildRegs cr;
     if (own) {
@@ -356,22 +417,48 @@ k_flat_moments(const float4* __restrict__ pts, int n, const float* __restrict__ 
     for (int b = i0; b < i1; b += MOM_STAGE) {
         const int cnt = min(MOM_STAGE, i1 - b);
         __syncthreads();
-        if (threadIdx.x < cnt) {
-            const int i = b + threadIdx.x;
+        for (int q = threadIdx.x; q < cnt; q += MOM_THREADS) {
             float x, y, z;
-            const bool fin = load_point<XF>(pts, i, r, x, y, z, nullptr);  // reported by k_flat_lse
-            sp[threadIdx.x] = make_float4(x, y, z, fin ? __ldg(lse + i) : CUDART_INF_F);
+            const bool fin = load_point<XF>(pts, b + q, r, x, y, z, nullptr);  // reported by k_flat_lse
+            sp[q] = make_float4(x, y, z, fin ? __ldg(lse + b + q) : CUDART_INF_F);
         }
         __syncthreads();
-        // plain FP32 sums over 16 points, then one compensated fold
-        int q = 0;
-        for (; q + 16 <= cnt; q += 16) {
+        // this warp's points of the stage (a NaN keeps its point)
+        if (group * GROUP >= J) continue;  // no component (after the block barriers: they come first in a stage)
+        // plain FP32 sums over 16 points (a block without a point for this
+        // warp leaves them and the fold unchanged), then one compensated fold
+        const float* gm = gmax ? gmax + group * gstride + b : nullptr;
+        auto group_max = [&](int q) { return gm && q < cnt ? __ldg(gm + q) : CUDART_INF_F; };
+        float g0 = group_max(lane), g1 = group_max(32 + lane);  // loaded two blocks of 32 ahead
+        for (int w = 0; w < cnt; w += 32) {
+            const float gc = g0;
+            g0 = g1;
+            g1 = group_max(w + 64 + lane);
+            const bool mine = w + lane < cnt && !(sp[w + lane].w - gc > SKIP);
+            const unsigned live = __ballot_sync(FULL, mine);
+#pragma unroll 1
+            for (int h = 0; h < 32; h += 16) {
+                unsigned mm = (live >> h) & 0xFFFFu;
+                if (mm == 0) continue;
+                const float4* z = sp + w + h;
+                if (mm == 0xFFFFu) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u) pair(sp[q + u]);
-            fold_mom<NM>(in, s, c);
+                    for (int u = 0; u < 16; ++u) pair(z[u]);
+                } else {
+                    while (mm & (mm - 1)) {  // two at a time
+                        const int p0 = __ffs(mm) - 1;
+                        mm &= mm - 1;
+                        const int p1 = __ffs(mm) - 1;
+                        mm &= mm - 1;
+                        const float4 z0 = z[p0], z1 = z[p1];
+                        pair(z0);
+                        pair(z1);
+                    }
+                    if (mm) pair(z[__ffs(mm) - 1]);
+                }
+                fold_mom<NM>(in, s, c);
+            }
         }
-        for (; q < cnt; ++q) pair(sp[q]);
-        fold_mom<NM>(in, s, c);
     }
     if (own) {
 #pragma unroll
@@ -428,50 +515,62 @@ __global__ void k_flat_reg_init(const double* __restrict__ T_init, double* __res
     }
 }
 
+// Also the round's solve, by the last CTA to finish (as a launch of its own it
+// took 7 us a round).
 __global__ void __launch_bounds__(MOM_THREADS)
 k_flat_terms(const float2* __restrict__ part, int max_ctas, const int* __restrict__ meta,
              const NodeEst* __restrict__ est, const float4* __restrict__ rterm, int n,
-             float2* __restrict__ tpart, double* __restrict__ dbg) {
+             float2* __restrict__ tpart, double* __restrict__ dbg, unsigned* __restrict__ arrived, int it,
+             double* T, float* Rt, double* T_hist, double* obj, int* status) {
     __shared__ float2 red[RED_WARPS][4][RED_COMPS];
+    __shared__ bool last;
     const int J = meta[0];
+    const unsigned ctas = unsigned((J + RED_COMPS - 1) / RED_COMPS);
+    if (J == 0 && blockIdx.x == 0)  // no component: a singular system, T kept
+        sum_terms_and_solve(tpart, 0, it, T, Rt, T_hist, obj, status);
     if (blockIdx.x * RED_COMPS >= J) return;  // uniform over the CTA
     const FlatPlan pl = flat_plan(J, n, max_ctas);
     float S[4], C[4];
     reduce_slices<4>(part, pl, J, red, S, C);
-    if (threadIdx.x >= 32) return;
-    const int lane = threadIdx.x, j = blockIdx.x * RED_COMPS + lane;
-    float v[32], c[32];
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x, j = blockIdx.x * RED_COMPS + lane;
+        float v[32], c[32];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) { v[k] = 0.f; c[k] = 0.f; }
-    if (j < J) {
-        const float4 cm = est[j].a;
-        const float M0 = S[0] + C[0];
-        float o0 = 0.f, o1 = 0.f, o2 = 0.f;
-        if (M0 > 0.f) {
-            const float inv = 1.0f / M0;
-            o0 = (S[1] + C[1]) * inv;
-            o1 = (S[2] + C[2]) * inv;
-            o2 = (S[3] + C[3]) * inv;
-            float w[NTERM];
-            node_terms(rterm[3 * j], rterm[3 * j + 1], rterm[3 * j + 2], cm, M0, o0, o1, o2, M0 / float(n), w);
+        for (int k = 0; k < 32; ++k) { v[k] = 0.f; c[k] = 0.f; }
+        if (j < J) {
+            const float4 cm = est[j].a;
+            const float M0 = S[0] + C[0];
+            float o0 = 0.f, o1 = 0.f, o2 = 0.f;
+            if (M0 > 0.f) {
+                const float inv = 1.0f / M0;
+                o0 = (S[1] + C[1]) * inv;
+                o1 = (S[2] + C[2]) * inv;
+                o2 = (S[3] + C[3]) * inv;
+                float w[NTERM];
+                node_terms(rterm[3 * j], rterm[3 * j + 1], rterm[3 * j + 2], cm, M0, o0, o1, o2, M0 / float(n), w);
 #pragma unroll
-            for (int k = 0; k < NTERM; ++k) pair_add(v[k], c[k], w[k], 0.f);
+                for (int k = 0; k < NTERM; ++k) pair_add(v[k], c[k], w[k], 0.f);
+            }
+            dbg[4 * j + 0] = double(M0);
+            dbg[4 * j + 1] = double(M0) * (double(cm.x) + double(o0));
+            dbg[4 * j + 2] = double(M0) * (double(cm.y) + double(o1));
+            dbg[4 * j + 3] = double(M0) * (double(cm.z) + double(o2));
         }
-        dbg[4 * j + 0] = double(M0);
-        dbg[4 * j + 1] = double(M0) * (double(cm.x) + double(o0));
-        dbg[4 * j + 2] = double(M0) * (double(cm.y) + double(o1));
-        dbg[4 * j + 3] = double(M0) * (double(cm.z) + double(o2));
+        float ws, we;
+        warp_reduce_scatter32(v, c, ws, we);
+        if (lane < NTERM) tpart[NTERM * blockIdx.x + lane] = make_float2(ws, we);
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();
+            last = atomicAdd(arrived, 1u) == ctas - 1;
+            if (last) {
+                *arrived = 0u;  // ready for the next round
+                __threadfence();
+            }
+        }
     }
-    float ws, we;
-    warp_reduce_scatter32(v, c, ws, we);
-    if (lane < NTERM) tpart[NTERM * blockIdx.x + lane] = make_float2(ws, we);
-}
-
-__global__ void __launch_bounds__(MOM_THREADS)
-k_flat_solve(const float2* __restrict__ tpart, const int* __restrict__ meta, int it,
-             double* __restrict__ T, float* __restrict__ Rt, double* __restrict__ T_hist,
-             double* __restrict__ obj, int* __restrict__ status) {
-    sum_terms_and_solve(tpart, (meta[0] + RED_COMPS - 1) / RED_COMPS, it, T, Rt, T_hist, obj, status);
+    __syncthreads();
+    if (last) sum_terms_and_solve(tpart, int(ctas), it, T, Rt, T_hist, obj, status);
 }
 
 __global__ void k_flat_copy_T(const double* __restrict__ T, double* __restrict__ out) {
@@ -578,6 +677,9 @@ struct hgmm_flat {
     int* meta = nullptr;
     double* eps = nullptr;
     float* lse = nullptr;
+    float* gmax = nullptr;  // per group of GROUP components and point: the largest score (or null)
+    int* slot = nullptr;    // from the tree: component of each node
+    double* wt = nullptr;   // ... and its path product; the last: their sum
     float2* part = nullptr;
     float2* tpart = nullptr;
     double* T = nullptr;
@@ -591,7 +693,7 @@ namespace {
 
 void free_flat(hgmm_flat* f) {
     if (!f) return;
-    void* ptrs[] = {f->comp, f->est, f->rterm, f->meta, f->eps, f->lse, f->part, f->tpart,
+    void* ptrs[] = {f->comp, f->est, f->rterm, f->meta, f->eps, f->lse, f->gmax, f->slot, f->wt, f->part, f->tpart,
                     f->T, f->Rt, f->obj, f->dbg, f->status};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -635,9 +737,16 @@ int hgmm_flat_create(int64_t max_points, int32_t max_components, hgmm_flat** out
     f->max_ctas = 4 * (f->n_sm > 0 ? f->n_sm : 1);
     const int tiles_max = (max_components + MOM_THREADS - 1) / MOM_THREADS;
     const size_t part_ctas = size_t(f->max_ctas > tiles_max ? f->max_ctas : tiles_max);
+    // without the group maxima (too large, or no memory for them) every pair is computed
+    const size_t groups = size_t(max_points) * size_t((max_components + GROUP - 1) / GROUP);
+    if (groups > GMAX_KEPT || !falloc(&f->gmax, groups)) {
+        f->gmax = nullptr;
+        cudaGetLastError();
+    }
     const bool good = falloc(&f->comp, max_components) && falloc(&f->est, max_components) &&
                       falloc(&f->rterm, 3 * size_t(max_components)) && falloc(&f->meta, 4) &&
                       falloc(&f->eps, 1) && falloc(&f->lse, size_t(max_points)) &&
+                      falloc(&f->slot, max_components) && falloc(&f->wt, size_t(max_components) + 1) &&
                       falloc(&f->part, part_ctas * MOM_THREADS * NMOM_MAX) &&
                       falloc(&f->tpart, size_t((max_components + RED_COMPS - 1) / RED_COMPS) * NTERM) && falloc(&f->T, 16) && falloc(&f->Rt, 12) &&
                       falloc(&f->obj, 1) && falloc(&f->dbg, 4 * size_t(max_components)) &&
@@ -661,8 +770,10 @@ int hgmm_flat_from_tree(hgmm_flat* f, const hgmm_tree* t, int32_t level, void* s
     const int64_t n_cand = level_offset(L);
     if (n_cand > f->cap_comp) return HGMM_ECAPACITY;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    k_flat_from_tree<<<1, FROM_TREE_THREADS, 0, s>>>(t->stat, t->root, L, int(n_cand), f->comp, f->est,
-                                                    f->rterm, f->meta, f->eps, f->status);
+    k_flat_select<<<1, FROM_TREE_THREADS, 0, s>>>(t->stat, t->root, L, int(n_cand), f->slot, f->wt,
+                                                 f->wt + f->cap_comp, f->meta, f->eps, f->status);
+    k_flat_write<<<int((n_cand + 63) / 64), 64, 0, s>>>(t->stat, int(n_cand), f->slot, f->wt, f->wt + f->cap_comp,
+                                                       f->eps, f->comp, f->est, f->rterm, f->status);
     f->jcap = int(n_cand);
     f->have = true;
     return launched();
@@ -680,9 +791,10 @@ int hgmm_flat_fit(hgmm_flat* f, const float* d_points, int64_t n, int32_t em_ite
     const int mgrid = moment_grid(f);
     const int lse_grid = int((n + LSE_POINTS - 1) / LSE_POINTS);
     for (int it = 0; it < em_iters; ++it) {
-        k_flat_lse<false><<<lse_grid, LSE_THREADS, 0, s>>>(pts, int(n), nullptr, f->est, f->meta, f->lse, f->status);
+        k_flat_lse<false><<<lse_grid, LSE_THREADS, 0, s>>>(pts, int(n), nullptr, f->est, f->meta, f->lse, f->gmax, n,
+                                                           f->status);
         k_flat_moments<10, false><<<mgrid, MOM_THREADS, 0, s>>>(pts, int(n), nullptr, f->lse, f->est, f->meta,
-                                                               mgrid, f->part);
+                                                               mgrid, f->gmax, n, f->part);
         k_flat_mstep<<<rgrid, MOM_THREADS, 0, s>>>(f->part, mgrid, f->meta, int(n), n_min, f->eps, f->comp,
                                                    f->est, f->status);
     }
@@ -701,12 +813,13 @@ int hgmm_flat_register(hgmm_flat* f, const float* d_src, int64_t n, const double
     const int lse_grid = int((n + LSE_POINTS - 1) / LSE_POINTS);
     k_flat_reg_init<<<1, 32, 0, s>>>(d_T_init, f->T, f->Rt, f->obj);
     for (int it = 0; it < iters; ++it) {
-        k_flat_lse<true><<<lse_grid, LSE_THREADS, 0, s>>>(pts, int(n), f->Rt, f->est, f->meta, f->lse, f->status);
+        k_flat_lse<true><<<lse_grid, LSE_THREADS, 0, s>>>(pts, int(n), f->Rt, f->est, f->meta, f->lse, f->gmax, n,
+                                                          f->status);
         k_flat_moments<4, true><<<mgrid, MOM_THREADS, 0, s>>>(pts, int(n), f->Rt, f->lse, f->est, f->meta, mgrid,
-                                                             f->part);
+                                                             f->gmax, n, f->part);
         k_flat_terms<<<rgrid, MOM_THREADS, 0, s>>>(f->part, mgrid, f->meta, f->est, f->rterm, int(n),
-                                                   f->tpart, f->dbg);
-        k_flat_solve<<<1, MOM_THREADS, 0, s>>>(f->tpart, f->meta, it, f->T, f->Rt, d_T_hist, f->obj, f->status);
+                                                   f->tpart, f->dbg, reinterpret_cast<unsigned*>(f->meta + 2), it,
+                                                   f->T, f->Rt, d_T_hist, f->obj, f->status);
     }
     if (d_T_out) k_flat_copy_T<<<1, 32, 0, s>>>(f->T, d_T_out);
     return launched();
