@@ -49,7 +49,7 @@ void free_tree(hgmm_tree* t) {
     void* ptrs[] = {t->est, t->stat, t->seg_start, t->seg_count, t->pts[0], t->pts[1],
                     t->codes, t->items, t->item_range, t->meta, t->partials, t->item_cnt,
                     t->item_off, t->slice_tot, t->root, t->root_part, t->root_counter, t->em_cnt, t->mslices, t->mcnt, t->lv_part, t->lv_slices, t->lv_cnt, t->status, t->reg_acc, t->reg_acc2, t->reg_part,
-                    t->reg_bar, t->reg_T, t->reg_Rt, t->reg_dbg, t->reg_obj, t->rnode, t->trace, t->stage_tgt,
+                    t->reg_bar, t->reg_T, t->reg_Rt, t->reg_dbg, t->reg_obj, t->rnode, t->rblk, t->trace, t->stage_tgt,
                     t->stage_src, t->stage_T};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -175,6 +175,7 @@ int hgmm_tree_create(int64_t max_points, int32_t max_depth, hgmm_tree** out) {
     good &= dalloc(&t->reg_acc2, 6 * t->max_nodes);
     good &= dalloc(&t->reg_part, NTERM * nb);
     good &= dalloc(&t->rnode, 3 * t->max_nodes);
+    good &= dalloc(&t->rblk, t->max_nodes / 8 * REG_BLOCK_F4);
     good &= dalloc(&t->trace, int64_t(TRACE_MAX_ITERS) * std::max(t->reg_grid, t->reg_grid_wide) * 6);
     good &= dalloc(&t->reg_bar, 8);
     good &= dalloc(&t->reg_T, 16);

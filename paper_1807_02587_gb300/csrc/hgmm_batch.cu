@@ -27,6 +27,7 @@ struct BatchWs {
     NodeEst* est;
     NodeStat* stat;
     float4* rnode;
+    float4* rblk;
     int* seg_start;
     int* seg_count;
     RootDev* root;
@@ -85,7 +86,7 @@ struct RegSmem {
 };
 
 // dynamic shared memory of k_batch: the staged top levels of the current
-// pair's tree (3 float4 per node, padded per block of 8 siblings), then the
+// pair's tree (sibling blocks), then the
 // CTA's fixed-point histogram of their registration moments (4 words per node)
 constexpr size_t BATCH_DYN_SMEM =
     STAGED_F4 * sizeof(float4) + 4 * STAGED_NODES * sizeof(unsigned long long);
@@ -233,11 +234,12 @@ __device__ void run_pair(const BatchArgs& a, const BatchWs& w, int cid, int pair
         const int r = threadIdx.x >> 2, c = threadIdx.x & 3;
         if (r < 3) w.Rt[c == 3 ? 9 + r : r * 3 + c] = float(v);
     }
-    {
-        const int ns = n_nodes < STAGED_NODES ? n_nodes : STAGED_NODES;
-        stage_nodes(sm_est, w.est, ns);
-    }
+    // the descent's sibling blocks: all of them in global memory, shared over
+    // the cluster, and the staged levels' in every CTA's shared memory
+    const int n_staged = n_nodes < STAGED_NODES ? n_nodes : STAGED_NODES;
+    for (int g = 32 * (rank * wpb + warp); g < n_nodes; g += 32 * cs * wpb) pack_blocks(w.rblk, w.est, g, n_nodes, n_nodes);
     cl.sync();
+    for (int i = threadIdx.x; i < n_staged / 8 * BLOCK_F4; i += blockDim.x) sm_est[i] = __ldcg(w.rblk + i);
     const double ext = __ldcg(&w.root->extent) > 0.0 ? __ldcg(&w.root->extent) : 1.0;
     const float qscale = float(FIX / ext);
     // large sources: nodes recorded in the first round (the hand-off codes are
@@ -254,13 +256,13 @@ __device__ void run_pair(const BatchArgs& a, const BatchWs& w, int cid, int pair
             sort_source_by_node(src, n_s, n_nodes, w.codes, w.pts[0], rank, cs, cl,
                                 reinterpret_cast<int*>(sm_est));
             src = w.pts[0];
-            stage_nodes(sm_est, w.est, n_nodes < STAGED_NODES ? n_nodes : STAGED_NODES);
+            for (int i = threadIdx.x; i < n_staged / 8 * BLOCK_F4; i += blockDim.x) sm_est[i] = __ldcg(w.rblk + i);
         }
         __syncthreads();
-        descend_points<true>(src, n_s, w.est, sm_est, depth, rgs.Rt, qscale, w.acc, rank, cs, hist,
+        descend_points<true>(src, n_s, w.rblk, sm_est, depth, rgs.Rt, qscale, w.acc, rank, cs, hist,
                              it == 0 && sort_src ? w.codes : nullptr);
         __syncthreads();
-        flush_node_hist(hist, n_nodes < STAGED_NODES ? n_nodes : STAGED_NODES, w.acc);
+        flush_node_hist(hist, n_staged, w.acc);
         cl.sync();
         float v[32], c[32];  // NTERM terms, padded to a warp's width
 #pragma unroll
@@ -476,7 +478,8 @@ int hgmm_batch_create(int64_t max_points, int32_t max_depth, int32_t max_pairs, 
     bool good = true;
     for (int c = 0; c < mc && good; ++c) {
         BatchWs& w = ws[c];
-        good &= balloc(b, &w.est, nodes) && balloc(b, &w.stat, nodes) && balloc(b, &w.rnode, 3 * nodes);
+        good &= balloc(b, &w.est, nodes) && balloc(b, &w.stat, nodes) && balloc(b, &w.rnode, 3 * nodes) &&
+                balloc(b, &w.rblk, nodes / 8 * BLOCK_F4);
         good &= balloc(b, &w.seg_start, nodes) && balloc(b, &w.seg_count, nodes);
         good &= balloc(b, &w.root, 1) && balloc(b, &w.pts[0], max_points) && balloc(b, &w.pts[1], max_points);
         good &= balloc(b, &w.codes, max_points) && balloc(b, &w.item_range, 2 * parents) &&

@@ -1483,45 +1483,92 @@ __device__ __forceinline__ long long to_fix(float v) {
     return __float2ll_rn(c);
 }
 
-// Algorithm 1 for the points of this CTA (grid-stride by warps) with the
-// current transform; adds each point's (gamma, gamma (z' - mu_j)) to the
-// chosen node's fixed-point moments.
+// What the descent reads, by sibling block (8 nodes with one parent, the
+// smallest unit it ever loads): per pair of children ten constants of both
+// (-mu_x, -mu_y, -mu_z, -C, W00, W10, W11, W20, W21, W22: the operands of
+// packed FP32x2 arithmetic) in five float4, then the children's stop flags as
+// a bit mask, and padding.  The shared-memory loads bound the descent of large
+// sources: each 16-byte load returns 512 bytes to a warp, four cycles of the
+// SM's 128-byte path, and node records of three float4 took 24 of them per
+// level (16.8M points: 3,450 warps per SM x 3.5 levels x 24 x 4 cycles = 560 us,
+// measured 567 us per round).  A block is 20 loads and one word.  Its stride of
+// 21 float4 puts the same constant of eight consecutive blocks on different
+// banks.
 constexpr int STAGED_NODES = 584;  // levels 0..2 (8 + 64 + 512 nodes) live in shared memory
-// Staged layout: node g at float4 slot 3 g + g / 8, i.e. one float4 of padding
-// after each block of 8 siblings (100 words), so that the same child of
-// different parents falls on different banks (block b starts at bank 4 b mod
-// 32): the lanes of a warp descending under different parents load without
-// conflicts between up to 8 consecutive parents.
-constexpr int STAGED_F4 = 3 * STAGED_NODES + STAGED_NODES / 8;
+constexpr int BLOCK_F4 = REG_BLOCK_F4;
+constexpr int STAGED_F4 = BLOCK_F4 * STAGED_NODES / 8;
 static_assert(STAGED_NODES % 8 == 0, "whole sibling blocks are staged");
 
-__device__ __forceinline__ int staged_slot(int g) { return 3 * g + (g >> 3); }
+// First float of a child's constants in its block; constant q is 2 q further.
+__device__ __forceinline__ int block_child(int c) { return 20 * (c >> 1) + (c & 1); }
 
-// Copy the first ns nodes (ns <= STAGED_NODES) of est to the staged layout
-// (all threads of the CTA; the caller synchronises).
-__device__ __forceinline__ void stage_nodes(float4* sm_est, const NodeEst* __restrict__ est, int ns) {
-    const float4* g = reinterpret_cast<const float4*>(est);
-    for (int i = threadIdx.x; i < 3 * ns; i += blockDim.x) {
-        const int node = i / 3;
-        sm_est[i + (node >> 3)] = __ldcg(g + i);
+// The blocks of the 32 nodes from `base` on (a multiple of 32; those below n)
+// of a tree of n_nodes nodes, by a warp.  A node's stop flag is set where the
+// descent ends with it: its complexity is at most lambda_c (c.z), or it has
+// children and none of them is live.
+__device__ __forceinline__ void pack_blocks(float4* blocks, const NodeEst* est, int base, int n, int n_nodes) {
+    const int lane = threadIdx.x & 31;
+    const int g = base + lane;
+    const bool in = g < n;
+    const NodeEst* e = est + (in ? g : base);
+    const float4 a = __ldcg(&e->a), b = __ldcg(&e->b), c = __ldcg(&e->c);
+    bool stop = c.z != 0.f;
+    if (8 * int64_t(g) + 16 <= n_nodes) {  // the children of node g are 8 g + 8 ... 8 g + 15
+        const NodeEst* ch = est + 8 * g + 8;
+        float top = -CUDART_INF_F;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) top = fmaxf(top, __ldcg(&ch[k].a.w));
+        stop = stop || !(top > -CUDART_INF_F);
+    }
+    const unsigned stops = __ballot_sync(FULL, in && stop);
+    if (!in) return;
+    float* blk = reinterpret_cast<float*>(blocks + (g >> 3) * BLOCK_F4);
+    float* o = blk + block_child(g & 7);
+    o[0] = -a.x;
+    o[2] = -a.y;
+    o[4] = -a.z;
+    o[6] = -a.w;
+    o[8] = b.x;
+    o[10] = b.y;
+    o[12] = b.z;
+    o[14] = b.w;
+    o[16] = c.x;
+    o[18] = c.y;
+    if ((g & 7) == 0) blk[80] = __uint_as_float((stops >> lane) & 0xFFu);
+}
+
+// Negated log2 scores u = -log2(pi N(z | child)) of a point over the eight
+// children of the block at blk (load(p): a float4), two children per packed
+// operation.
+template <class Load>
+__device__ __forceinline__ void block_scores(const float4* blk, Load load, float x, float y, float z,
+                                             float2 (&u)[4]) {
+    auto lo = [](const float4& v) { return make_float2(v.x, v.y); };
+    auto hi = [](const float4& v) { return make_float2(v.z, v.w); };
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4 q0 = load(blk + 5 * k), q1 = load(blk + 5 * k + 1), q2 = load(blk + 5 * k + 2);
+        const float4 q3 = load(blk + 5 * k + 3), q4 = load(blk + 5 * k + 4);
+        const float2 ex = __fadd2_rn(f2(x), lo(q0)), ey = __fadd2_rn(f2(y), hi(q0)), ez = __fadd2_rn(f2(z), lo(q1));
+        const float2 d0 = __fmul2_rn(lo(q2), ex);
+        const float2 d1 = __ffma2_rn(lo(q3), ey, __fmul2_rn(hi(q2), ex));
+        const float2 d2 = __ffma2_rn(hi(q4), ez, __ffma2_rn(lo(q4), ey, __fmul2_rn(hi(q3), ex)));
+        u[k] = __ffma2_rn(d2, d2, __ffma2_rn(d1, d1, __ffma2_rn(d0, d0, hi(q1))));
     }
 }
 
-// Child c of the sibling block that starts at node `first` (a multiple of 8:
-// level offsets and 8 x parent index are); `staged` = the block lies in the
-// staged levels, and `blk` is its first slot there (staged_slot(first)).
-__device__ __forceinline__ void load_child(const NodeEst* __restrict__ est, const float4* blk, bool staged,
-                                           int64_t first, int c, float4& ea, float4& eb, float4& ec) {
-    if (staged) {
-        ea = blk[3 * c];
-        eb = blk[3 * c + 1];
-        ec = blk[3 * c + 2];
-    } else {
-        const NodeEst* e = est + first + c;
-        ea = __ldg(&e->a);
-        eb = __ldg(&e->b);
-        ec = __ldg(&e->c);
+// The scores below the node whose first child is `first`; returns the stop
+// flags.  Staged levels read shared memory, deeper levels the cache.
+__device__ __forceinline__ unsigned child_scores(const float4* blocks, const float4* sm_blocks, int first, float x,
+                                                 float y, float z, float2 (&u)[4]) {
+    if (first < STAGED_NODES) {
+        const float4* blk = sm_blocks + (first >> 3) * BLOCK_F4;
+        block_scores(blk, [](const float4* p) { return *p; }, x, y, z, u);
+        return __float_as_uint(blk[BLOCK_F4 - 1].x);
     }
+    const float4* blk = blocks + int64_t(first >> 3) * BLOCK_F4;
+    block_scores(blk, [](const float4* p) { return __ldca(p); }, x, y, z, u);
+    return __float_as_uint(__ldca(&blk[BLOCK_F4 - 1].x));
 }
 
 // Sums (v[0..NV)) over the lanes of the warp that hold the same key (all 32
@@ -1558,21 +1605,66 @@ __device__ __forceinline__ int warp_group_sum(int key, V (&v)[NV]) {
     return rank;
 }
 
-// KEYS: key_out (if not null) receives each point's chosen node (all ones:
-// none), for the source reorder between the first and the second round.
+// The words of a node's moments: the CTA's histogram or global memory.
+__device__ __forceinline__ unsigned long long* moment_words(int node, unsigned long long* hist,
+                                                            unsigned long long* acc) {
+    static_assert(ACC_REPLICAS == 1, "one accumulator copy per node");
+    return hist && node < STAGED_NODES ? hist + 4 * node : acc + 4 * int64_t(node);
+}
+
+// The warp's moments (q[0..4) of the node `chosen` per lane, -1: none; |q| <=
+// 2^40) into their nodes' words.
+__device__ __forceinline__ void add_moments(int chosen, long long (&q)[4], unsigned long long* hist,
+                                            unsigned long long* acc) {
+    const int lane = threadIdx.x & 31;
+    const int first = __shfl_sync(FULL, chosen, 0);
+    if (__all_sync(FULL, chosen == first)) {
+        // one group (every point of the warp chose the same node, as most do
+        // once the source is in node order): warp reductions of two biased
+        // limbs per value, q + 2^40 = l0 + 2^21 l1 with l0 < 2^21, l1 <= 2^20,
+        // so the 32-lane sums stay below 2^26: the same exact integer totals
+        // as the group tree; every lane has them, and four lanes add one each
+        if (first < 0) return;
+        long long mine = 0;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const unsigned long long u = (unsigned long long)(q[v] + (1ll << 40));
+            const unsigned s0 = __reduce_add_sync(FULL, unsigned(u) & 0x1FFFFFu);
+            const unsigned s1 = __reduce_add_sync(FULL, unsigned(u >> 21));
+            const long long t = (long long)s0 + ((long long)s1 << 21) - (32ll << 40);
+            if (lane == v) mine = t;
+        }
+        if (lane < 4) atomicAdd(moment_words(first, hist, acc) + lane, (unsigned long long)mine);
+        return;
+    }
+    const int rank = warp_group_sum<4, long long>(chosen, q);
+    if (chosen >= 0 && rank == 0) {
+        unsigned long long* dst = moment_words(chosen, hist, acc);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) atomicAdd(dst + v, (unsigned long long)q[v]);
+    }
+}
+
+// Algorithm 1 for the points of this CTA with the current transform; adds each
+// point's (gamma, gamma (z' - mu_j)) to the chosen node's fixed-point moments.
+// blocks: all sibling blocks in global memory; sm_blocks: those of the staged
+// levels.  KEYS: key_out (if not null) receives each point's chosen node (all
+// ones: none), for the source reorder between the first and the second round.
 // hist (shared memory, 4 x STAGED_NODES fixed-point words, zero on entry, or
 // null): the groups whose node is one of the staged top levels add into the
 // CTA's own histogram instead of global memory; flush_node_hist then moves it
 // to the global accumulators with one atomic per touched word.  The top
 // levels are where most points stop on large planar structures, so this
 // keeps thousands of warps from serialising on a few hot addresses.
-template <bool KEYS = false>
+// Two points per lane that share a block's loads were tried: 16M points in
+// node order 459 us a round against 466, but 11.5 against 9.9 us at 4,000
+// points and 1,195 against 805 for a round in random order.
+template <bool KEYS>
 __device__ __forceinline__ void descend_points(const float4* __restrict__ src, int n,
-                                               const NodeEst* __restrict__ est, const float4* sm_est,
-                                               int depth, const float* Rt_sm, float qscale,
+                                               const float4* __restrict__ blocks, const float4* sm_blocks, int depth,
+                                               const float* Rt_sm, float qscale,
                                                unsigned long long* __restrict__ acc, int cta, int ncta,
-                                               unsigned long long* hist = nullptr,
-                                               uint32_t* __restrict__ key_out = nullptr) {
+                                               unsigned long long* hist, uint32_t* __restrict__ key_out = nullptr) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float r00 = Rt_sm[0], r01 = Rt_sm[1], r02 = Rt_sm[2], r10 = Rt_sm[3], r11 = Rt_sm[4];
     const float r12 = Rt_sm[5], r20 = Rt_sm[6], r21 = Rt_sm[7], r22 = Rt_sm[8];
@@ -1587,101 +1679,84 @@ __device__ __forceinline__ void descend_points(const float4* __restrict__ src, i
         const int base = ch * 32;
         const int i = base + lane;
         const bool valid = i < n;
-        float4 z = valid ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float x = fmaf(r00, z.x, fmaf(r01, z.y, fmaf(r02, z.z, tx)));
-        const float y = fmaf(r10, z.x, fmaf(r11, z.y, fmaf(r12, z.z, ty)));
-        const float w = fmaf(r20, z.x, fmaf(r21, z.y, fmaf(r22, z.z, tz)));
+        const float4 s = valid ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float x = fmaf(r00, s.x, fmaf(r01, s.y, fmaf(r02, s.z, tx)));
+        const float y = fmaf(r10, s.x, fmaf(r11, s.y, fmaf(r12, s.z, ty)));
+        const float z = fmaf(r20, s.x, fmaf(r21, s.y, fmaf(r22, s.z, tz)));
         int chosen = -1;
-        float gamma = 0.f, cmx = 0.f, cmy = 0.f, cmz = 0.f;
-        int local = 0;  // index within its level of the current search node
-        int off = 0;    // first node of the level (32-bit: a depth-5 tree has 37,448 nodes)
-        for (int l = 0; l < depth && valid; ++l) {
-            const int first = off + 8 * local;
-            off = 8 * off + 8;  // the next level's first node
-            float sc8[8];
-            float best = -CUDART_INF_F;
-            int bi = -1;
-            float bstop = 0.f;  // the best child's stop flag (its mean is read once, after the descent)
-            // one child's log2 score from its three records, and the running argmax
-            auto score = [&](int c, const float4 ea, const float4 eb, const float4 ec) {
-                const float ex = x - ea.x, ey = y - ea.y, ez = w - ea.z;
-                const float d0 = eb.x * ex;
-                const float d1 = fmaf(eb.z, ey, eb.y * ex);
-                const float d2 = fmaf(ec.y, ez, fmaf(ec.x, ey, eb.w * ex));
-                float sc = fmaf(-d0, d0, ea.w);
-                sc = fmaf(-d1, d1, sc);
-                sc = fmaf(-d2, d2, sc);
-                sc8[c] = sc;
-                if (sc > best) {
-                    best = sc;
-                    bi = c;
-                    bstop = ec.z;
-                }
-            };
-            // the staged levels (the same level for every lane still
-            // descending) read shared memory, deeper levels the cache
-            if (first < STAGED_NODES) {
-                const float4* blk = sm_est + staged_slot(first);
+        int first = 0;  // the current search node's first child
+        float2 u[4];
+        float best = 0.f;
+        int left = valid ? depth : 0;  // levels left
+        while (left > 0) {
+            const unsigned stops = child_scores(blocks, sm_blocks, first, x, y, z, u);
+            // the best child, by a tournament (a chain of eight compares and
+            // selects was 5 % of a round): the lowest index among equals
+            float m[4];
+            int w[4];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) score(c, blk[3 * c], blk[3 * c + 1], blk[3 * c + 2]);
-            } else {
-                const NodeEst* e = est + first;
-#pragma unroll
-                for (int c = 0; c < 8; ++c) score(c, __ldg(&e[c].a), __ldg(&e[c].b), __ldg(&e[c].c));
+            for (int k = 0; k < 4; ++k) {
+                m[k] = fminf(u[k].x, u[k].y);
+                w[k] = 2 * k + (u[k].x == m[k] ? 0 : 1);
             }
-            if (bi < 0) break;  // the current node has no live children
+            const float m01 = fminf(m[0], m[1]), m23 = fminf(m[2], m[3]);
+            const int w01 = m[0] == m01 ? w[0] : w[1], w23 = m[2] == m23 ? w[2] : w[3];
+            best = fminf(m01, m23);
+            const int bi = m01 == best ? w01 : w23;
+            if (!(best < CUDART_INF_F)) {
+                // no child has a finite score (a point so far away that every
+                // square overflows, or a root without live nodes): the descent
+                // ended with the node above, whose block is scored once more
+                if (chosen < 0) break;
+                first = chosen & ~7;
+                left = 1;
+                continue;
+            }
+            chosen = first + bi;
+            first = 8 * chosen + 8;
+            if ((stops >> bi) & 1u) break;  // Complexity <= lambda_c, or no live children
+            --left;
+        }
+        // the posterior of the chosen child among its siblings: once, after
+        // the descent (inside the loop its exponentials were on every level's
+        // critical path)
+        float gamma = 0.f;
+        if (chosen >= 0) {
             float sum = 0.f;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) sum += ex2_fast(sc8[c] - best);
+            for (int k = 0; k < 4; ++k) {
+                const float2 d = sub2(f2(best), u[k]);
+                sum += ex2_fast(d.x);
+                sum += ex2_fast(d.y);
+            }
             gamma = rcp_fast(sum);
-            chosen = first + bi;
-            local = 8 * local + bi;
-            if (bstop != 0.f) break;  // Complexity <= lambda_c
         }
-        const bool has = chosen >= 0;
-        if (has) {
-            const float4 cm = chosen < STAGED_NODES ? sm_est[staged_slot(chosen)] : __ldg(&est[chosen].a);
-            cmx = cm.x; cmy = cm.y; cmz = cm.z;
-        }
-        if (KEYS && key_out && valid) key_out[i] = has ? uint32_t(chosen) : 0xFFFFFFFFu;  // the point's node
         // each point's moments as fixed-point integers before any sum: the
         // per-warp group sums and the node totals are then exact integer
         // sums, independent of the order of the points
+        const bool has = chosen >= 0;
+        if (KEYS && key_out && valid) key_out[i] = has ? uint32_t(chosen) : 0xFFFFFFFFu;
         long long q[4] = {0, 0, 0, 0};
         if (has) {
-            q[0] = to_fix(gamma * 4294967296.0f);
-            q[1] = to_fix(gamma * (x - cmx) * qscale);
-            q[2] = to_fix(gamma * (y - cmy) * qscale);
-            q[3] = to_fix(gamma * (w - cmz) * qscale);
-        }
-        int rank;
-        if (__all_sync(FULL, chosen == __shfl_sync(FULL, chosen, 0))) {
-            // one group (every point of the warp chose the same node, as
-            // most do once the source is in node order): warp reductions of
-            // two biased limbs per value, q + 2^40 = l0 + 2^21 l1 with
-            // l0 < 2^21, l1 <= 2^20, so the 32-lane sums stay below 2^26:
-            // the same exact integer totals as the group tree
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const unsigned long long u = (unsigned long long)(q[v] + (1ll << 40));
-                const unsigned s0 = __reduce_add_sync(FULL, unsigned(u) & 0x1FFFFFu);
-                const unsigned s1 = __reduce_add_sync(FULL, unsigned(u >> 21));
-                q[v] = (long long)s0 + ((long long)s1 << 21) - (32ll << 40);
+            const int o = (chosen >> 3) * (4 * BLOCK_F4) + block_child(chosen & 7);
+            float mx, my, mz;  // the node's negated mean
+            if (chosen < STAGED_NODES) {
+                const float* m = reinterpret_cast<const float*>(sm_blocks) + o;
+                mx = m[0];
+                my = m[2];
+                mz = m[4];
+            } else {
+                const float* m = reinterpret_cast<const float*>(blocks) + o;
+                mx = __ldca(m);
+                my = __ldca(m + 2);
+                mz = __ldca(m + 4);
             }
-            rank = lane;
-        } else {
-            rank = warp_group_sum<4, long long>(chosen, q);
+            q[0] = to_fix(gamma * 4294967296.0f);
+            q[1] = to_fix(gamma * (x + mx) * qscale);
+            q[2] = to_fix(gamma * (y + my) * qscale);
+            q[3] = to_fix(gamma * (z + mz) * qscale);
         }
-        if (has && rank == 0) {
-            unsigned long long* dst =
-                (hist && chosen < STAGED_NODES)
-                    ? hist + 4 * chosen
-                    : acc + 4 * (int64_t(chosen) * ACC_REPLICAS + (cta & (ACC_REPLICAS - 1)));
-            atomicAdd(dst + 0, (unsigned long long)q[0]);
-            atomicAdd(dst + 1, (unsigned long long)q[1]);
-            atomicAdd(dst + 2, (unsigned long long)q[2]);
-            atomicAdd(dst + 3, (unsigned long long)q[3]);
-        }
+        add_moments(chosen, q, hist, acc);
     }
 }
 
@@ -1690,7 +1765,6 @@ __device__ __forceinline__ void descend_points(const float4* __restrict__ src, i
 // __syncthreads that follows descend_points.
 __device__ __forceinline__ void flush_node_hist(unsigned long long* hist, int n_staged,
                                                 unsigned long long* __restrict__ acc) {
-    static_assert(ACC_REPLICAS == 1, "one accumulator copy per node");
     for (int i = threadIdx.x; i < 4 * n_staged; i += blockDim.x) {
         const unsigned long long v = hist[i];
         if (v) {

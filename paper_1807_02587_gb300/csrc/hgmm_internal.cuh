@@ -42,6 +42,7 @@ constexpr int REG_THREADS = 256;      // registration descent CTA
 constexpr int MSTEP_THREADS = 128;    // registration M-step CTA
 constexpr int NTERM = 28;             // per-round sums: 21 of H, 6 of g, the objective
 constexpr int TRACE_MAX_ITERS = 64;   // rounds the registration trace can hold
+constexpr int REG_BLOCK_F4 = 21;      // float4 per sibling block of the registration descent
 constexpr int ACC_REPLICAS = 1;       // copies of each node's registration moments
 constexpr int MSTEP_SLICES = 8;        // run slices per parent in the level-wide M-step
 constexpr int MSTEP_SLICED_PARENTS = 64;  // levels with at most this many parents are sliced
@@ -185,6 +186,7 @@ struct hgmm_tree {
     unsigned long long* reg_acc2 = nullptr; // nodes x 6 fixed-point second moments (full Eq. 7)
     float2* reg_part = nullptr;             // blocks x 27 (sum, compensation)
     float4* rnode = nullptr;                // nodes x 3: P (6), mu - mu32 (3), FP32
+    float4* rblk = nullptr;                 // sibling blocks of the descent (pack_blocks)
     unsigned* reg_bar = nullptr;            // grid barrier words (8)
     double* reg_T = nullptr;                // 16 doubles current T
     float* reg_Rt = nullptr;                // 12 floats (R row-major, t)

@@ -29,7 +29,7 @@ namespace hgmm {
 namespace {
 
 __global__ void k_reg_init(const double* __restrict__ T_init, int n_nodes, float lam_c,
-                           const NodeStat* __restrict__ stat, NodeEst* __restrict__ est,
+                           const NodeStat* __restrict__ stat, NodeEst* est, float4* __restrict__ blocks,
                            unsigned long long* __restrict__ acc, double* __restrict__ T,
                            float* __restrict__ Rt, unsigned* __restrict__ bar,
                            double* __restrict__ obj) {
@@ -39,6 +39,10 @@ __global__ void k_reg_init(const double* __restrict__ T_init, int n_nodes, float
         if (lam_c >= 0.f)
             est[i].c.z = (stat[i].live && stat[i].complexity <= double(lam_c)) ? 1.f : 0.f;
     }
+    // the descent's sibling blocks, from the records just written by this warp
+    __syncwarp();
+    const int w0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31;
+    if (w0 < n_nodes) pack_blocks(blocks, est, w0, n_nodes, n_nodes);
     if (i == 0) {
         for (int k = 0; k < 16; ++k) T[k] = T_init ? T_init[k] : ((k % 5 == 0) ? 1.0 : 0.0);
         for (int r = 0; r < 3; ++r) {
@@ -55,6 +59,7 @@ struct RegArgs {
     const float4* src;
     int n;
     const NodeEst* est;
+    const float4* blocks;  // sibling blocks (pack_blocks)
     const float4* rnode;
     const RootDev* root;
     int depth;
@@ -122,7 +127,7 @@ __global__ void __launch_bounds__(REG_THREADS, MINB) k_register(RegArgs a) {
     __shared__ float2 sm[REG_THREADS / 32][NTERM];
     __shared__ float2 fin[8][NTERM];
     __shared__ double tot[NTERM];
-    // dynamic: the staged top levels (3 float4 per node, padded), then the CTA's
+    // dynamic: the staged top levels' sibling blocks, then the CTA's
     // fixed-point histogram of their moments (4 words per node)
     extern __shared__ float4 reg_dyn[];
     float4* sm_est = reg_dyn;
@@ -135,7 +140,7 @@ __global__ void __launch_bounds__(REG_THREADS, MINB) k_register(RegArgs a) {
     // for all rounds (the stop flags were set by k_reg_init before launch);
     // the starting pose (k_reg_init) into shared memory
     {
-        stage_nodes(sm_est, a.est, ns);
+        for (int i = threadIdx.x; i < ns / 8 * BLOCK_F4; i += blockDim.x) sm_est[i] = __ldcg(a.blocks + i);
         for (int i = threadIdx.x; i < 4 * STAGED_NODES; i += blockDim.x) hist[i] = 0ull;
         if (threadIdx.x < 12) {
             T_sm[threadIdx.x] = __ldcg(a.T + threadIdx.x);
@@ -147,7 +152,7 @@ __global__ void __launch_bounds__(REG_THREADS, MINB) k_register(RegArgs a) {
     const float qscale = float(FIX / ext);  // fixed-point units per metre
     for (int it = 0; it < a.iters; ++it) {
         trace_mark(a.trace, it, 0);
-        descend_points<KEYS>(a.src, a.n, a.est, sm_est, a.depth, Rt_sm, qscale, a.acc, blockIdx.x, gridDim.x,
+        descend_points<KEYS>(a.src, a.n, a.blocks, sm_est, a.depth, Rt_sm, qscale, a.acc, blockIdx.x, gridDim.x,
                              hist, a.keys);
         __syncthreads();
         flush_node_hist(hist, ns, a.acc);
@@ -718,7 +723,7 @@ int hgmm_register_impl(hgmm_tree* t, const float4* src, int64_t n64, const doubl
         // lam_c < 0: the build's threshold (set here too, so that an earlier
         // call with another threshold does not leave its stop flags behind)
         if (lam_c < 0.f) lam_c = t->prm.lam_c;
-        k_reg_init<<<(n_nodes + 255) / 256, 256, 0, s>>>(T_init, n_nodes, lam_c, t->stat, t->est,
+        k_reg_init<<<(n_nodes + 255) / 256, 256, 0, s>>>(T_init, n_nodes, lam_c, t->stat, t->est, t->rblk,
                                                           t->reg_acc, t->reg_T, t->reg_Rt,
                                                           t->reg_bar, t->reg_obj);
     }
@@ -737,6 +742,7 @@ int hgmm_register_impl(hgmm_tree* t, const float4* src, int64_t n64, const doubl
         a.src = pts;
         a.n = n;
         a.est = t->est;
+        a.blocks = t->rblk;
         a.rnode = t->rnode;
         a.root = t->root;
         a.depth = t->depth;
@@ -782,7 +788,7 @@ int hgmm_register_impl(hgmm_tree* t, const float4* src, int64_t n64, const doubl
             k_src_scatter<<<reorder_ctas, REORDER_THREADS, 0, s>>>(src, n, t->codes, cnt, tot, sorted);
             src = sorted;
             // the remaining rounds start from the pose after round 1
-            k_reg_init<<<(n_nodes + 255) / 256, 256, 0, s>>>(t->reg_T, n_nodes, lam_c, t->stat, t->est,
+            k_reg_init<<<(n_nodes + 255) / 256, 256, 0, s>>>(t->reg_T, n_nodes, lam_c, t->stat, t->est, t->rblk,
                                                               t->reg_acc, t->reg_T, t->reg_Rt,
                                                               t->reg_bar, t->reg_obj);
         }
@@ -808,7 +814,7 @@ int hgmm_register_descent_impl(hgmm_tree* t, const float4* src, int64_t n64, con
     const int n = int(n64);
     const int n_nodes = int(hgmm_node_count(t->depth));
     const float lam_c = d.lam_c >= 0.f ? d.lam_c : t->prm.lam_c;
-    k_reg_init<<<(n_nodes + 255) / 256, 256, 0, s>>>(T_init, n_nodes, lam_c, t->stat, t->est, t->reg_acc,
+    k_reg_init<<<(n_nodes + 255) / 256, 256, 0, s>>>(T_init, n_nodes, lam_c, t->stat, t->est, t->rblk, t->reg_acc,
                                                       t->reg_T, t->reg_Rt, t->reg_bar, t->reg_obj);
     const int tgrid = (n_nodes + VAR_THREADS - 1) / VAR_THREADS;
     const int dgrid = std::max(1, std::min(4 * t->n_sm, (n + VAR_THREADS - 1) / VAR_THREADS));
