@@ -964,9 +964,8 @@ def profile_register_main(args):
     """Registration of a large cloud for an external profiler: the N-point
     plane/box/sphere cloud moved by the large-build section's motion (2
     degrees, 1 % of the extent), registered to its depth-4 tree 3 times with
-    10 rounds.  A source of 2^20 points or more takes two k_register launches
-    per call (the one-round launch that records the nodes, then the other
-    nine rounds on the reordered source)."""
+    10 rounds.  A source of 2^20 points or more is put into spatial order by
+    four launches before the k_register launch."""
     import torch
     from paper_1807_02587_gb300 import binding as B
     from paper_1807_02587_gb300 import synth

@@ -34,8 +34,8 @@
  *   - No entry point except hgmm_tree_create / hgmm_tree_destroy allocates or
  *     frees device memory (hgmm_register_pair_host creates the CUDA stream and
  *     graph it replays), so build + register can be captured in a CUDA graph
- *     (the registration is one cooperative launch; two, around an on-device
- *     reorder, for sources of 2^20 points or more).
+ *     (the registration is one cooperative launch, after an on-device reorder
+ *     for sources of 2^20 points or more).
  *   - Device-side waits are bounded: the registration's arrival and partial-
  *     count waits give up after about a second, record HGMM_ETIMEOUT and
  *     return.

@@ -162,6 +162,8 @@ int hgmm_tree_create(int64_t max_points, int32_t max_depth, hgmm_tree** out) {
     good &= dalloc(&t->mcnt, MSTEP_SLICED_PARENTS);
     // the one-launch build takes clouds of up to a few hundred thousand
     // points, also in a tree made for more
+    t->refine_ok = hgmm_reorder_smem_attr();
+    if (!t->refine_ok) cudaGetLastError();  // large sources then keep their order
     t->levels_ok = levels_smem_attr();
     if (!t->levels_ok) cudaGetLastError();  // the level-wide launches then build every cloud
     if (t->levels_ok) {

@@ -259,8 +259,8 @@ __device__ void run_pair(const BatchArgs& a, const BatchWs& w, int cid, int pair
             for (int i = threadIdx.x; i < n_staged / 8 * BLOCK_F4; i += blockDim.x) sm_est[i] = __ldcg(w.rblk + i);
         }
         __syncthreads();
-        descend_points<true>(src, n_s, w.rblk, sm_est, depth, rgs.Rt, qscale, w.acc, rank, cs, hist,
-                             it == 0 && sort_src ? w.codes : nullptr);
+        descend_points(src, n_s, w.rblk, sm_est, depth, rgs.Rt, qscale, w.acc, rank, cs, hist,
+                       it == 0 && sort_src ? w.codes : nullptr);
         __syncthreads();
         flush_node_hist(hist, n_staged, w.acc);
         cl.sync();

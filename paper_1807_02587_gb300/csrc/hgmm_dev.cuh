@@ -1648,8 +1648,8 @@ __device__ __forceinline__ void add_moments(int chosen, long long (&q)[4], unsig
 // Algorithm 1 for the points of this CTA with the current transform; adds each
 // point's (gamma, gamma (z' - mu_j)) to the chosen node's fixed-point moments.
 // blocks: all sibling blocks in global memory; sm_blocks: those of the staged
-// levels.  KEYS: key_out (if not null) receives each point's chosen node (all
-// ones: none), for the source reorder between the first and the second round.
+// levels.  key_out (if not null) receives each point's chosen node (all ones:
+// none), for the batch's source reorder after its first round.
 // hist (shared memory, 4 x STAGED_NODES fixed-point words, zero on entry, or
 // null): the groups whose node is one of the staged top levels add into the
 // CTA's own histogram instead of global memory; flush_node_hist then moves it
@@ -1659,7 +1659,6 @@ __device__ __forceinline__ void add_moments(int chosen, long long (&q)[4], unsig
 // Two points per lane that share a block's loads were tried: 16M points in
 // node order 459 us a round against 466, but 11.5 against 9.9 us at 4,000
 // points and 1,195 against 805 for a round in random order.
-template <bool KEYS>
 __device__ __forceinline__ void descend_points(const float4* __restrict__ src, int n,
                                                const float4* __restrict__ blocks, const float4* sm_blocks, int depth,
                                                const float* Rt_sm, float qscale,
@@ -1735,7 +1734,7 @@ __device__ __forceinline__ void descend_points(const float4* __restrict__ src, i
         // per-warp group sums and the node totals are then exact integer
         // sums, independent of the order of the points
         const bool has = chosen >= 0;
-        if (KEYS && key_out && valid) key_out[i] = has ? uint32_t(chosen) : 0xFFFFFFFFu;
+        if (key_out && valid) key_out[i] = has ? uint32_t(chosen) : 0xFFFFFFFFu;
         long long q[4] = {0, 0, 0, 0};
         if (has) {
             const int o = (chosen >> 3) * (4 * BLOCK_F4) + block_child(chosen & 7);

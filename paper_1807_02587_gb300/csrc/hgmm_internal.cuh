@@ -146,6 +146,7 @@ struct hgmm_tree {
     int em_coop_grid = 0;  // co-resident CTAs of the cooperative per-level EM kernel (0: unavailable)
     bool levels_ok = false;  // the one-launch build of the levels fits on the device
     int reg_grid = 0;       // CTAs of the registration kernel, two per SM
+    bool refine_ok = false;  // the source reorder's shared memory fits on the device
     int reg_grid_wide = 0;  // three per SM, for large sources (0: not co-resident)
     // last build
     int64_t n = 0;
@@ -242,6 +243,7 @@ int hgmm_register_descent_impl(hgmm_tree* t, const float4* src, int64_t n, const
 int hgmm_export_labels_impl(hgmm_tree* t, int level, int* d_out, cudaStream_t s);
 int hgmm_debug_posteriors_impl(hgmm_tree* t, int level, float* h_gamma);
 int hgmm_register_grid(int n_sm, int per_sm);
+bool hgmm_reorder_smem_attr();
 int hgmm_em_coop_grid(int n_sm, int est_grid);
 bool hgmm_estep_smem_attr();
 int hgmm_barrier_timeout_probe_impl(hgmm_tree* t, long long limit, cudaStream_t s);

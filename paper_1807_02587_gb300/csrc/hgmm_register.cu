@@ -75,7 +75,6 @@ struct RegArgs {
     double* dbg;
     int* status;
     unsigned long long* trace;  // optional: [iter][cta][TRACE_EVENTS] globaltimer ns
-    uint32_t* keys;             // k_register<true>: each point's chosen node (one-round launches)
 };
 
 constexpr int TRACE_EVENTS = 6;
@@ -120,7 +119,7 @@ __device__ __forceinline__ void trace_mark(unsigned long long* tr, int it, int e
 // latency chain and the node terms and the solve want the registers; three
 // (80) for large sources, whose descent is throughput-bound and gains from
 // the extra warps (a few bytes of spills, outside the descent).
-template <bool KEYS, int MINB>
+template <int MINB>
 __global__ void __launch_bounds__(REG_THREADS, MINB) k_register(RegArgs a) {
     __shared__ float Rt_sm[12];
     __shared__ double T_sm[12];
@@ -152,8 +151,7 @@ __global__ void __launch_bounds__(REG_THREADS, MINB) k_register(RegArgs a) {
     const float qscale = float(FIX / ext);  // fixed-point units per metre
     for (int it = 0; it < a.iters; ++it) {
         trace_mark(a.trace, it, 0);
-        descend_points<KEYS>(a.src, a.n, a.blocks, sm_est, a.depth, Rt_sm, qscale, a.acc, blockIdx.x, gridDim.x,
-                             hist, a.keys);
+        descend_points(a.src, a.n, a.blocks, sm_est, a.depth, Rt_sm, qscale, a.acc, blockIdx.x, gridDim.x, hist);
         __syncthreads();
         flush_node_hist(hist, ns, a.acc);
         __syncthreads();
@@ -297,16 +295,35 @@ __global__ void k_barrier_timeout_probe(unsigned* bar, int* status, long long li
 // ------------------------------------------------ source reorder (large clouds)
 // A large source cloud in arbitrary order sends each warp's 32 points down
 // ~20 different paths of the tree, so the descent adds its moments with one
-// atomic group per node and warp and its child loads diverge.  Such a cloud
-// runs its first round in the caller's order, with every point's chosen node
-// recorded; it is then counting-sorted by that node (into a library buffer)
-// and runs the remaining rounds in that order, where the 32 points of a warp
-// mostly follow one path.  The node moments are exact integer sums of the
-// points' fixed-point moments, so the order of the points does not change
-// the result at all.
+// atomic group per node and warp and its child loads diverge.  Such a cloud is
+// first put into spatial order (in a library buffer): a counting sort by grid
+// cell at the starting pose, then, per 2,048 consecutive points, one by their
+// place within the cell.  Neighbours stay neighbours under every pose, so the
+// 32 points of a warp follow nearly one path in all rounds; the node moments
+// are exact integer sums of the points' fixed-point moments, so the order does
+// not change the result at all.  (Ordering by the node that each point chose
+// in a first round in the caller's order goes stale as the pose moves and
+// pays that round in full: 16M points, 10 rounds, 1,600 us for the first two
+// rounds and the sort, then 466 us a round; from the converged pose 368.)
+// The grid's cells have a sixteenth of the target's extent and repeat every
+// extent, so no point is outside it.  16.8M points: 328 us, of which the
+// counts take 52, the scatter 159 and the refinement 111 (1.3 GB to move at
+// least: 200 us).
+//
+// The line: 10 rounds with and without the sort take, in random order, 257 /
+// 286 us at 300k points, 356 / 493 at 600k, 481 / 666 at 1.1M, 4,429 / 7,919
+// at 16M; already in spatial order 256 / 225, 350 / 305, 467 / 428, 4,085 /
+// 3,747.  Smaller sources are mostly single sweeps or frames in the sensor's
+// order, which would pay 15 % for nothing; larger ones are accumulated or
+// sampled, which gain more than an ordered one loses.
 constexpr int REORDER_MIN_POINTS = 1 << 20;
-constexpr int REORDER_KEYS = 8192;  // node ids of trees up to depth 4 (4,680 nodes); the last: no node
-constexpr int REORDER_THREADS = 256;
+constexpr int REORDER_KEYS = 4096;  // 16 x 16 x 16 cells
+constexpr int REORDER_THREADS = 1024;
+constexpr int REORDER_MAX_CTAS = 512;  // k_src_colscan: 32 groups of up to 16 rows
+constexpr int REFINE_BITS = 11;
+constexpr int REFINE_TILE = 1 << REFINE_BITS;
+constexpr int REFINE_THREADS = 256;
+constexpr size_t REFINE_SMEM = REFINE_TILE * (sizeof(float4) + sizeof(int));
 
 // Contiguous range of points of CTA b (of nb).
 __device__ __forceinline__ void cta_range(int n, int b, int nb, int& lo, int& hi) {
@@ -314,78 +331,206 @@ __device__ __forceinline__ void cta_range(int n, int b, int nb, int& lo, int& hi
     hi = int((int64_t(b + 1) * n) / nb);
 }
 
-// Pass 1: each CTA's key counts (cnt[b][key]) over its contiguous range.
-__global__ void __launch_bounds__(REORDER_THREADS) k_src_count(const uint32_t* __restrict__ keys, int n,
+// Bits 0..7 of x to every third bit.
+__device__ __forceinline__ unsigned spread3(unsigned x) {
+    x = (x | x << 8) & 0x0300F00Fu;
+    x = (x | x << 4) & 0x030C30C3u;
+    return (x | x << 2) & 0x09249249u;
+}
+
+// A point's place on the grid at pose Rt: the cell (upper 12 bits) and the
+// place within it (lower 12 bits), both along a Morton curve.  scale: 256 / extent.
+__device__ __forceinline__ unsigned src_cell(const float4 s, const float* Rt, float scale) {
+    const float x = fmaf(Rt[0], s.x, fmaf(Rt[1], s.y, fmaf(Rt[2], s.z, Rt[9])));
+    const float y = fmaf(Rt[3], s.x, fmaf(Rt[4], s.y, fmaf(Rt[5], s.z, Rt[10])));
+    const float z = fmaf(Rt[6], s.x, fmaf(Rt[7], s.y, fmaf(Rt[8], s.z, Rt[11])));
+    return spread3(unsigned(__float2int_rd(x * scale)) & 255u) | spread3(unsigned(__float2int_rd(y * scale)) & 255u) << 1 |
+           spread3(unsigned(__float2int_rd(z * scale)) & 255u) << 2;
+}
+
+__device__ __forceinline__ float cell_scale(const RootDev* root) {
+    return 256.f / float(root->extent > 0.0 ? root->extent : 1.0);
+}
+
+// Pass 1: each CTA's cell counts (cnt[b][cell]) over its contiguous range.
+__global__ void __launch_bounds__(REORDER_THREADS) k_src_count(const float4* __restrict__ src, int n,
+                                                               const float* __restrict__ Rt_g,
+                                                               const RootDev* __restrict__ root,
                                                                int* __restrict__ cnt) {
     __shared__ int h[REORDER_KEYS];
+    __shared__ float Rt[12];
     for (int k = threadIdx.x; k < REORDER_KEYS; k += blockDim.x) h[k] = 0;
+    if (threadIdx.x < 12) Rt[threadIdx.x] = Rt_g[threadIdx.x];
     __syncthreads();
+    const float scale = cell_scale(root);
     int lo, hi;
     cta_range(n, blockIdx.x, gridDim.x, lo, hi);
-    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) atomicAdd(&h[keys[i] & (REORDER_KEYS - 1)], 1);
+    for (int i = lo + threadIdx.x; i < hi; i += 4 * blockDim.x) {
+        float4 p[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (i + j * int(blockDim.x) < hi) p[j] = src[i + j * blockDim.x];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (i + j * int(blockDim.x) < hi) atomicAdd(&h[src_cell(p[j], Rt, scale) >> 12], 1);
+    }
     __syncthreads();
     for (int k = threadIdx.x; k < REORDER_KEYS; k += blockDim.x) cnt[int64_t(blockIdx.x) * REORDER_KEYS + k] = h[k];
 }
 
-// Pass 2a (one thread per key): cnt[b][key] becomes the exclusive prefix
-// over the CTAs b of that key's counts, and tot[key] the key's total.
-__global__ void k_src_colscan(int* __restrict__ cnt, int nb, int* __restrict__ tot) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= REORDER_KEYS) return;
-    int s = 0;
-    for (int b = 0; b < nb; ++b) {
-        const int c = cnt[int64_t(b) * REORDER_KEYS + k];
-        cnt[int64_t(b) * REORDER_KEYS + k] = s;
-        s += c;
-    }
-    tot[k] = s;
-}
-
-// Pass 2b (one CTA of 1024 threads): tot[key] becomes the exclusive prefix
-// over the keys (keys in order, CTAs in order within a key).
-__global__ void __launch_bounds__(1024) k_src_keyscan(int* __restrict__ tot) {
-    constexpr int PER = REORDER_KEYS / 1024;
-    __shared__ int part[1024];
-    int v[PER], s = 0;
+// Pass 2a (32 cells per CTA, 32 groups of rows): cnt[b][cell] becomes the
+// exclusive prefix over the CTAs b of that cell's counts, and tot[cell] the
+// cell's total.  A group's rows are loaded together: one thread per cell that
+// walked all 304 rows took most of the sort's time in load latency.
+__global__ void __launch_bounds__(1024) k_src_colscan(int* __restrict__ cnt, int nb, int* __restrict__ tot) {
+    __shared__ int sum[32][32];
+    constexpr int ROWS = REORDER_MAX_CTAS / 32;
+    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    const int k = blockIdx.x * 32 + lane;
+    const int per = (nb + 31) / 32;  // <= ROWS
+    int v[ROWS], s = 0;
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        v[j] = tot[threadIdx.x * PER + j];
-        s += v[j];
+    for (int j = 0; j < ROWS; ++j) {
+        const int b = grp * per + j;
+        v[j] = j < per && b < nb ? cnt[int64_t(b) * REORDER_KEYS + k] : 0;
     }
-    part[threadIdx.x] = s;
+#pragma unroll
+    for (int j = 0; j < ROWS; ++j) s += v[j];
+    sum[grp][lane] = s;
     __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const int u = threadIdx.x >= off ? part[threadIdx.x - off] : 0;
-        __syncthreads();
-        part[threadIdx.x] += u;
-        __syncthreads();
+    int base = 0, all = 0;
+#pragma unroll 8
+    for (int q = 0; q < 32; ++q) {
+        const int t = sum[q][lane];
+        if (q < grp) base += t;
+        all += t;
     }
-    int base = part[threadIdx.x] - s;
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        tot[threadIdx.x * PER + j] = base;
+    for (int j = 0; j < ROWS; ++j) {
+        const int b = grp * per + j;
+        if (j < per && b < nb) cnt[int64_t(b) * REORDER_KEYS + k] = base;
         base += v[j];
     }
+    if (grp == 0) tot[k] = all;
 }
 
-// Pass 3: every point to its key's next slot of its CTA (shared-memory
-// counters: the order within a CTA's key is not fixed, which the exact
+// Exclusive prefix over v[0..N) in shared memory (16-byte aligned), by the whole CTA (T threads,
+// wsum: T / 32 ints of shared memory); ends with __syncthreads().
+template <int N, int T>
+__device__ __forceinline__ void cta_exclusive_scan(int* v, int* wsum) {
+    static_assert(N % T == 0 && T % 32 == 0 && T <= 1024, "whole runs, one warp of warp totals");
+    constexpr int PER = N / T;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    static_assert(PER % 4 == 0, "runs of int4");
+    int4* run = reinterpret_cast<int4*>(v) + threadIdx.x * (PER / 4);
+    int4 x[PER / 4];
+    int s = 0;
+#pragma unroll
+    for (int j = 0; j < PER / 4; ++j) {
+        x[j] = run[j];
+        s += x[j].x + x[j].y + x[j].z + x[j].w;
+    }
+    int inc = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(FULL, inc, o);
+        if (lane >= o) inc += u;
+    }
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    int base = inc - s;
+    for (int q = 0; q < warp; ++q) base += wsum[q];
+#pragma unroll
+    for (int j = 0; j < PER / 4; ++j) {
+        const int b1 = base + x[j].x, b2 = b1 + x[j].y, b3 = b2 + x[j].z;
+        run[j] = make_int4(base, b1, b2, b3);
+        base = b3 + x[j].w;
+    }
+    __syncthreads();
+}
+
+// Pass 2b: every point to its cell's next slot of its CTA (shared-memory
+// counters: the order within a CTA's cell is not fixed, which the exact
 // fixed-point moments of the descent do not see).
 __global__ void __launch_bounds__(REORDER_THREADS) k_src_scatter(const float4* __restrict__ src, int n,
-                                                                 const uint32_t* __restrict__ keys,
+                                                                 const float* __restrict__ Rt_g,
+                                                                 const RootDev* __restrict__ root,
                                                                  const int* __restrict__ cnt,
-                                                                 const int* __restrict__ base,
+                                                                 const int* __restrict__ tot,
                                                                  float4* __restrict__ dst) {
-    __shared__ int pos[REORDER_KEYS];
-    for (int k = threadIdx.x; k < REORDER_KEYS; k += blockDim.x)
-        pos[k] = base[k] + cnt[int64_t(blockIdx.x) * REORDER_KEYS + k];
+    __shared__ alignas(16) int pos[REORDER_KEYS];
+    __shared__ int wsum[REORDER_THREADS / 32];
+    __shared__ float Rt[12];
+    if (threadIdx.x < 12) Rt[threadIdx.x] = Rt_g[threadIdx.x];
+    for (int k = threadIdx.x; k < REORDER_KEYS; k += blockDim.x) pos[k] = tot[k];
     __syncthreads();
+    cta_exclusive_scan<REORDER_KEYS, REORDER_THREADS>(pos, wsum);
+    for (int k = threadIdx.x; k < REORDER_KEYS; k += blockDim.x)
+        pos[k] += cnt[int64_t(blockIdx.x) * REORDER_KEYS + k];
+    __syncthreads();
+    const float scale = cell_scale(root);
     int lo, hi;
     cta_range(n, blockIdx.x, gridDim.x, lo, hi);
-    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        const uint32_t key = keys[i] & (REORDER_KEYS - 1);
-        const int slot = atomicAdd(&pos[key], 1);
-        if (slot >= 0 && slot < n) dst[slot] = src[i];
+    for (int i = lo + threadIdx.x; i < hi; i += 4 * blockDim.x) {
+        float4 p[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (i + j * int(blockDim.x) < hi) p[j] = src[i + j * blockDim.x];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (i + j * int(blockDim.x) < hi) {
+                const int slot = atomicAdd(&pos[src_cell(p[j], Rt, scale) >> 12], 1);
+                if (slot >= 0 && slot < n) dst[slot] = p[j];
+            }
+    }
+}
+
+// Pass 3: the points of every tile of REFINE_TILE consecutive ones (now in
+// cell order) by cell and place within the cell, in REFINE_TILE buckets: a
+// tile that spans D cells keeps REFINE_BITS - ceil(log2 D) bits of the place.
+// One load and one store of every point, bound by the phases between them
+// (histogram, scan, scatter in shared memory): four CTAs per SM overlap theirs
+// (tiles of 4,096 points with two CTAs took 189 us for 16.8M points, these 111).
+__global__ void __launch_bounds__(REFINE_THREADS, 4) k_src_refine(float4* pts, int n, const float* __restrict__ Rt_g,
+                                                               const RootDev* __restrict__ root) {
+    constexpr int PER = REFINE_TILE / REFINE_THREADS;
+    extern __shared__ float4 tile[];  // REFINE_TILE points, then the buckets
+    int* bucket = reinterpret_cast<int*>(tile + REFINE_TILE);
+    __shared__ int wsum[REFINE_THREADS / 32];
+    __shared__ float Rt[12];
+    if (threadIdx.x < 12) Rt[threadIdx.x] = Rt_g[threadIdx.x];
+    for (int k = threadIdx.x; k < REFINE_TILE; k += blockDim.x) bucket[k] = 0;
+    __syncthreads();
+    const float scale = cell_scale(root);
+    const int64_t base = int64_t(blockIdx.x) * REFINE_TILE;
+    const int m = int(min(int64_t(REFINE_TILE), int64_t(n) - base));
+    const unsigned c0 = src_cell(pts[base], Rt, scale) >> 12, c1 = src_cell(pts[base + m - 1], Rt, scale) >> 12;
+    const int shift = 12 - REFINE_BITS + 32 - __clz(int(c1 - c0));  // the cells' range has 32 - clz bits
+    float4 p[PER];
+    int at[PER];  // bucket, and above its bits the rank in the bucket
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = threadIdx.x + j * REFINE_THREADS;
+        if (i < m) p[j] = pts[base + i];
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = threadIdx.x + j * REFINE_THREADS;
+        if (i >= m) continue;
+        const unsigned g = src_cell(p[j], Rt, scale) - (c0 << 12);
+        const int key = int(g >> shift) & (REFINE_TILE - 1);
+        at[j] = key | atomicAdd(&bucket[key], 1) << REFINE_BITS;
+    }
+    __syncthreads();
+    cta_exclusive_scan<REFINE_TILE, REFINE_THREADS>(bucket, wsum);
+#pragma unroll
+    for (int j = 0; j < PER; ++j)
+        if (threadIdx.x + j * REFINE_THREADS < m) tile[bucket[at[j] & (REFINE_TILE - 1)] + (at[j] >> REFINE_BITS)] = p[j];
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = threadIdx.x + j * REFINE_THREADS;
+        if (i < m) pts[base + i] = tile[i];
     }
 }
 
@@ -727,19 +872,29 @@ int hgmm_register_impl(hgmm_tree* t, const float4* src, int64_t n64, const doubl
                                                           t->reg_acc, t->reg_T, t->reg_Rt,
                                                           t->reg_bar, t->reg_obj);
     }
-    // a large source that fits the tree's free point buffer is reordered
-    // after its first round: node keys in the dead hand-off codes, per-CTA
-    // counts and key totals in the build's partials (both free after the
-    // build); CTAs: two per SM, fewer if the counts would not fit
-    const int reorder_ctas =
-        int(std::min<int64_t>(2 * t->n_sm, t->max_items * NPART * 2 / REORDER_KEYS - 1));
-    const bool reorder = iters > 1 && n >= REORDER_MIN_POINTS && n64 <= t->cap && reorder_ctas >= 32 &&
-                         n_nodes < REORDER_KEYS && !t->trace_on;
+    // a large source that fits the tree's free point buffer is put into
+    // spatial order there, with the CTAs' cell counts and the cells' totals in
+    // the build's partials (free after the build); CTAs: two per SM, fewer if
+    // the counts would not fit
+    const int reorder_ctas = int(std::min<int64_t>(std::min(2 * t->n_sm, REORDER_MAX_CTAS),
+                                                   t->max_items * NPART * 2 / REORDER_KEYS - 1));
+    if (iters > 1 && n >= REORDER_MIN_POINTS && n64 <= t->cap && reorder_ctas >= 32 && t->refine_ok && !t->trace_on) {
+        ProfScope ps_(t, K_REG_INIT, s);
+        float4* sorted = t->pts[t->depth & 1];
+        int* cnt = reinterpret_cast<int*>(t->partials);
+        int* tot = cnt + int64_t(reorder_ctas) * REORDER_KEYS;
+        k_src_count<<<reorder_ctas, REORDER_THREADS, 0, s>>>(src, n, t->reg_Rt, t->root, cnt);
+        k_src_colscan<<<REORDER_KEYS / 32, 1024, 0, s>>>(cnt, reorder_ctas, tot);
+        k_src_scatter<<<reorder_ctas, REORDER_THREADS, 0, s>>>(src, n, t->reg_Rt, t->root, cnt, tot, sorted);
+        k_src_refine<<<(n + REFINE_TILE - 1) / REFINE_TILE, REFINE_THREADS, REFINE_SMEM, s>>>(sorted, n, t->reg_Rt,
+                                                                                               t->root);
+        src = sorted;
+    }
     const bool wide = n >= REG_WIDE_MIN_POINTS && t->reg_grid_wide > 0;
     const int grid = wide ? t->reg_grid_wide : t->reg_grid;
-    auto launch = [&](const float4* pts, int rounds, double* hist, uint32_t* keys) -> int {
+    if (iters > 0) {
         RegArgs a;
-        a.src = pts;
+        a.src = src;
         a.n = n;
         a.est = t->est;
         a.blocks = t->rblk;
@@ -747,54 +902,28 @@ int hgmm_register_impl(hgmm_tree* t, const float4* src, int64_t n64, const doubl
         a.root = t->root;
         a.depth = t->depth;
         a.n_nodes = n_nodes;
-        a.iters = rounds;
+        a.iters = iters;
         a.acc = t->reg_acc;
         a.part = t->reg_part;
         a.bar = t->reg_bar;
         a.T = t->reg_T;
         a.Rt = t->reg_Rt;
-        a.T_hist = hist;
+        a.T_hist = T_hist;
         a.dbg = t->reg_dbg;
         a.obj = t->reg_obj;
         a.status = t->status;
-        a.keys = keys;
-        a.trace = (t->trace_on && rounds <= TRACE_MAX_ITERS) ? t->trace : nullptr;
-        if (a.trace) cudaMemsetAsync(t->trace, 0, size_t(rounds) * grid * TRACE_EVENTS * 8, s);
-        t->trace_iters = a.trace ? rounds : 0;
+        a.trace = (t->trace_on && iters <= TRACE_MAX_ITERS) ? t->trace : nullptr;
+        if (a.trace) cudaMemsetAsync(t->trace, 0, size_t(iters) * grid * TRACE_EVENTS * 8, s);
+        t->trace_iters = a.trace ? iters : 0;
         t->trace_grid = a.trace ? grid : 0;
         void* args[] = {&a};
         ProfScope ps_(t, K_DESCEND, s);
-        const void* fn = wide ? (keys ? (const void*)k_register<true, 3> : (const void*)k_register<false, 3>)
-                              : (keys ? (const void*)k_register<true, 2> : (const void*)k_register<false, 2>);
-        const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(REG_THREADS), args,
-                                                          REG_DYN_SMEM, s);
+        const cudaError_t e = cudaLaunchCooperativeKernel(wide ? (const void*)k_register<3> : (const void*)k_register<2>,
+                                                          dim3(grid), dim3(REG_THREADS), args, REG_DYN_SMEM, s);
         if (e != cudaSuccess) {
             fprintf(stderr, "hgmm: cooperative launch failed: %s\n", cudaGetErrorString(e));
             return HGMM_ECUDA;
         }
-        return HGMM_OK;
-    };
-    if (reorder) {
-        // round 1 in the caller's order, recording each point's node
-        if (int rc = launch(src, 1, T_hist, t->codes)) return rc;
-        {
-            ProfScope ps_(t, K_REG_INIT, s);
-            float4* sorted = t->pts[t->depth & 1];
-            int* cnt = reinterpret_cast<int*>(t->partials);
-            int* tot = cnt + int64_t(reorder_ctas) * REORDER_KEYS;
-            k_src_count<<<reorder_ctas, REORDER_THREADS, 0, s>>>(t->codes, n, cnt);
-            k_src_colscan<<<REORDER_KEYS / 256, 256, 0, s>>>(cnt, reorder_ctas, tot);
-            k_src_keyscan<<<1, 1024, 0, s>>>(tot);
-            k_src_scatter<<<reorder_ctas, REORDER_THREADS, 0, s>>>(src, n, t->codes, cnt, tot, sorted);
-            src = sorted;
-            // the remaining rounds start from the pose after round 1
-            k_reg_init<<<(n_nodes + 255) / 256, 256, 0, s>>>(t->reg_T, n_nodes, lam_c, t->stat, t->est, t->rblk,
-                                                              t->reg_acc, t->reg_T, t->reg_Rt,
-                                                              t->reg_bar, t->reg_obj);
-        }
-        if (int rc = launch(src, iters - 1, T_hist ? T_hist + 16 : nullptr, nullptr)) return rc;
-    } else if (iters > 0) {
-        if (int rc = launch(src, iters, T_hist, nullptr)) return rc;
     }
     if (T_out) {
         ProfScope ps_(t, K_COPY_T, s);
@@ -856,19 +985,20 @@ int hgmm_register_grid(int n_sm, int per_sm) {
     // for; 0 if that build does not reach per_sm CTAs per SM (the caller then
     // keeps to the two-per-SM build)
     if (per_sm != 2 && per_sm != 3) return 0;
-    const void* fns[2] = {per_sm == 3 ? (const void*)k_register<false, 3> : (const void*)k_register<false, 2>,
-                          per_sm == 3 ? (const void*)k_register<true, 3> : (const void*)k_register<true, 2>};
-    int got = per_sm;
-    for (const void* fn : fns) {
-        int k = 0;
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(REG_DYN_SMEM)) !=
-                cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, fn, REG_THREADS, REG_DYN_SMEM) != cudaSuccess || k < 1)
-            return 0;
-        got = std::min(got, k);
-    }
+    const void* fn = per_sm == 3 ? (const void*)k_register<3> : (const void*)k_register<2>;
+    int k = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(REG_DYN_SMEM)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, fn, REG_THREADS, REG_DYN_SMEM) != cudaSuccess || k < 1)
+        return 0;
+    const int got = std::min(per_sm, k);
     if (per_sm == 3 && got < 3) return 0;
     return n_sm * got;  // <= co-resident CTAs (cooperative launch)
+}
+
+// The source reorder's dynamic shared memory; false: sources keep their order.
+bool hgmm_reorder_smem_attr() {
+    return cudaFuncSetAttribute(k_src_refine, cudaFuncAttributeMaxDynamicSharedMemorySize, int(REFINE_SMEM)) ==
+           cudaSuccess;
 }
 
 int hgmm_trace_read_impl(hgmm_tree* t, unsigned long long* h, int64_t cap) {
