@@ -160,6 +160,13 @@ __device__ void sort_source_by_node(const float4* __restrict__ src, int n, int n
     cl.sync();  // the sorted cloud is complete for the whole cluster
 }
 
+// The registration's descent as a function of its own (see called_estep_items).
+__device__ __noinline__ void called_descent(const float4* src, int n, const float4* blocks, const float4* sm_blocks,
+                                            int depth, const float* Rt, float qscale, unsigned long long* acc, int cta,
+                                            int ncta, unsigned long long* hist, uint32_t* key_out) {
+    descend_points(src, n, blocks, sm_blocks, depth, Rt, qscale, acc, cta, ncta, hist, key_out);
+}
+
 // One pair, run by all CTAs of this cluster.
 template <bool COMP>
 __device__ void run_pair(const BatchArgs& a, const BatchWs& w, int cid, int pair, cg::cluster_group& cl,
@@ -259,7 +266,7 @@ __device__ void run_pair(const BatchArgs& a, const BatchWs& w, int cid, int pair
             for (int i = threadIdx.x; i < n_staged / 8 * BLOCK_F4; i += blockDim.x) sm_est[i] = __ldcg(w.rblk + i);
         }
         __syncthreads();
-        descend_points(src, n_s, w.rblk, sm_est, depth, rgs.Rt, qscale, w.acc, rank, cs, hist,
+        called_descent(src, n_s, w.rblk, sm_est, depth, rgs.Rt, qscale, w.acc, rank, cs, hist,
                        it == 0 && sort_src ? w.codes : nullptr);
         __syncthreads();
         flush_node_hist(hist, n_staged, w.acc);
