@@ -77,57 +77,102 @@ __global__ void k_fill_items(int level, int n, int n_parents, const int* __restr
     items[j] = item_at(j, level, n, n_parents, item_range, seg_start, seg_count);
 }
 
-// The level-wide E-step: the arithmetic of estep_range (so the result is
-// the same bit for bit), with each item's points (one contiguous run of at
-// most TILE float4) brought into shared memory by one bulk asynchronous copy,
-// ESTEP_STAGES items ahead of the compute, so that no warp waits on a global
-// load.  One thread issues the copies; each completes on its stage's
-// mbarrier; a stage is refilled after the CTA's barrier at the end of the
-// item that used it (with an async-proxy fence).  All waits are bounded: on
-// a timeout the CTA records ST_TIMEOUT, waits (bounded) for its copies in
-// flight and stops.
+// The level-wide E-step's threads: each holds two of the accumulator sets that
+// estep_range spreads over EST_THREADS.
+constexpr int ESTEP_CTA = EST_THREADS / 2;
 constexpr int ESTEP_STAGES = 4;
 // Dynamic shared memory of k_estep: the compensated sums (s, c) of every
-// lane's ten packed moment pairs, [value][thread], kept out of the register
-// file so that three CTAs fit on an SM.
+// set's ten packed moment pairs, [value][set], kept out of the register file.
 constexpr size_t ESTEP_DYN_SMEM = size_t(2) * 10 * EST_THREADS * sizeof(float2);
 
-// fold_pair with the compensated sums in shared memory (the same arithmetic).
+// fold_pair of a thread's two sets (2 t and 2 t + 1) with the compensated sums
+// in shared memory (the same arithmetic).
 template <bool COMP>
-__device__ __forceinline__ void fold_pair_smem(float2 (&in)[10], float2* acc_s, float2* acc_c) {
-    const int t = threadIdx.x;
+__device__ __forceinline__ void fold_sets(float2 (&in)[2][10], float2* acc_s, float2* acc_c) {
+    float4* s4 = reinterpret_cast<float4*>(acc_s) + threadIdx.x;
+    float4* c4 = reinterpret_cast<float4*>(acc_c) + threadIdx.x;
 #pragma unroll
     for (int v = 0; v < 10; ++v) {
-        float2 sv = acc_s[v * EST_THREADS + t];
+        const float4 sv = s4[v * ESTEP_CTA];
+        const float2 s[2] = {make_float2(sv.x, sv.y), make_float2(sv.z, sv.w)};
+        float2 t[2];
         if (COMP) {
-            float2 cv = acc_c[v * EST_THREADS + t];
-            const float2 tt = __fadd2_rn(sv, in[v]);
-            const float2 bp = sub2(tt, sv);
-            const float2 e = __fadd2_rn(sub2(sv, sub2(tt, bp)), sub2(in[v], bp));
-            sv = tt;
-            cv = __fadd2_rn(cv, e);
-            acc_c[v * EST_THREADS + t] = cv;
+            const float4 cv = c4[v * ESTEP_CTA];
+            const float2 c[2] = {make_float2(cv.x, cv.y), make_float2(cv.z, cv.w)};
+            float2 d[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                t[j] = __fadd2_rn(s[j], in[j][v]);
+                const float2 bp = sub2(t[j], s[j]);
+                d[j] = __fadd2_rn(c[j], __fadd2_rn(sub2(s[j], sub2(t[j], bp)), sub2(in[j][v], bp)));
+            }
+            c4[v * ESTEP_CTA] = make_float4(d[0].x, d[0].y, d[1].x, d[1].y);
         } else {
-            sv = __fadd2_rn(sv, in[v]);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) t[j] = __fadd2_rn(s[j], in[j][v]);
         }
-        acc_s[v * EST_THREADS + t] = sv;
-        in[v] = make_float2(0.f, 0.f);
+        s4[v * ESTEP_CTA] = make_float4(t[0].x, t[0].y, t[1].x, t[1].y);
+        in[0][v] = in[1][v] = make_float2(0.f, 0.f);
     }
 }
 
+// flush_run of all sets (which are cleared), two passes of EST_THREADS / 2:
+// the sums over the lanes and warps of estep_range, in its order.
 template <bool COMP>
-__device__ __forceinline__ void flush_pair_smem(float2* acc_s, float2* acc_c, float2 (*red)[NPART],
-                                                float2* __restrict__ out) {
-    float2 s2[10], c2[10];
-    const int t = threadIdx.x;
+__device__ __forceinline__ void flush_sets(float2* acc_s, float2* acc_c, float2 (*red)[NPART],
+                                           float2* __restrict__ out) {
+    __syncthreads();  // every thread's sets are folded
+    // both passes side by side: levels of many small parents flush often
+    float s[2][20], c[2][20];
 #pragma unroll
-    for (int v = 0; v < 10; ++v) {
-        s2[v] = acc_s[v * EST_THREADS + t];
-        c2[v] = COMP ? acc_c[v * EST_THREADS + t] : make_float2(0.f, 0.f);
-        acc_s[v * EST_THREADS + t] = make_float2(0.f, 0.f);
-        acc_c[v * EST_THREADS + t] = make_float2(0.f, 0.f);
+    for (int j = 0; j < 2; ++j) {
+        const int t = threadIdx.x + j * ESTEP_CTA;
+#pragma unroll
+        for (int v = 0; v < 10; ++v) {
+            const float2 s2 = acc_s[v * EST_THREADS + t];
+            const float2 c2 = COMP ? acc_c[v * EST_THREADS + t] : make_float2(0.f, 0.f);
+            s[j][v] = s2.x;
+            s[j][10 + v] = s2.y;
+            c[j][v] = c2.x;
+            c[j][10 + v] = c2.y;
+            acc_s[v * EST_THREADS + t] = make_float2(0.f, 0.f);
+            acc_c[v * EST_THREADS + t] = make_float2(0.f, 0.f);
+        }
     }
-    flush_pair<COMP>(s2, c2, red, out);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) flush_warp<COMP>(s[j], c[j], (threadIdx.x + j * ESTEP_CTA) >> 5, red);
+    flush_rows<COMP>(red, out);
+}
+
+// estep_point_pair with the point's eight children on two lanes instead of
+// four: half the shuffles, point loads and loop instructions per point (353 ->
+// 267 lane instructions; 16M points built in 9.71 -> 8.70 ms, with 12 instead
+// of 24 warps per SM), and two independent chains per thread.  The sums keep
+// the quad's tree: (01) + (23) here, (45) + (67) on the other lane.  The FMA pipe is busy half of the time; per-warp hand-over of the stages instead
+// of a CTA barrier per item was slower (16M points built in 8.97 ms against
+// 8.71), and so was a loop that is not unrolled over the item (9.53).
+__device__ __forceinline__ void estep_point_half(const ChildPair (&cp)[2], const float4 z, bool valid,
+                                                 float2 (&in)[2][10]) {
+    float2 ex[2], ey[2], ez[2], u[2], p[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        ex[j] = add1(cp[j].nmx, z.x);
+        ey[j] = add1(cp[j].nmy, z.y);
+        ez[j] = add1(cp[j].nmz, z.z);
+        u[j] = neg_score_at(cp[j], ex[j], ey[j], ez[j]);
+    }
+    float umin = fminf(fminf(u[0].x, u[0].y), fminf(u[1].x, u[1].y));
+    umin = fminf(umin, __shfl_xor_sync(FULL, umin, 1));
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const float2 arg = from1(umin, u[j]);  // = score - max score
+        p[j] = make_float2(ex2_fast(arg.x), ex2_fast(arg.y));
+    }
+    float tot = (p[0].x + p[0].y) + (p[1].x + p[1].y);
+    tot += __shfl_xor_sync(FULL, tot, 1);
+    const float rinv = valid ? rcp_fast(tot) : 0.0f;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) accum_pair(in[j], mul1(p[j], rinv), ex[j], ey[j], ez[j]);
 }
 
 // The level-wide E-step: the arithmetic of estep_range (so the result is
@@ -140,26 +185,22 @@ __device__ __forceinline__ void flush_pair_smem(float2* acc_s, float2* acc_c, fl
 // fence).  All waits are bounded: on a timeout the CTA records ST_TIMEOUT,
 // waits (bounded) for its copies in flight and stops.
 template <bool COMP>
-__global__ void __launch_bounds__(EST_THREADS, 3)
+__global__ void __launch_bounds__(ESTEP_CTA, 3)
 k_estep(const float4* __restrict__ pts, const Item* __restrict__ items,
         const int* __restrict__ meta, const NodeEst* __restrict__ est_lvl,
         float2* __restrict__ partials, int* __restrict__ status) {
     __shared__ float2 red[EST_THREADS / 32][NPART];
     __shared__ __align__(16) float4 stage[ESTEP_STAGES][TILE];
     __shared__ __align__(8) uint64_t full[ESTEP_STAGES];
-    extern __shared__ float2 estep_dyn[];
-    float2* acc_s = estep_dyn;
-    float2* acc_c = estep_dyn + 10 * EST_THREADS;
+    extern __shared__ float4 estep_dyn[];
+    float2* acc_s = reinterpret_cast<float2*>(estep_dyn);
+    float2* acc_c = acc_s + 10 * EST_THREADS;
     const int n_items = meta[0];
     const int C = meta[1];
     const int ib = blockIdx.x * C, ie = min(ib + C, n_items);
     if (ib >= ie) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int q = lane >> 2, k = lane & 3;
-    for (int v = 0; v < 10; ++v) {
-        acc_s[v * EST_THREADS + threadIdx.x] = make_float2(0.f, 0.f);
-        acc_c[v * EST_THREADS + threadIdx.x] = make_float2(0.f, 0.f);
-    }
+    const int q = threadIdx.x >> 1, h = threadIdx.x & 1;  // point of a step, half of its children
+    for (int v = threadIdx.x; v < 10 * EST_THREADS; v += ESTEP_CTA) acc_s[v] = acc_c[v] = make_float2(0.f, 0.f);
     if (threadIdx.x == 0) {
         for (int st = 0; st < ESTEP_STAGES; ++st) tc::mbar_init(&full[st], 1);
         tc::fence_mbar_init();
@@ -171,26 +212,27 @@ k_estep(const float4* __restrict__ pts, const Item* __restrict__ items,
         }
     }
     __syncthreads();
-    float2 in[10];
+    float2 in[2][10];
 #pragma unroll
-    for (int v = 0; v < 10; ++v) in[v] = make_float2(0.f, 0.f);
+    for (int v = 0; v < 10; ++v) in[0][v] = in[1][v] = make_float2(0.f, 0.f);
     int nfold = 0;
     int cur = -1, run = -1;
     bool live = false;
-    ChildPair cp;
+    ChildPair cp[2];
     int it = ib;
     for (; it < ie; ++it) {
         const Item w = items[it];
         if (w.parent != cur) {
             if (cur >= 0) {
-                fold_pair_smem<COMP>(in, acc_s, acc_c);
+                fold_sets<COMP>(in, acc_s, acc_c);
                 nfold = 0;
-                flush_pair_smem<COMP>(acc_s, acc_c, red, partials + int64_t(run) * NPART);
+                flush_sets<COMP>(acc_s, acc_c, red, partials + int64_t(run) * NPART);
             }
             cur = w.parent;
             run = it;
-            load_child_pair(est_lvl + 8 * cur + 2 * k, cp);
-            live = parent_has_live_child(cp);
+            load_child_pair(est_lvl + 8 * cur + 4 * h, cp[0]);
+            load_child_pair(est_lvl + 8 * cur + 4 * h + 2, cp[1]);
+            live = parent_has_live_child(cp[0]) || parent_has_live_child(cp[1]);
         }
         const int st = (it - ib) % ESTEP_STAGES;
         const uint32_t parity = uint32_t((it - ib) / ESTEP_STAGES) & 1u;
@@ -198,15 +240,26 @@ k_estep(const float4* __restrict__ pts, const Item* __restrict__ items,
         // (in bounds, discarded): the CTA's vote at the end of the item stops it
         const bool landed = tc::mbar_wait_bounded(&full[st], parity, tc::MBAR_SPIN_LIMIT);
         const float4* zs = stage[st];
-        // a parent without a live child: zero posteriors, nothing to add
-        for (int base = 0; live && base < w.count; base += 64) {
-            const int idx = base + warp * 8 + q;
-            const bool valid = idx < w.count;
-            const float4 z = zs[min(idx, w.count - 1)];
-            estep_point_pair(cp, z, valid, in);
-            if (++nfold == EST_FOLD) {
-                fold_pair_smem<COMP>(in, acc_s, acc_c);
+        if (!live) {
+            // a parent without a live child: zero posteriors, nothing to add
+        } else if (w.count == TILE && nfold % (TILE / 64) == 0) {
+            // a whole item (all but a parent's last): no bounds, and the fold
+            // falls on its end
+#pragma unroll
+            for (int base = 0; base < TILE; base += 64) estep_point_half(cp, zs[base + q], true, in);
+            nfold += TILE / 64;
+            if (nfold == EST_FOLD) {
+                fold_sets<COMP>(in, acc_s, acc_c);
                 nfold = 0;
+            }
+        } else {
+            for (int base = 0; base < w.count; base += 64) {
+                const int idx = base + q;
+                estep_point_half(cp, zs[min(idx, w.count - 1)], idx < w.count, in);
+                if (++nfold == EST_FOLD) {
+                    fold_sets<COMP>(in, acc_s, acc_c);
+                    nfold = 0;
+                }
             }
         }
         // every thread is done with this stage (one barrier per item, which
@@ -231,8 +284,8 @@ k_estep(const float4* __restrict__ pts, const Item* __restrict__ items,
                                       tc::MBAR_SPIN_LIMIT);
         return;
     }
-    fold_pair_smem<COMP>(in, acc_s, acc_c);
-    flush_pair_smem<COMP>(acc_s, acc_c, red, partials + int64_t(run) * NPART);
+    fold_sets<COMP>(in, acc_s, acc_c);
+    flush_sets<COMP>(acc_s, acc_c, red, partials + int64_t(run) * NPART);
 }
 
 // The level-wide M-step: CTA (p, j) reduces slice j of parent p's runs into
@@ -778,9 +831,9 @@ int hgmm_build_impl(hgmm_tree* t, const float4* pts, int64_t n64, int depth,
             {
                 ProfScope ps_(t, K_ESTEP, s);
                 if (comp)
-                    k_estep<true><<<G, EST_THREADS, ESTEP_DYN_SMEM, s>>>(cur, t->items, t->meta, est_lvl, t->partials, t->status);
+                    k_estep<true><<<G, ESTEP_CTA, ESTEP_DYN_SMEM, s>>>(cur, t->items, t->meta, est_lvl, t->partials, t->status);
                 else
-                    k_estep<false><<<G, EST_THREADS, ESTEP_DYN_SMEM, s>>>(cur, t->items, t->meta, est_lvl, t->partials, t->status);
+                    k_estep<false><<<G, ESTEP_CTA, ESTEP_DYN_SMEM, s>>>(cur, t->items, t->meta, est_lvl, t->partials, t->status);
             }
             {
                 ProfScope ps_(t, K_MSTEP, s);
@@ -1005,12 +1058,12 @@ extern "C" int hgmm_fit_level0_noalloc(const float* d_points, int64_t n, const h
                                                             items);
     for (int k = 0; k < prm.em_iters; ++k) {
         if (prm.precision == 0) {
-            k_estep<true><<<G, EST_THREADS, ESTEP_DYN_SMEM, s>>>(reinterpret_cast<const float4*>(d_points), items,
+            k_estep<true><<<G, ESTEP_CTA, ESTEP_DYN_SMEM, s>>>(reinterpret_cast<const float4*>(d_points), items,
                                                     meta, est, partials, status);
             k_mstep<true><<<dim3(1, 1), 256, 0, s>>>(0, ni, item_range, meta, partials, seg, root,
                                             prm.n_min, stat, est, status, nullptr, nullptr);
         } else {
-            k_estep<false><<<G, EST_THREADS, ESTEP_DYN_SMEM, s>>>(reinterpret_cast<const float4*>(d_points), items,
+            k_estep<false><<<G, ESTEP_CTA, ESTEP_DYN_SMEM, s>>>(reinterpret_cast<const float4*>(d_points), items,
                                                      meta, est, partials, status);
             k_mstep<false><<<dim3(1, 1), 256, 0, s>>>(0, ni, item_range, meta, partials, seg, root,
                                              prm.n_min, stat, est, status, nullptr, nullptr);

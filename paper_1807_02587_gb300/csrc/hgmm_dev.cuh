@@ -444,19 +444,31 @@ __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
 // x - y, rounded once (as __fsub_rn)
 __device__ __forceinline__ float2 sub2(float2 x, float2 y) { return __ffma2_rn(y, f2(-1.f), x); }
 
+// x + y, y - x and x y with one y for both halves: scalar instructions, which
+// take as long on the FMA pipe as the packed ones and want no copy of y into a
+// pair of registers.
+__device__ __forceinline__ float2 add1(float2 x, float y) { return make_float2(__fadd_rn(x.x, y), __fadd_rn(x.y, y)); }
+__device__ __forceinline__ float2 from1(float y, float2 x) { return make_float2(__fsub_rn(y, x.x), __fsub_rn(y, x.y)); }
+__device__ __forceinline__ float2 mul1(float2 x, float y) { return make_float2(__fmul_rn(x.x, y), __fmul_rn(x.y, y)); }
+
 // u = -log2(pi N(z | child)) of both children (exactly the negated
-// child_score) and the offsets e = z - mu.
-__device__ __forceinline__ float2 neg_score_pair(const ChildPair& p, float zx, float zy, float zz, float2& ex,
-                                                 float2& ey, float2& ez) {
-    ex = __fadd2_rn(f2(zx), p.nmx);
-    ey = __fadd2_rn(f2(zy), p.nmy);
-    ez = __fadd2_rn(f2(zz), p.nmz);
+// child_score) from the offsets e = z - mu.
+__device__ __forceinline__ float2 neg_score_at(const ChildPair& p, float2 ex, float2 ey, float2 ez) {
     const float2 d0 = __fmul2_rn(p.w00, ex);
     const float2 d1 = __ffma2_rn(p.w11, ey, __fmul2_rn(p.w10, ex));
     const float2 d2 = __ffma2_rn(p.w22, ez, __ffma2_rn(p.w21, ey, __fmul2_rn(p.w20, ex)));
     float2 u = __ffma2_rn(d0, d0, p.nC);
     u = __ffma2_rn(d1, d1, u);
     return __ffma2_rn(d2, d2, u);
+}
+
+// The same with the offsets.
+__device__ __forceinline__ float2 neg_score_pair(const ChildPair& p, float zx, float zy, float zz, float2& ex,
+                                                 float2& ey, float2& ez) {
+    ex = __fadd2_rn(f2(zx), p.nmx);
+    ey = __fadd2_rn(f2(zy), p.nmy);
+    ez = __fadd2_rn(f2(zz), p.nmz);
+    return neg_score_at(p, ex, ey, ez);
 }
 
 // accum10 of both children: a[v].x / .y = moment v of child 2k / 2k + 1.
@@ -575,27 +587,30 @@ __device__ __forceinline__ void flush_rs_level(float* s, float* c, int lane) {
     }
 }
 
-// Block-wide reduction of the (s, c) accumulators into partial slot `run`.
-// Within a warp the eight lanes of each child pair reduce-scatter their 20
-// values (18 compensated additions and 36 shuffles per lane instead of 60
-// and 120 for a butterfly); each value's warp total then sits in exactly
-// one lane, which stores it for the fixed-order sum over the warps.
+// A warp's share of the block-wide reduction of the (s, c) accumulators: the
+// eight lanes of each child pair reduce-scatter their 20 values (18
+// compensated additions and 36 shuffles per lane instead of 60 and 120 for a
+// butterfly); each value's warp total then sits in exactly one lane, which
+// stores it in row `warp` of red.
 template <bool COMP>
-__device__ __forceinline__ void flush_run(float* s, float* c, float2 (*red)[NPART],
-                                          float2* __restrict__ out) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = lane & 3;
+__device__ __forceinline__ void flush_warp(float* s, float* c, int warp, float2 (*red)[NPART]) {
+    const int lane = threadIdx.x & 31, k = lane & 3;
     flush_rs_level<COMP, 20, 16>(s, c, lane);  // 10 values left
     flush_rs_level<COMP, 10, 8>(s, c, lane);   // 5
     flush_rs_level<COMP, 5, 4>(s, c, lane);    // 3 (lower lane) or 2 (upper lane)
-    {
-        // the values this lane now holds: a half of 20 by lane bit 4, of
-        // that a half of 10 by bit 3, of that the first 3 or last 2 by bit 2
-        const int base = ((lane & 16) ? 10 : 0) + ((lane & 8) ? 5 : 0) + ((lane & 4) ? 3 : 0);
-        const int cnt = (lane & 4) ? 2 : 3;
+    // the values this lane now holds: a half of 20 by lane bit 4, of
+    // that a half of 10 by bit 3, of that the first 3 or last 2 by bit 2
+    const int base = ((lane & 16) ? 10 : 0) + ((lane & 8) ? 5 : 0) + ((lane & 4) ? 3 : 0);
+    const int cnt = (lane & 4) ? 2 : 3;
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
-            if (i < cnt) red[warp][k * 20 + base + i] = make_float2(s[i], COMP ? c[i] : 0.f);
-    }
+    for (int i = 0; i < 3; ++i)
+        if (i < cnt) red[warp][k * 20 + base + i] = make_float2(s[i], COMP ? c[i] : 0.f);
+}
+
+// The fixed-order sum over the EST_THREADS / 32 rows of red into out, between
+// two CTA barriers.
+template <bool COMP>
+__device__ __forceinline__ void flush_rows(float2 (*red)[NPART], float2* __restrict__ out) {
     __syncthreads();
     if (threadIdx.x < NPART) {
         float S = 0.f, Cc = 0.f;
@@ -607,6 +622,14 @@ __device__ __forceinline__ void flush_run(float* s, float* c, float2 (*red)[NPAR
         out[threadIdx.x] = make_float2(S, Cc);
     }
     __syncthreads();
+}
+
+// Block-wide reduction of the (s, c) accumulators into a partial.
+template <bool COMP>
+__device__ __forceinline__ void flush_run(float* s, float* c, float2 (*red)[NPART],
+                                          float2* __restrict__ out) {
+    flush_warp<COMP>(s, c, threadIdx.x >> 5, red);
+    flush_rows<COMP>(red, out);
 #pragma unroll
     for (int v = 0; v < 20; ++v) { s[v] = 0.f; c[v] = 0.f; }
 }
@@ -1570,7 +1593,7 @@ __device__ __forceinline__ void block_scores(const float4* blk, Load load, float
     for (int k = 0; k < 4; ++k) {
         const float4 q0 = load(blk + 5 * k), q1 = load(blk + 5 * k + 1), q2 = load(blk + 5 * k + 2);
         const float4 q3 = load(blk + 5 * k + 3), q4 = load(blk + 5 * k + 4);
-        const float2 ex = __fadd2_rn(f2(x), lo(q0)), ey = __fadd2_rn(f2(y), hi(q0)), ez = __fadd2_rn(f2(z), lo(q1));
+        const float2 ex = add1(lo(q0), x), ey = add1(hi(q0), y), ez = add1(lo(q1), z);
         const float2 d0 = __fmul2_rn(lo(q2), ex);
         const float2 d1 = __ffma2_rn(lo(q3), ey, __fmul2_rn(hi(q2), ex));
         const float2 d2 = __ffma2_rn(hi(q4), ez, __ffma2_rn(lo(q4), ey, __fmul2_rn(hi(q3), ex)));
@@ -1745,7 +1768,7 @@ __device__ __forceinline__ void descend_points(const float4* __restrict__ src, i
             float sum = 0.f;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const float2 d = sub2(f2(best), u[k]);
+                const float2 d = from1(best, u[k]);
                 sum += ex2_fast(d.x);
                 sum += ex2_fast(d.y);
             }

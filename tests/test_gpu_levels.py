@@ -29,7 +29,9 @@ def _cloud(kind, n):
 @pytest.mark.parametrize("kind,n,depth", [
     ("scene", 8, 1), ("scene", 255, 2), ("scene", 257, 3), ("scene", 1024, 3), ("scene", 1025, 4),
     ("scene", 256 * CHUNKS, 2), ("scene", 256 * CHUNKS + 1, 2), ("scene", 512 * CHUNKS + 1, 2),
-    ("scene", 409600, 2), ("blob", 150001, 4)])
+    ("scene", 409600, 2), ("blob", 150001, 4),
+    # the level-wide E-step: two threads per point, whole and ragged items
+    ("scene", 409601, 3), ("blob", 700001, 4)])
 def test_em_iterations_of_every_level(kind, n, depth):
     from paper_1807_02587_gb300 import binding as B
     dev, Z = PT.device_cloud(_cloud(kind, n))
