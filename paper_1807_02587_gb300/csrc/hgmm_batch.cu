@@ -92,8 +92,13 @@ constexpr size_t BATCH_DYN_SMEM =
     STAGED_F4 * sizeof(float4) + 4 * STAGED_NODES * sizeof(unsigned long long);
 
 // Sources of at least this many points are reordered by their first-round
-// node before the second round (below that the sort costs about what it saves).
+// node before the second round (below that the sort costs about what it
+// saves), and, where at least twice as many rounds follow, once more before
+// round BATCH_RESORT_ROUND: the first order goes stale as the pose moves (256
+// pairs of 2,000 to 200,000 points, 30 rounds: 34.0 ms with the first sort
+// alone, 33.5 / 33.1 / 33.1 with a second before round 4 / 6 / 9).
 constexpr int BATCH_REORDER_MIN = 16384;
+constexpr int BATCH_RESORT_ROUND = 6;
 
 // Counting sort of the pair's source points by the node each reached in the
 // first round (keys: node id, all ones = none -> key n_nodes), by the
@@ -244,7 +249,8 @@ __device__ void run_pair(const BatchArgs& a, const BatchWs& w, int cid, int pair
     // the descent's sibling blocks: all of them in global memory, shared over
     // the cluster, and the staged levels' in every CTA's shared memory
     const int n_staged = n_nodes < STAGED_NODES ? n_nodes : STAGED_NODES;
-    for (int g = 32 * (rank * wpb + warp); g < n_nodes; g += 32 * cs * wpb) pack_blocks(w.rblk, w.est, g, n_nodes, n_nodes);
+    for (int g = 32 * (rank * wpb + warp); g < n_nodes; g += 32 * cs * wpb)
+        pack_blocks(w.rblk, w.est, g, n_nodes, n_nodes);
     cl.sync();
     for (int i = threadIdx.x; i < n_staged / 8 * BLOCK_F4; i += blockDim.x) sm_est[i] = __ldcg(w.rblk + i);
     const double ext = __ldcg(&w.root->extent) > 0.0 ? __ldcg(&w.root->extent) : 1.0;
@@ -254,20 +260,22 @@ __device__ void run_pair(const BatchArgs& a, const BatchWs& w, int cid, int pair
     // before the second; the sort borrows the staged nodes' shared memory
     const bool sort_src = a.iters >= 2 && n_s >= BATCH_REORDER_MIN &&
                           n_nodes + 1 <= int(STAGED_F4 * sizeof(float4) / sizeof(int));
+    const int resort = a.iters >= 3 * BATCH_RESORT_ROUND ? BATCH_RESORT_ROUND : -1;
     if (threadIdx.x < 12) {
         rgs.T[threadIdx.x] = __ldcg(w.T + threadIdx.x);
         rgs.Rt[threadIdx.x] = __ldcg(w.Rt + threadIdx.x);
     }
     for (int it = 0; it < a.iters; ++it) {
-        if (it == 1 && sort_src) {
-            sort_source_by_node(src, n_s, n_nodes, w.codes, w.pts[0], rank, cs, cl,
+        if (sort_src && (it == 1 || it == resort)) {
+            float4* sorted = w.pts[it == 1 ? 0 : 1];
+            sort_source_by_node(src, n_s, n_nodes, w.codes, sorted, rank, cs, cl,
                                 reinterpret_cast<int*>(sm_est));
-            src = w.pts[0];
+            src = sorted;
             for (int i = threadIdx.x; i < n_staged / 8 * BLOCK_F4; i += blockDim.x) sm_est[i] = __ldcg(w.rblk + i);
         }
         __syncthreads();
         called_descent(src, n_s, w.rblk, sm_est, depth, rgs.Rt, qscale, w.acc, rank, cs, hist,
-                       it == 0 && sort_src ? w.codes : nullptr);
+                       sort_src && (it == 0 || it == resort - 1) ? w.codes : nullptr);
         __syncthreads();
         flush_node_hist(hist, n_staged, w.acc);
         cl.sync();
