@@ -49,11 +49,13 @@ L2_FLUSH_BYTES = 512 << 20
 # (bytes of DRAM traffic a perfect kernel needs, FP32 flops with FMA = 2)
 KERNEL_WORK = {
     "estep": {"bytes": 16, "flops": 355, "unit": "target point"},
+    # all levels of the build in one launch: 8 E-steps and the labels per level
+    "build_levels": {"bytes": 16, "flops": DEPTH * (8 * 355 + 160), "unit": "target point"},
     "assign": {"bytes": 20, "flops": 160, "unit": "target point"},
     "scatter": {"bytes": 44, "flops": 0, "unit": "target point"},
     "register": {"bytes": 16, "flops": None, "unit": "source point"},
 }
-REGISTER_TRAFFIC_BYTES = 1966336
+REGISTER_TRAFFIC_BYTES = 2000128
 DESCEND_FLOPS_PER_LEVEL = 8 * 18 + 8 * 2 + 8  # 8 child scores, 8 exp2 + sum, rcp
 DESCEND_FLOPS_FIXED = 18 + 12  # transform, fixed-point conversion
 

@@ -81,9 +81,10 @@ constexpr int TRACE_EVENTS = 6;
 constexpr size_t REG_DYN_SMEM = STAGED_F4 * sizeof(float4) + 4 * STAGED_NODES * sizeof(unsigned long long);
 // three CTAs per SM (dynamic + ~4 KB static + 1 KB reserved each) within 228 KB
 static_assert(3 * (REG_DYN_SMEM + 5 * 1024) <= 228 * 1024, "three k_register CTAs must fit on one SM");
-// sources from this size on take the three-CTAs-per-SM build (measured: 1M
-// points run 10 rounds in 0.65 ms with two CTAs per SM against 0.68 with
-// three; 4M in 1.58 against 1.42; 16M in 6.0 against 5.2)
+// sources from this size on take the three-CTAs-per-SM build (measured, 30
+// rounds: 2.2M points 2.29 ms with two CTAs per SM against 2.13 with three; 4M
+// 3.63 against 3.30; 16M 14.5 against 12.6; 10 rounds of 1M, before the sibling
+// blocks, 0.65 against 0.68)
 constexpr int REG_WIDE_MIN_POINTS = 1 << 21;
 
 __device__ __forceinline__ unsigned long long gtimer() {
@@ -112,13 +113,11 @@ __device__ __forceinline__ void trace_mark(unsigned long long* tr, int it, int e
 // 5 pose solved.  All counters are monotonic over the launch (zeroed by
 // k_reg_init), so no CTA resets a word that another may still be reading;
 // every wait is bounded.
-// KEYS: the launch records each point's chosen node in a.keys (a one-round
-// launch before the source reorder).
 // MINB: co-resident CTAs per SM the build is register-limited for.  Two (128
 // registers) for sources of a few points per thread, where each round is a
 // latency chain and the node terms and the solve want the registers; three
 // (80) for large sources, whose descent is throughput-bound and gains from
-// the extra warps (a few bytes of spills, outside the descent).
+// the extra warps.
 template <int MINB>
 __global__ void __launch_bounds__(REG_THREADS, MINB) k_register(RegArgs a) {
     __shared__ float Rt_sm[12];
@@ -981,9 +980,8 @@ int hgmm_register_descent_impl(hgmm_tree* t, const float4* src, int64_t n64, con
 
 int hgmm_register_grid(int n_sm, int per_sm) {
     // static + dynamic shared memory exceeds the 48 KB default: opt in; the
-    // grid must be co-resident for both variants (KEYS) of the build asked
-    // for; 0 if that build does not reach per_sm CTAs per SM (the caller then
-    // keeps to the two-per-SM build)
+    // grid must be co-resident; 0 if the build asked for does not reach per_sm
+    // CTAs per SM (the caller then keeps to the two-per-SM build)
     if (per_sm != 2 && per_sm != 3) return 0;
     const void* fn = per_sm == 3 ? (const void*)k_register<3> : (const void*)k_register<2>;
     int k = 0;
