@@ -88,22 +88,6 @@ __device__ __forceinline__ double dot3(const double* a, const double* b) {
     return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
 
-// Gram-Schmidt of (a1, a2) into the columns b1, b2, b3 = b1 x b2.
-__device__ __forceinline__ void gram_schmidt(const double* a1, const double* a2, double* b1,
-                                             double* b2, double* b3, double* n1, double* dd,
-                                             double* n2) {
-    *n1 = sqrt(dot3(a1, a1));
-    const double i1 = *n1 > 0.0 ? 1.0 / *n1 : 0.0;
-    for (int i = 0; i < 3; ++i) b1[i] = a1[i] * i1;
-    *dd = dot3(b1, a2);
-    double u[3];
-    for (int i = 0; i < 3; ++i) u[i] = a2[i] - *dd * b1[i];
-    *n2 = sqrt(dot3(u, u));
-    const double i2 = *n2 > 0.0 ? 1.0 / *n2 : 0.0;
-    for (int i = 0; i < 3; ++i) b2[i] = u[i] * i2;
-    cross3(b1, b2, b3);
-}
-
 __device__ __forceinline__ void load_frame(const double* f, double* c, double& s, double* V) {
     for (int a = 0; a < 3; ++a) c[a] = f[a];
     s = f[3];
