@@ -296,6 +296,25 @@ k_flat_lse(const float4* __restrict__ pts, int n, const float* __restrict__ Rt,
             float hi[LSE_PPT];
 #pragma unroll
             for (int k = 0; k < LSE_PPT; ++k) hi[k] = -CUDART_INF_F;
+            if (c + 7 * LSE_SPLIT < cnt) {  // this phase's eight components are all there
+                float s[LSE_PPT][8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    ChildRegs cr;
+                    comp_from_smem(sc, c + u * LSE_SPLIT, cr);
+#pragma unroll
+                    for (int k = 0; k < LSE_PPT; ++k) {
+                        float ex, ey, ez;
+                        s[k][u] = child_score(cr, zx[k], zy[k], zz[k], ex, ey, ez);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < LSE_PPT; ++k) {
+                    hi[k] = chunk_max<8>(s[k]);
+                    lse_chunk<8>(s[k], hi[k], m[k], sum[k]);
+                }
+                c = cnt;
+            }
             for (; c < cnt; c += LSE_SPLIT) {
                 ChildRegs cr;
                 comp_from_smem(sc, c, cr);
@@ -307,6 +326,7 @@ k_flat_lse(const float4* __restrict__ pts, int n, const float* __restrict__ Rt,
                     lse_chunk<1>(s1, s1[0], m[k], sum[k]);
                 }
             }
+            __syncwarp();
             group_matters(group, hi);
         }
     }
