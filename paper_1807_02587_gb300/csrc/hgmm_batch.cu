@@ -250,7 +250,7 @@ __device__ void run_pair(const BatchArgs& a, const BatchWs& w, int cid, int pair
     // the cluster, and the staged levels' in every CTA's shared memory
     const int n_staged = n_nodes < STAGED_NODES ? n_nodes : STAGED_NODES;
     for (int g = 32 * (rank * wpb + warp); g < n_nodes; g += 32 * cs * wpb)
-        pack_blocks(w.rblk, w.est, g, n_nodes, n_nodes);
+        pack_blocks(w.rblk, w.est, g, n_nodes);
     cl.sync();
     for (int i = threadIdx.x; i < n_staged / 8 * BLOCK_F4; i += blockDim.x) sm_est[i] = __ldcg(w.rblk + i);
     const double ext = __ldcg(&w.root->extent) > 0.0 ? __ldcg(&w.root->extent) : 1.0;

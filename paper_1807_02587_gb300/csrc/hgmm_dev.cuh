@@ -1546,24 +1546,23 @@ static_assert(STAGED_NODES % 8 == 0, "whole sibling blocks are staged");
 // First float of a child's constants in its block; constant q is 2 q further.
 __device__ __forceinline__ int block_child(int c) { return 20 * (c >> 1) + (c & 1); }
 
-// The blocks of the 32 nodes from `base` on (a multiple of 32; those below n)
-// of a tree of n_nodes nodes, by a warp.  A node's stop flag is set where the
-// descent ends with it: its complexity is at most lambda_c (c.z), or it has
-// children and none of them is live.
-__device__ __forceinline__ void pack_blocks(float4* blocks, const NodeEst* est, int base, int n, int n_nodes) {
-    const int lane = threadIdx.x & 31;
-    const int g = base + lane;
-    const bool in = g < n;
-    const NodeEst* e = est + (in ? g : base);
-    const float4 a = __ldcg(&e->a), b = __ldcg(&e->b), c = __ldcg(&e->c);
-    bool stop = c.z != 0.f;
-    if (8 * int64_t(g) + 16 <= n_nodes) {  // the children of node g are 8 g + 8 ... 8 g + 15
-        const NodeEst* ch = est + 8 * g + 8;
-        float top = -CUDART_INF_F;
+// Whether node g of a tree of n_nodes nodes has children and none is live
+// (read through L2: est may have been written in this launch).
+__device__ __forceinline__ bool no_live_children(const NodeEst* est, int g, int n_nodes) {
+    if (8 * int64_t(g) + 16 > n_nodes) return false;
+    const NodeEst* ch = est + 8 * g + 8;  // the children of node g are 8 g + 8 ... 8 g + 15
+    float top = -CUDART_INF_F;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) top = fmaxf(top, __ldcg(&ch[k].a.w));
-        stop = stop || !(top > -CUDART_INF_F);
-    }
+    for (int k = 0; k < 8; ++k) top = fmaxf(top, __ldcg(&ch[k].a.w));
+    return !(top > -CUDART_INF_F);
+}
+
+// Node g's constants (a, b, c: its record) into its block, by all lanes of a
+// warp whose lane 0 holds a multiple of 32 (in: g is a node).  A node's stop
+// flag is set where the descent ends with it: its complexity is at most
+// lambda_c, or it has children and none of them is live.
+__device__ __forceinline__ void pack_node(float4* blocks, int g, bool in, const float4 a, const float4 b,
+                                          const float4 c, bool stop) {
     const unsigned stops = __ballot_sync(FULL, in && stop);
     if (!in) return;
     float* blk = reinterpret_cast<float*>(blocks + (g >> 3) * BLOCK_F4);
@@ -1578,7 +1577,17 @@ __device__ __forceinline__ void pack_blocks(float4* blocks, const NodeEst* est, 
     o[14] = b.w;
     o[16] = c.x;
     o[18] = c.y;
-    if ((g & 7) == 0) blk[80] = __uint_as_float((stops >> lane) & 0xFFu);
+    if ((g & 7) == 0) blk[80] = __uint_as_float((stops >> (threadIdx.x & 31)) & 0xFFu);
+}
+
+// The blocks of the 32 nodes from `base` on (a multiple of 32) of a tree of
+// n_nodes nodes whose records hold their stop flags (c.z), by a warp.
+__device__ __forceinline__ void pack_blocks(float4* blocks, const NodeEst* est, int base, int n_nodes) {
+    const int g = base + (threadIdx.x & 31);
+    const bool in = g < n_nodes;
+    const NodeEst* e = est + (in ? g : base);
+    const float4 a = __ldcg(&e->a), b = __ldcg(&e->b), c = __ldcg(&e->c);
+    pack_node(blocks, g, in, a, b, c, c.z != 0.f || (in && no_live_children(est, g, n_nodes)));
 }
 
 // Negated log2 scores u = -log2(pi N(z | child)) of a point over the eight

@@ -34,15 +34,20 @@ __global__ void k_reg_init(const double* __restrict__ T_init, int n_nodes, float
                            float* __restrict__ Rt, unsigned* __restrict__ bar,
                            double* __restrict__ obj) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n_nodes) {
+    const bool in = i < n_nodes;
+    float4 ea = make_float4(0.f, 0.f, 0.f, 0.f), eb = ea, ec = ea;
+    bool childless = false;
+    if (in) {
+        // the record, its children's and the complexity in one round trip
+        ea = __ldcg(&est[i].a);
+        eb = __ldcg(&est[i].b);
+        ec = __ldcg(&est[i].c);
+        const bool simple = stat[i].live && stat[i].complexity <= double(lam_c);
+        childless = no_live_children(est, i, n_nodes);
         for (int k = 0; k < 4 * ACC_REPLICAS; ++k) acc[4 * ACC_REPLICAS * int64_t(i) + k] = 0ull;
-        if (lam_c >= 0.f)
-            est[i].c.z = (stat[i].live && stat[i].complexity <= double(lam_c)) ? 1.f : 0.f;
+        if (lam_c >= 0.f) est[i].c.z = ec.z = simple ? 1.f : 0.f;
     }
-    // the descent's sibling blocks, from the records just written by this warp
-    __syncwarp();
-    const int w0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31;
-    if (w0 < n_nodes) pack_blocks(blocks, est, w0, n_nodes, n_nodes);
+    pack_node(blocks, i, in, ea, eb, ec, ec.z != 0.f || childless);  // the descent's sibling blocks
     if (i == 0) {
         for (int k = 0; k < 16; ++k) T[k] = T_init ? T_init[k] : ((k % 5 == 0) ? 1.0 : 0.0);
         for (int r = 0; r < 3; ++r) {
