@@ -293,9 +293,18 @@ k_mlp_backward(const __grid_constant__ CUtensorMap tmDY, const __grid_constant__
 // batch) cut into slices, and the bias gradients' partial column sums on
 // further CTAs.  Every operand is read where it lies, with M or N contiguous,
 // by TMA boxes of 64 columns x 64 rows; rows past the batch read zero.  A CTA
-// owns a 128 x 256 tile (128 x 64 for dW3) of one slice and writes it to its
-// slice's partials with one 1 KB bulk copy per row, staged through the operand
-// ring (rows 1040 bytes apart: no bank conflicts).
+// owns a tile of one slice (128 x 256 of dW1, 128 x 128 of dW2, 128 x 64 of
+// dW3) and writes it to its slice's partials with one bulk copy per row, staged
+// through the operand ring (rows 1040 bytes apart: no bank conflicts).
+//
+// The tensor core rounds its FP32 sums towards zero at every step, so a sum's
+// error grows with the number of rows that one accumulator takes.  A slice is
+// therefore cut once more, into as many accumulators as TMEM's 512 columns
+// hold (two for dW1, four for dW2 and dW3), added in FP32 when the tile is
+// read back: at most 1/16 (dW1) or 1/32 of the batch per accumulator.  Error of
+// dW1 / dW2 / dW3 against float64 on operands that BF16 holds exactly, 4,096
+// rows: 2.0e-7 / 1.0e-7 / 1.2e-7, with one accumulator per slice 4.6e-7 / 4.4e-7 /
+// 5.2e-7 (and 1 us less for a step of 1,024 to 4,096 rows: 57.3 against 58.4).
 constexpr int WG_THREADS = 256;
 constexpr int WG_STAGES = 4;
 constexpr int WG_BOX = 64 * 128;             // 64 rows x 64 BF16
@@ -305,12 +314,15 @@ constexpr int WG_SMEM = WG_STAGES * WG_STAGE + 1024;
 static_assert(OFF_B1 % 4 == 0 && OFF_W2 % 4 == 0 && OFF_B2 % 4 == 0 && OFF_W3 % 4 == 0 && OFF_B3 % 4 == 0,
               "whole vectors of weights");
 static_assert(128 * WG_ROW <= WG_STAGES * WG_STAGE, "staging inside the ring");
-constexpr int WG_TILES = 2 * (IN / 256) + 2 + 2;
+constexpr int WG_TILES1 = 2 * (IN / 256), WG_TILES2 = 2 * (HID / 128);
+constexpr int WG_TILES = WG_TILES1 + WG_TILES2 + 2;
 constexpr int WG_MAX_SLICES = 8;
+constexpr int WG_ACC1 = 2, WG_ACC23 = 4;     // accumulators per CTA of dW1; of dW2 and dW3
+static_assert(WG_ACC1 * 256 <= 512 && WG_ACC23 * 128 <= 512, "TMEM columns");
 constexpr int64_t WS_STRIDE = (N_PARAMS + 3) / 4 * 4;
 
 // K slices of a batch: 64-row chunks per slice (the tiles times the slices
-// are at most 112 CTAs: one wave beside the column sums).
+// are at most 128 CTAs: one wave beside the column sums).
 inline int wg_chunks(int batch) { return ((batch + 63) / 64 + WG_MAX_SLICES - 1) / WG_MAX_SLICES; }
 inline int wg_slices(int batch) {
     const int c = wg_chunks(batch);
@@ -353,18 +365,21 @@ k_mlp_wgrad(const __grid_constant__ CUtensorMap tmZ1, const __grid_constant__ CU
     const uint32_t base = (tc::smem_u32(wg_raw) + 1023u) & ~1023u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tile = blockIdx.x / slices, slice = blockIdx.x % slices;
-    constexpr int T1 = 2 * (IN / 256);
-    // tile -> product, first column of A (rows of D) and of B (columns of D)
-    const int which = tile < T1 ? 0 : (tile < T1 + 2 ? 1 : 2);
-    const int m0 = 128 * (tile & 1), n0 = which == 0 ? 256 * (tile >> 1) : 0;
+    // tile -> product, first column of A (rows of D) and of B (columns of D), columns
+    const int which = tile < WG_TILES1 ? 0 : (tile < WG_TILES1 + WG_TILES2 ? 1 : 2);
+    const int m0 = 128 * (tile & 1);
+    const int n0 = which == 0 ? 256 * (tile >> 1) : (which == 1 ? 128 * ((tile - WG_TILES1) >> 1) : 0);
+    const int width = which == 0 ? 256 : (which == 1 ? 128 : 64);
+    const int nb = width / 64;
     const void* ta = which == 0 ? &tmZ1 : (which == 1 ? &tmZ2 : &tmH2);
     const void* tb = which == 0 ? &tmX : (which == 1 ? &tmH1 : &tmDY);
-    const int nb = which == 2 ? 1 : 4;
-    const uint32_t idesc =
-        (which == 2 ? tc::idesc_bf16_f32(128, 64) : tc::idesc_bf16_f32(128, 256)) | (1u << 15) | (1u << 16);
+    const uint32_t idesc = tc::idesc_bf16_f32(128, width) | (1u << 15) | (1u << 16);
     const int k0 = slice * chunks, nk = min(chunks, (batch + 63) / 64 - k0);
+    // chunks per accumulator, and accumulators in use
+    const int per_acc = (chunks + (which == 0 ? WG_ACC1 : WG_ACC23) - 1) / (which == 0 ? WG_ACC1 : WG_ACC23);
+    const int accs = (nk + per_acc - 1) / per_acc;
     if (warp == 4) {
-        tc::tmem_alloc(&tmem_slot, 256);
+        tc::tmem_alloc(&tmem_slot, 512);
         tc::tmem_relinquish();
     }
     if (threadIdx.x == 160) {
@@ -402,10 +417,13 @@ k_mlp_wgrad(const __grid_constant__ CUtensorMap tmZ1, const __grid_constant__ CU
             tc::fence_after_sync();
             const uint32_t sa = base + st * WG_STAGE;
             const uint64_t da = smem_desc_mn(sa, WG_BOX), db = smem_desc_mn(sa + 2 * WG_BOX, WG_BOX);
+            const int acc = kt / per_acc;
+            const bool first = kt == acc * per_acc;
             if (lead) {
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)  // 16 rows of 128 bytes
-                    tc::mma_bf16(tmem, da + 128 * kk, db + 128 * kk, idesc, (kt | kk) != 0 ? 1u : 0u);
+                    tc::mma_bf16(tmem + uint32_t(acc * width), da + 128 * kk, db + 128 * kk, idesc,
+                                 !first || kk != 0 ? 1u : 0u);
                 tc::mma_commit(&empty[st]);
             }
             __syncwarp();
@@ -421,14 +439,27 @@ k_mlp_wgrad(const __grid_constant__ CUtensorMap tmZ1, const __grid_constant__ CU
             if (which == 2) {
                 float v[16];
                 tc::tmem_ld16(tacc, v);
+                for (int q = 1; q < accs; ++q) {
+                    float x[16];
+                    tc::tmem_ld16(tacc + uint32_t(q * width), x);
+#pragma unroll
+                    for (int o = 0; o < OUT; ++o) v[o] += x[o];
+                }
 #pragma unroll
                 for (int o = 0; o < OUT; ++o) out[OFF_W3 + o * HID + m] = v[o];
             } else {
                 const uint32_t row = base + uint32_t(r * WG_ROW);
 #pragma unroll 1
-                for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < nb; ++c) {
                     float v[64];
                     tc::tmem_ld64(tacc + uint32_t(64 * c), v);
+#pragma unroll 1
+                    for (int q = 1; q < accs; ++q) {
+                        float x[64];
+                        tc::tmem_ld64(tacc + uint32_t(q * width + 64 * c), x);
+#pragma unroll
+                        for (int o = 0; o < 64; ++o) v[o] += x[o];
+                    }
 #pragma unroll
                     for (int q = 0; q < 16; ++q)
                         asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
@@ -436,7 +467,8 @@ k_mlp_wgrad(const __grid_constant__ CUtensorMap tmZ1, const __grid_constant__ CU
                                         "f"(v[4 * q + 2]), "f"(v[4 * q + 3]) : "memory");
                 }
                 tc::fence_proxy_async();
-                bulk_s2g(out + (which == 0 ? OFF_W1 + int64_t(m) * IN + n0 : OFF_W2 + int64_t(m) * HID), row, 1024u);
+                bulk_s2g(out + (which == 0 ? OFF_W1 + int64_t(m) * IN + n0 : OFF_W2 + int64_t(m) * HID + n0), row,
+                         uint32_t(4 * width));
                 bulk_commit();
                 bulk_wait();
             }
@@ -452,7 +484,7 @@ k_mlp_wgrad(const __grid_constant__ CUtensorMap tmZ1, const __grid_constant__ CU
     if (threadIdx.x == 0 && *(volatile int*)&fail) atomicOr(err, ERR_TIMEOUT);
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 4) tc::tmem_dealloc(tmem, 256);
+    if (warp == 4) tc::tmem_dealloc(tmem, 512);
 }
 
 // ------------------------------------------------------- gradients and update
