@@ -36,9 +36,9 @@
  *     graph it replays), so build + register can be captured in a CUDA graph
  *     (the registration is one cooperative launch, after an on-device reorder
  *     for sources of 2^20 points or more).
- *   - Device-side waits are bounded: the registration's arrival and partial-
- *     count waits give up after about a second, record HGMM_ETIMEOUT and
- *     return.
+ *   - Device-side waits are bounded: the waits of the build's cooperative
+ *     launch and the registration's arrival and partial-count waits give up
+ *     after about a second, record HGMM_ETIMEOUT and return.
  */
 #ifndef HGMM_H
 #define HGMM_H
@@ -117,6 +117,13 @@ void hgmm_tree_destroy(hgmm_tree* t);
  * levels (level l holds 8^(l+1) nodes) and J components per node (must be
  * 8).  p may be NULL for the defaults.  Enqueued on `stream`; non-finite
  * input is reported by hgmm_sync as HGMM_ENONFINITE.
+ * Clouds of up to about 400,000 points (precision 0) build their first four
+ * levels in one cooperative launch, which waits until the device holds all of
+ * its CTAs at once.  Where the device refuses that (a context or stream that
+ * owns too few SMs), and for larger clouds and precision 1, every level is a
+ * sequence of plain launches; the two orders of summation agree to about
+ * 1e-14.  A refusal inside a stream capture ends the capture, as it does for
+ * hgmm_register.
  * Errors: HGMM_EINVAL (n < 8, J != 8, depth not in [1, max_depth],
  * unaligned pointer), HGMM_ECAPACITY, HGMM_ECUDA. */
 int hgmm_build(hgmm_tree* t, const float* d_points, int64_t n, int32_t depth,
@@ -239,6 +246,13 @@ int hgmm_debug_reg_moments(hgmm_tree* t, double* h_m, int64_t cap);
  * returns normally (no fault, no hang): the next hgmm_sync returns
  * HGMM_ETIMEOUT and the tree stays usable.  Enqueued on `stream`. */
 int hgmm_debug_barrier_timeout(hgmm_tree* t, int64_t spin_limit, void* stream);
+
+/* Fallback check: while enabled, the build's cooperative launch (clouds of up
+ * to about 400,000 points, precision 0) asks for more CTAs than the device can
+ * hold, so that the runtime refuses it (nothing runs, no error remains) and
+ * hgmm_build takes the level-wide launches, as it does in a context that owns
+ * too few SMs. */
+int hgmm_debug_refuse_build(hgmm_tree* t, int32_t enable);
 
 /* ---- per-kernel timing (tracing) ----
  * hgmm_profile(t, 1) clears and starts recording a CUDA event pair around

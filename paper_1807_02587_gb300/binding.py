@@ -86,6 +86,7 @@ def _load():
         "hgmm_node_count": (i64, [i32]),
         "hgmm_profile": (ctypes.c_int, [vp, i32]),
         "hgmm_debug_barrier_timeout": (ctypes.c_int, [vp, i64, vp]),
+        "hgmm_debug_refuse_build": (ctypes.c_int, [vp, i32]),
         "hgmm_trace": (ctypes.c_int, [vp, i32]),
         "hgmm_fit_level0_noalloc": (ctypes.c_int, [vp, i64, P(hgmm_params), vp, vp]),
         "hgmm_batch_create": (ctypes.c_int, [i64, i32, i32, P(vp)]),
@@ -315,6 +316,10 @@ HGMM_PROF_KERNELS = 16
 def hgmm_debug_barrier_timeout(h, spin_limit: int, stream=None) -> None:
     _check(_lib.hgmm_debug_barrier_timeout(h, int(spin_limit), _stream_ptr(stream)),
            "hgmm_debug_barrier_timeout")
+
+
+def hgmm_debug_refuse_build(h, enable: bool) -> None:
+    _check(_lib.hgmm_debug_refuse_build(h, 1 if enable else 0), "hgmm_debug_refuse_build")
 
 
 def hgmm_fit_level0_noalloc(points, prm: hgmm_params | None = None, stream=None, out=None):

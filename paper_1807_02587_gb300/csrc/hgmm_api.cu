@@ -429,6 +429,12 @@ int hgmm_debug_barrier_timeout(hgmm_tree* t, int64_t spin_limit, void* stream) {
     return hgmm_barrier_timeout_probe_impl(t, spin_limit, static_cast<cudaStream_t>(stream));
 }
 
+int hgmm_debug_refuse_build(hgmm_tree* t, int32_t enable) {
+    if (!t) return HGMM_EINVAL;
+    t->levels_refuse = enable != 0;
+    return HGMM_OK;
+}
+
 int hgmm_trace(hgmm_tree* t, int32_t enable) {
     if (!t) return HGMM_EINVAL;
     t->trace_on = enable != 0;

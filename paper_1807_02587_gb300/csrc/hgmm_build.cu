@@ -742,7 +742,7 @@ int hgmm_build_impl(hgmm_tree* t, const float4* pts, int64_t n64, int depth,
     const bool comp = p.precision == 0;
     // clouds whose points fit the CTAs' shared memory: the first levels (all
     // of them up to depth 4) in one launch
-    const int taken = comp && t->levels_ok ? levels_taken(n64, depth, G) : 0;
+    int taken = comp && t->levels_ok ? levels_taken(n64, depth, G) : 0;
     if (taken > 0) {
         LevelsArgs a;
         a.pts = pts;
@@ -771,7 +771,15 @@ int hgmm_build_impl(hgmm_tree* t, const float4* pts, int64_t n64, int depth,
         a.cnt = t->lv_cnt;
         a.status = t->status;
         ProfScope ps_(t, K_LEVELS, s);
-        if (int rc = levels_launch(a, G, s)) return rc;
+        const int rc = levels_launch(a, G, t->levels_refuse, s);
+        if (rc == LEVELS_REFUSED) {
+            ps_.drop = true;
+            taken = 0;
+        } else if (rc) {
+            return rc;
+        }
+    }
+    if (taken > 0) {
         if (taken == depth || (p.debug_stop_level > 0 && p.debug_stop_level <= taken)) return HGMM_OK;
         cur = t->pts[(taken - 1) & 1];
         perm_prev = t->perm[taken - 1];

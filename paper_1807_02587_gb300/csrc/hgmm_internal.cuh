@@ -145,6 +145,7 @@ struct hgmm_tree {
     int est_grid = 0;   // CTAs of the persistent build E-step
     int em_coop_grid = 0;  // co-resident CTAs of the cooperative per-level EM kernel (0: unavailable)
     bool levels_ok = false;  // the one-launch build of the levels fits on the device
+    bool levels_refuse = false;  // checking aid: its launch asks for more CTAs than fit
     int reg_grid = 0;       // CTAs of the registration kernel, two per SM
     bool refine_ok = false;  // the source reorder's shared memory fits on the device
     int reg_grid_wide = 0;  // three per SM, for large sources (0: not co-resident)
@@ -219,12 +220,16 @@ struct ProfScope {
     int id;
     cudaStream_t s;
     cudaEvent_t a = nullptr, b = nullptr;
+    bool drop = false;  // the launch was refused: record nothing
     ProfScope(hgmm_tree* t_, int id_, cudaStream_t s_) : t(t_), id(id_), s(s_) {
         if (t->prof_on && cudaEventCreate(&a) == cudaSuccess && cudaEventCreate(&b) == cudaSuccess)
             cudaEventRecord(a, s);
     }
     ~ProfScope() {
-        if (a && b) {
+        if (a && b && drop) {
+            cudaEventDestroy(a);
+            cudaEventDestroy(b);
+        } else if (a && b) {
             cudaEventRecord(b, s);
             t->prof.push_back({id, a, b});
         }

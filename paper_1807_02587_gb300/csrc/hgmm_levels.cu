@@ -652,7 +652,7 @@ int levels_taken(int64_t n, int depth, int est_grid) {
     return L;
 }
 
-int levels_launch(LevelsArgs& a, int est_grid, cudaStream_t s) {
+int levels_launch(LevelsArgs& a, int est_grid, bool refuse, cudaStream_t s) {
     // CTAs: as many as a level has chunks or runs, at most the E-step's grid
     // (a barrier of fewer CTAs is cheaper); one chunk of the level-wide
     // launches per CTA
@@ -665,13 +665,18 @@ int levels_launch(LevelsArgs& a, int est_grid, cudaStream_t s) {
         many = many || local;
         want = std::max(want, local ? a.n / LV_RUN_POINTS + n_par : items + n_par - 1);
     }
-    const int grid = int(std::min<int64_t>(want, est_grid));
+    const int grid = refuse ? 64 * est_grid : int(std::min<int64_t>(want, est_grid));
     a.n_chunks = est_grid;
     if (cudaMemsetAsync(a.cnt, 0, size_t(levels_counters()) * sizeof(unsigned), s) != cudaSuccess) return HGMM_ECUDA;
     void* args[] = {&a};
     const size_t smem = (many ? LV_LOCAL_UNITS : 1) * LV_RUN_POINTS * sizeof(float4);
-    if (cudaLaunchCooperativeKernel((const void*)k_build_levels, dim3(grid), dim3(LV_THREADS), args, smem, s) !=
-        cudaSuccess) {
+    const cudaError_t e =
+        cudaLaunchCooperativeKernel((const void*)k_build_levels, dim3(grid), dim3(LV_THREADS), args, smem, s);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        return LEVELS_REFUSED;
+    }
+    if (e != cudaSuccess) {
         fprintf(stderr, "hgmm: cooperative build launch failed: %s\n", cudaGetErrorString(cudaGetLastError()));
         return HGMM_ECUDA;
     }

@@ -42,6 +42,11 @@ int64_t levels_slots(int64_t n);
 int levels_counters();
 bool levels_smem_attr();
 int levels_taken(int64_t n, int depth, int est_grid);
-int levels_launch(LevelsArgs& a, int est_grid, cudaStream_t s);
+// HGMM_OK, HGMM_ECUDA, or LEVELS_REFUSED: the device cannot hold the launch's
+// CTAs at once (a context that owns part of its SMs), nothing has run, and the
+// level-wide launches, which need no co-residency, build the tree.  refuse:
+// checking aid, asks for more CTAs than any device holds.
+constexpr int LEVELS_REFUSED = 1;
+int levels_launch(LevelsArgs& a, int est_grid, bool refuse, cudaStream_t s);
 
 }  // namespace hgmm
