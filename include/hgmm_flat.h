@@ -34,8 +34,12 @@ typedef struct hgmm_flat hgmm_flat;
 
 /* A flat model for clouds of up to max_points points and up to
  * max_components components, on the current device; owns all of its
- * scratch (no allocation after this call).  Errors: HGMM_EINVAL,
- * HGMM_ENOMEM. */
+ * scratch (no allocation after this call).  Device memory: per component
+ * 0.4 KB, per point 4 bytes, 13 MB of partial sums, and a table of 4 bytes per
+ * point and 32 components, at most 256 MB, that lets the calls it is large
+ * enough for skip components far from a point (the same results; without room
+ * for the table, or in larger calls, every component is computed).  Errors:
+ * HGMM_EINVAL, HGMM_ENOMEM. */
 int hgmm_flat_create(int64_t max_points, int32_t max_components, hgmm_flat** out);
 void hgmm_flat_destroy(hgmm_flat* f);
 

@@ -23,6 +23,7 @@
 //                   sums those in a fixed order and one of its warps solves in
 //                   FP64 and updates T <- dT T (warp_solve_update).
 // Every sum has a fixed order, so a registration is bit-reproducible.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 
@@ -53,7 +54,10 @@ constexpr int LSE_POINTS = LSE_THREADS / LSE_SPLIT * LSE_PPT;  // points per CTA
 constexpr int LSE_TILE = 512;    // components staged per pass
 constexpr int GROUP = 8 * LSE_SPLIT;  // components of one chunk of a point group's lanes, and of a warp of moments
 static_assert(GROUP == 32 && LSE_TILE % GROUP == 0, "whole groups");
-constexpr size_t GMAX_KEPT = size_t(1) << 30;  // largest table of group maxima (4 GB)
+// Largest table of group maxima: 2^26 floats (256 MB), 456,000 points and the
+// 4,680 candidates of a depth-4 tree.  A call that needs more computes every
+// pair (the same bits, 1.2 times the time).
+constexpr size_t GMAX_KEPT = size_t(1) << 26;
 constexpr int MOM_THREADS = 256; // one component per thread
 constexpr int MOM_STAGE = 2048;  // points staged per pass (a slice of an ordinary cloud)
 constexpr int NMOM_MAX = 10;
@@ -697,7 +701,8 @@ struct hgmm_flat {
     int* meta = nullptr;
     double* eps = nullptr;
     float* lse = nullptr;
-    float* gmax = nullptr;  // per group of GROUP components and point: the largest score (or null)
+    float* gmax = nullptr;  // per group of GROUP components and point: the largest score
+    size_t gmax_cap = 0;    // ... its size (0: none)
     int* slot = nullptr;    // from the tree: component of each node
     double* wt = nullptr;   // ... and its path product; the last: their sum
     float2* part = nullptr;
@@ -740,6 +745,11 @@ int moment_grid(const hgmm_flat* f) {
     return tiles > f->max_ctas ? tiles : f->max_ctas;
 }
 
+// The table of group maxima for a call on n points, or null if it does not fit.
+float* group_maxima(const hgmm_flat* f, int64_t n) {
+    return size_t(n) * size_t((f->jcap + GROUP - 1) / GROUP) <= f->gmax_cap ? f->gmax : nullptr;
+}
+
 int launched() { return cudaGetLastError() == cudaSuccess ? HGMM_OK : HGMM_ECUDA; }
 
 }  // namespace
@@ -757,12 +767,6 @@ int hgmm_flat_create(int64_t max_points, int32_t max_components, hgmm_flat** out
     f->max_ctas = 4 * (f->n_sm > 0 ? f->n_sm : 1);
     const int tiles_max = (max_components + MOM_THREADS - 1) / MOM_THREADS;
     const size_t part_ctas = size_t(f->max_ctas > tiles_max ? f->max_ctas : tiles_max);
-    // without the group maxima (too large, or no memory for them) every pair is computed
-    const size_t groups = size_t(max_points) * size_t((max_components + GROUP - 1) / GROUP);
-    if (groups > GMAX_KEPT || !falloc(&f->gmax, groups)) {
-        f->gmax = nullptr;
-        cudaGetLastError();
-    }
     const bool good = falloc(&f->comp, max_components) && falloc(&f->est, max_components) &&
                       falloc(&f->rterm, 3 * size_t(max_components)) && falloc(&f->meta, 4) &&
                       falloc(&f->eps, 1) && falloc(&f->lse, size_t(max_points)) &&
@@ -776,6 +780,13 @@ int hgmm_flat_create(int64_t max_points, int32_t max_components, hgmm_flat** out
         free_flat(f);
         cudaGetLastError();
         return HGMM_ENOMEM;
+    }
+    // last: the object works without it
+    f->gmax_cap = std::min(GMAX_KEPT, size_t(max_points) * size_t((max_components + GROUP - 1) / GROUP));
+    if (!falloc(&f->gmax, f->gmax_cap)) {
+        f->gmax = nullptr;
+        f->gmax_cap = 0;
+        cudaGetLastError();
     }
     *out = f;
     return HGMM_OK;
@@ -810,11 +821,12 @@ int hgmm_flat_fit(hgmm_flat* f, const float* d_points, int64_t n, int32_t em_ite
     const int rgrid = (f->jcap + RED_COMPS - 1) / RED_COMPS;
     const int mgrid = moment_grid(f);
     const int lse_grid = int((n + LSE_POINTS - 1) / LSE_POINTS);
+    float* gmax = group_maxima(f, n);
     for (int it = 0; it < em_iters; ++it) {
-        k_flat_lse<false><<<lse_grid, LSE_THREADS, 0, s>>>(pts, int(n), nullptr, f->est, f->meta, f->lse, f->gmax, n,
+        k_flat_lse<false><<<lse_grid, LSE_THREADS, 0, s>>>(pts, int(n), nullptr, f->est, f->meta, f->lse, gmax, n,
                                                            f->status);
         k_flat_moments<10, false><<<mgrid, MOM_THREADS, 0, s>>>(pts, int(n), nullptr, f->lse, f->est, f->meta,
-                                                               mgrid, f->gmax, n, f->part);
+                                                               mgrid, gmax, n, f->part);
         k_flat_mstep<<<rgrid, MOM_THREADS, 0, s>>>(f->part, mgrid, f->meta, int(n), n_min, f->eps, f->comp,
                                                    f->est, f->status);
     }
@@ -831,12 +843,13 @@ int hgmm_flat_register(hgmm_flat* f, const float* d_src, int64_t n, const double
     const int rgrid = (f->jcap + RED_COMPS - 1) / RED_COMPS;
     const int mgrid = moment_grid(f);
     const int lse_grid = int((n + LSE_POINTS - 1) / LSE_POINTS);
+    float* gmax = group_maxima(f, n);
     k_flat_reg_init<<<1, 32, 0, s>>>(d_T_init, f->T, f->Rt, f->obj);
     for (int it = 0; it < iters; ++it) {
-        k_flat_lse<true><<<lse_grid, LSE_THREADS, 0, s>>>(pts, int(n), f->Rt, f->est, f->meta, f->lse, f->gmax, n,
+        k_flat_lse<true><<<lse_grid, LSE_THREADS, 0, s>>>(pts, int(n), f->Rt, f->est, f->meta, f->lse, gmax, n,
                                                           f->status);
         k_flat_moments<4, true><<<mgrid, MOM_THREADS, 0, s>>>(pts, int(n), f->Rt, f->lse, f->est, f->meta, mgrid,
-                                                             f->gmax, n, f->part);
+                                                             gmax, n, f->part);
         k_flat_terms<<<rgrid, MOM_THREADS, 0, s>>>(f->part, mgrid, f->meta, f->est, f->rterm, int(n),
                                                    f->tpart, f->dbg, reinterpret_cast<unsigned*>(f->meta + 2), it,
                                                    f->T, f->Rt, d_T_hist, f->obj, f->status);
