@@ -94,10 +94,34 @@ __device__ __forceinline__ void load_frame(const double* f, double* c, double& s
     for (int v = 0; v < 9; ++v) V[v] = f[4 + v];
 }
 
+// Gram-Schmidt of a network output's first six values into the columns b1, b2,
+// b3 = b1 x b2 of R'.
+__device__ __forceinline__ void decode_basis(const float* y, double* b1, double* b2, double* b3) {
+    double a1[3], a2[3], u[3];
+    for (int k = 0; k < 3; ++k) {
+        a1[k] = y[k];
+        a2[k] = y[3 + k];
+    }
+    const double s1 = dot3(a1, a1);
+    const double i1 = s1 > 0.0 ? rsqrt_f64(s1) : 0.0;
+    for (int k = 0; k < 3; ++k) b1[k] = a1[k] * i1;
+    const double dd = dot3(b1, a2);
+    for (int k = 0; k < 3; ++k) u[k] = a2[k] - dd * b1[k];
+    const double s2 = dot3(u, u);
+    const double i2 = s2 > 0.0 ? rsqrt_f64(s2) : 0.0;
+    for (int k = 0; k < 3; ++k) b2[k] = u[k] * i2;
+    cross3(b1, b2, b3);
+}
+
 // Sixteen lanes per pair, lane (r, c) = entry (r, c) of T: a handful of pairs
 // is one dependent FP64 chain, so the entries share its instructions (one
-// pair: 6.8 us with one thread, 4.6 here).
+// pair: 6.8 us with one thread, 4.6 here).  The chain before the entries is
+// run sixteen times over, so from a few thousand pairs on, where the FP64 pipes
+// are busy, k_decode_many's one thread per pair is faster: calls of 4,096 /
+// 8,192 / 65,536 pairs take 12.8 / 21 / 118 us here, 9.5 / 9.5 / 24 there; at
+// 2,048 both take the 9.2 of the launch.
 constexpr int DECODE_THREADS = 128;
+constexpr int DECODE_FEW = 2048;
 __global__ void __launch_bounds__(DECODE_THREADS)
 k_decode(const float* __restrict__ Y, const double* __restrict__ F, int n, double* __restrict__ T) {
     const int64_t i = (int64_t(blockIdx.x) * DECODE_THREADS + threadIdx.x) >> 4;
@@ -108,22 +132,8 @@ k_decode(const float* __restrict__ Y, const double* __restrict__ F, int n, doubl
     load_frame(F + 32 * i, cs, ss, Vs);
     load_frame(F + 32 * i + 16, ct, st, Vt);
     const float* y = Y + i * OUT;
-    double a1[3], a2[3], b1[3], b2[3], b3[3];
-    for (int k = 0; k < 3; ++k) {
-        a1[k] = y[k];
-        a2[k] = y[3 + k];
-    }
-    // Gram-Schmidt of (a1, a2) into the columns b1, b2, b3 = b1 x b2
-    const double s1 = dot3(a1, a1);
-    const double i1 = s1 > 0.0 ? rsqrt_f64(s1) : 0.0;
-    for (int k = 0; k < 3; ++k) b1[k] = a1[k] * i1;
-    const double dd = dot3(b1, a2);
-    double u[3];
-    for (int k = 0; k < 3; ++k) u[k] = a2[k] - dd * b1[k];
-    const double s2 = dot3(u, u);
-    const double i2 = s2 > 0.0 ? rsqrt_f64(s2) : 0.0;
-    for (int k = 0; k < 3; ++k) b2[k] = u[k] * i2;
-    cross3(b1, b2, b3);
+    double b1[3], b2[3], b3[3];
+    decode_basis(y, b1, b2, b3);
     // R' (columns b1..b3); A = Vt R', R = A Vs^T: lane (r, c) forms entry (r,
     // c) of both; lane (r, 3) the translation's Vt y_t instead of A's entry
     const double vt0 = r == 0 ? Vt[0] : (r == 1 ? Vt[3] : Vt[6]);
@@ -143,6 +153,28 @@ k_decode(const float* __restrict__ Y, const double* __restrict__ F, int n, doubl
     const double ctr = r == 0 ? ct[0] : (r == 1 ? ct[1] : ct[2]);
     const double t = ctr + st * Arc - (R0 * cs[0] + R1 * cs[1] + R2 * cs[2]);
     T[16 * i + e] = e >= 12 ? (e == 15 ? 1.0 : 0.0) : (c == 3 ? t : Rrc);
+}
+
+// The same, one thread per pair.
+__global__ void __launch_bounds__(DECODE_THREADS)
+k_decode_many(const float* __restrict__ Y, const double* __restrict__ F, int n, double* __restrict__ T) {
+    const int64_t i = int64_t(blockIdx.x) * DECODE_THREADS + threadIdx.x;
+    if (i >= n) return;
+    double cs[3], ct[3], Vs[9], Vt[9], ss, st, b[3][3];
+    load_frame(F + 32 * i, cs, ss, Vs);
+    load_frame(F + 32 * i + 16, ct, st, Vt);
+    const float* y = Y + i * OUT;
+    decode_basis(y, b[0], b[1], b[2]);
+    double* o = T + 16 * i;
+    for (int r = 0; r < 3; ++r) {
+        double A[3], R[3];
+        for (int c = 0; c < 3; ++c) A[c] = Vt[3 * r] * b[c][0] + Vt[3 * r + 1] * b[c][1] + Vt[3 * r + 2] * b[c][2];
+        for (int c = 0; c < 3; ++c) R[c] = A[0] * Vs[3 * c] + A[1] * Vs[3 * c + 1] + A[2] * Vs[3 * c + 2];
+        const double vt = Vt[3 * r] * y[6] + Vt[3 * r + 1] * y[7] + Vt[3 * r + 2] * y[8];
+        for (int c = 0; c < 3; ++c) o[4 * r + c] = R[c];
+        o[4 * r + 3] = ct[r] + st * vt - (R[0] * cs[0] + R[1] * cs[1] + R[2] * cs[2]);
+    }
+    for (int c = 0; c < 4; ++c) o[12 + c] = c == 3 ? 1.0 : 0.0;
 }
 
 __global__ void k_encode(const double* __restrict__ T, const double* __restrict__ F, int n,
@@ -905,8 +937,12 @@ int hgmm_propose(hgmm_tree* tgt, hgmm_tree* src, hgmm_mlp* m, void* stream, doub
 
 int hgmm_pose_decode(const float* d_y, const double* d_frames, int32_t n, double* d_T, void* stream) {
     if (!d_y || !d_frames || !d_T || n < 1) return HGMM_EINVAL;
-    k_decode<<<(n + DECODE_THREADS / 16 - 1) / (DECODE_THREADS / 16), DECODE_THREADS, 0,
-               static_cast<cudaStream_t>(stream)>>>(d_y, d_frames, n, d_T);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (n <= DECODE_FEW)
+        k_decode<<<(n + DECODE_THREADS / 16 - 1) / (DECODE_THREADS / 16), DECODE_THREADS, 0, s>>>(d_y, d_frames, n,
+                                                                                                  d_T);
+    else
+        k_decode_many<<<(n + DECODE_THREADS - 1) / DECODE_THREADS, DECODE_THREADS, 0, s>>>(d_y, d_frames, n, d_T);
     return cudaGetLastError() == cudaSuccess ? HGMM_OK : HGMM_ECUDA;
 }
 
