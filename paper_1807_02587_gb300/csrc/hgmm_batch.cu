@@ -166,10 +166,11 @@ __device__ void sort_source_by_node(const float4* __restrict__ src, int n, int n
 }
 
 // The registration's descent as a function of its own (see called_estep_items).
+template <bool STAGED>
 __device__ __noinline__ void called_descent(const float4* src, int n, const float4* blocks, const float4* sm_blocks,
                                             int depth, const float* Rt, float qscale, unsigned long long* acc, int cta,
                                             int ncta, unsigned long long* hist, uint32_t* key_out) {
-    descend_points(src, n, blocks, sm_blocks, depth, Rt, qscale, acc, cta, ncta, hist, key_out);
+    descend_points<STAGED>(src, n, blocks, sm_blocks, depth, Rt, qscale, acc, cta, ncta, hist, key_out);
 }
 
 // One pair, run by all CTAs of this cluster.
@@ -274,8 +275,11 @@ __device__ void run_pair(const BatchArgs& a, const BatchWs& w, int cid, int pair
             for (int i = threadIdx.x; i < n_staged / 8 * BLOCK_F4; i += blockDim.x) sm_est[i] = __ldcg(w.rblk + i);
         }
         __syncthreads();
-        called_descent(src, n_s, w.rblk, sm_est, depth, rgs.Rt, qscale, w.acc, rank, cs, hist,
-                       sort_src && (it == 0 || it == resort - 1) ? w.codes : nullptr);
+        uint32_t* const keys = sort_src && (it == 0 || it == resort - 1) ? w.codes : nullptr;
+        if (n_nodes <= STAGED_NODES)
+            called_descent<true>(src, n_s, w.rblk, sm_est, depth, rgs.Rt, qscale, w.acc, rank, cs, hist, keys);
+        else
+            called_descent<false>(src, n_s, w.rblk, sm_est, depth, rgs.Rt, qscale, w.acc, rank, cs, hist, keys);
         __syncthreads();
         flush_node_hist(hist, n_staged, w.acc);
         cl.sync();

@@ -1611,10 +1611,12 @@ __device__ __forceinline__ void block_scores(const float4* blk, Load load, float
 }
 
 // The scores below the node whose first child is `first`; returns the stop
-// flags.  Staged levels read shared memory, deeper levels the cache.
+// flags.  Staged levels read shared memory, deeper levels the cache.  STAGED:
+// every level is staged.
+template <bool STAGED>
 __device__ __forceinline__ unsigned child_scores(const float4* blocks, const float4* sm_blocks, int first, float x,
                                                  float y, float z, float2 (&u)[4]) {
-    if (first < STAGED_NODES) {
+    if (STAGED || first < STAGED_NODES) {
         const float4* blk = sm_blocks + (first >> 3) * BLOCK_F4;
         block_scores(blk, [](const float4* p) { return *p; }, x, y, z, u);
         return __float_as_uint(blk[BLOCK_F4 - 1].x);
@@ -1712,6 +1714,12 @@ __device__ __forceinline__ void add_moments(int chosen, long long (&q)[4], unsig
 // Two points per lane that share a block's loads were tried: 16M points in
 // node order 459 us a round against 466, but 11.5 against 9.9 us at 4,000
 // points and 1,195 against 805 for a round in random order.
+// STAGED: a tree whose levels are all staged (up to depth 3).  Without it such
+// trees pay for the branch to the cached levels, where a small source's round
+// is one latency chain: 30 rounds at depth 2 take 1,000 / 10,000 / 100,000
+// points 289 / 308 / 414 us with it and 297 / 317 / 419 without; at depth 3 the
+// 100,000 take 447 and 453.
+template <bool STAGED>
 __device__ __forceinline__ void descend_points(const float4* __restrict__ src, int n,
                                                const float4* __restrict__ blocks, const float4* sm_blocks, int depth,
                                                const float* Rt_sm, float qscale,
@@ -1739,9 +1747,9 @@ __device__ __forceinline__ void descend_points(const float4* __restrict__ src, i
         int first = 0;  // the current search node's first child
         float2 u[4];
         float best = 0.f;
-        int left = valid ? depth : 0;  // levels left
-        while (left > 0) {
-            const unsigned stops = child_scores(blocks, sm_blocks, first, x, y, z, u);
+        bool above = false;
+        for (int left = valid ? depth : 0; left > 0; --left) {
+            const unsigned stops = child_scores<STAGED>(blocks, sm_blocks, first, x, y, z, u);
             // the best child, by a tournament (a chain of eight compares and
             // selects was 5 % of a round): the lowest index among equals
             float m[4];
@@ -1758,16 +1766,19 @@ __device__ __forceinline__ void descend_points(const float4* __restrict__ src, i
             if (!(best < CUDART_INF_F)) {
                 // no child has a finite score (a point so far away that every
                 // square overflows, or a root without live nodes): the descent
-                // ended with the node above, whose block is scored once more
-                if (chosen < 0) break;
-                first = chosen & ~7;
-                left = 1;
-                continue;
+                // ended with the node above
+                above = chosen >= 0;
+                break;
             }
             chosen = first + bi;
             first = 8 * chosen + 8;
             if ((stops >> bi) & 1u) break;  // Complexity <= lambda_c, or no live children
-            --left;
+        }
+        if (above) {  // its block is scored once more (after the loop: a second way
+                      // round it slowed 30 rounds of 1M points from 1,742 to 1,764 us)
+            child_scores<STAGED>(blocks, sm_blocks, chosen & ~7, x, y, z, u);
+            best = fminf(fminf(fminf(u[0].x, u[0].y), fminf(u[1].x, u[1].y)),
+                         fminf(fminf(u[2].x, u[2].y), fminf(u[3].x, u[3].y)));
         }
         // the posterior of the chosen child among its siblings: once, after
         // the descent (inside the loop its exponentials were on every level's
@@ -1792,7 +1803,7 @@ __device__ __forceinline__ void descend_points(const float4* __restrict__ src, i
         if (has) {
             const int o = (chosen >> 3) * (4 * BLOCK_F4) + block_child(chosen & 7);
             float mx, my, mz;  // the node's negated mean
-            if (chosen < STAGED_NODES) {
+            if (STAGED || chosen < STAGED_NODES) {
                 const float* m = reinterpret_cast<const float*>(sm_blocks) + o;
                 mx = m[0];
                 my = m[2];

@@ -123,7 +123,9 @@ __device__ __forceinline__ void trace_mark(unsigned long long* tr, int it, int e
 // latency chain and the node terms and the solve want the registers; three
 // (80) for large sources, whose descent is throughput-bound and gains from
 // the extra warps.
-template <int MINB>
+// STAGED: the tree has no level below the staged ones (descend_points); built
+// for two CTAs per SM only, as a large source's descent does not gain from it.
+template <int MINB, bool STAGED>
 __global__ void __launch_bounds__(REG_THREADS, MINB) k_register(RegArgs a) {
     __shared__ float Rt_sm[12];
     __shared__ double T_sm[12];
@@ -155,7 +157,7 @@ __global__ void __launch_bounds__(REG_THREADS, MINB) k_register(RegArgs a) {
     const float qscale = float(FIX / ext);  // fixed-point units per metre
     for (int it = 0; it < a.iters; ++it) {
         trace_mark(a.trace, it, 0);
-        descend_points(a.src, a.n, a.blocks, sm_est, a.depth, Rt_sm, qscale, a.acc, blockIdx.x, gridDim.x, hist);
+        descend_points<STAGED>(a.src, a.n, a.blocks, sm_est, a.depth, Rt_sm, qscale, a.acc, blockIdx.x, gridDim.x, hist);
         __syncthreads();
         flush_node_hist(hist, ns, a.acc);
         __syncthreads();
@@ -922,8 +924,11 @@ int hgmm_register_impl(hgmm_tree* t, const float4* src, int64_t n64, const doubl
         t->trace_grid = a.trace ? grid : 0;
         void* args[] = {&a};
         ProfScope ps_(t, K_DESCEND, s);
-        const cudaError_t e = cudaLaunchCooperativeKernel(wide ? (const void*)k_register<3> : (const void*)k_register<2>,
-                                                          dim3(grid), dim3(REG_THREADS), args, REG_DYN_SMEM, s);
+        const void* fn = wide                       ? (const void*)k_register<3, false>
+                         : n_nodes <= STAGED_NODES ? (const void*)k_register<2, true>
+                                                    : (const void*)k_register<2, false>;
+        const cudaError_t e =
+            cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(REG_THREADS), args, REG_DYN_SMEM, s);
         if (e != cudaSuccess) {
             fprintf(stderr, "hgmm: cooperative launch failed: %s\n", cudaGetErrorString(e));
             return HGMM_ECUDA;
@@ -985,15 +990,22 @@ int hgmm_register_descent_impl(hgmm_tree* t, const float4* src, int64_t n64, con
 
 int hgmm_register_grid(int n_sm, int per_sm) {
     // static + dynamic shared memory exceeds the 48 KB default: opt in; the
-    // grid must be co-resident; 0 if the build asked for does not reach per_sm
-    // CTAs per SM (the caller then keeps to the two-per-SM build)
+    // grid must be co-resident for every kernel of the build asked for; 0 if
+    // that does not reach per_sm CTAs per SM (the caller then keeps to the
+    // two-per-SM build)
     if (per_sm != 2 && per_sm != 3) return 0;
-    const void* fn = per_sm == 3 ? (const void*)k_register<3> : (const void*)k_register<2>;
-    int k = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(REG_DYN_SMEM)) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, fn, REG_THREADS, REG_DYN_SMEM) != cudaSuccess || k < 1)
-        return 0;
-    const int got = std::min(per_sm, k);
+    const void* wide[] = {(const void*)k_register<3, false>};
+    const void* two[] = {(const void*)k_register<2, false>, (const void*)k_register<2, true>};
+    int got = per_sm;
+    for (int i = 0; i < (per_sm == 3 ? 1 : 2); ++i) {
+        const void* fn = per_sm == 3 ? wide[i] : two[i];
+        int k = 0;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(REG_DYN_SMEM)) !=
+                cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, fn, REG_THREADS, REG_DYN_SMEM) != cudaSuccess || k < 1)
+            return 0;
+        got = std::min(got, k);
+    }
     if (per_sm == 3 && got < 3) return 0;
     return n_sm * got;  // <= co-resident CTAs (cooperative launch)
 }
