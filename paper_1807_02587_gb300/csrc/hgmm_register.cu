@@ -28,7 +28,14 @@ namespace hgmm {
 
 namespace {
 
-__global__ void k_reg_init(const double* __restrict__ T_init, int n_nodes, float lam_c,
+// Start of a registration: stop flags for its threshold, zeroed moments and
+// counters, the starting pose and (blocks not null: the variants read the
+// records themselves) the descent's sibling blocks.  Loads of a node's record
+// and of its children's bound it: 64 threads per CTA spread them over the SMs
+// (256 took 8.0 us for the 4,680 nodes of depth 4, these 6.3, as without blocks;
+// depth 5 8.2 and 7.1).
+constexpr int REG_INIT_THREADS = 64;
+__global__ void __launch_bounds__(REG_INIT_THREADS) k_reg_init(const double* __restrict__ T_init, int n_nodes, float lam_c,
                            const NodeStat* __restrict__ stat, NodeEst* est, float4* __restrict__ blocks,
                            unsigned long long* __restrict__ acc, double* __restrict__ T,
                            float* __restrict__ Rt, unsigned* __restrict__ bar,
@@ -39,15 +46,17 @@ __global__ void k_reg_init(const double* __restrict__ T_init, int n_nodes, float
     bool childless = false;
     if (in) {
         // the record, its children's and the complexity in one round trip
-        ea = __ldcg(&est[i].a);
-        eb = __ldcg(&est[i].b);
-        ec = __ldcg(&est[i].c);
+        if (blocks) {
+            ea = __ldcg(&est[i].a);
+            eb = __ldcg(&est[i].b);
+            ec = __ldcg(&est[i].c);
+        }
         const bool simple = stat[i].live && stat[i].complexity <= double(lam_c);
-        childless = no_live_children(est, i, n_nodes);
+        if (blocks) childless = no_live_children(est, i, n_nodes);
         for (int k = 0; k < 4 * ACC_REPLICAS; ++k) acc[4 * ACC_REPLICAS * int64_t(i) + k] = 0ull;
         if (lam_c >= 0.f) est[i].c.z = ec.z = simple ? 1.f : 0.f;
     }
-    pack_node(blocks, i, in, ea, eb, ec, ec.z != 0.f || childless);  // the descent's sibling blocks
+    if (blocks) pack_node(blocks, i, in, ea, eb, ec, ec.z != 0.f || childless);
     if (i == 0) {
         for (int k = 0; k < 16; ++k) T[k] = T_init ? T_init[k] : ((k % 5 == 0) ? 1.0 : 0.0);
         for (int r = 0; r < 3; ++r) {
@@ -874,9 +883,8 @@ int hgmm_register_impl(hgmm_tree* t, const float4* src, int64_t n64, const doubl
         // lam_c < 0: the build's threshold (set here too, so that an earlier
         // call with another threshold does not leave its stop flags behind)
         if (lam_c < 0.f) lam_c = t->prm.lam_c;
-        k_reg_init<<<(n_nodes + 255) / 256, 256, 0, s>>>(T_init, n_nodes, lam_c, t->stat, t->est, t->rblk,
-                                                          t->reg_acc, t->reg_T, t->reg_Rt,
-                                                          t->reg_bar, t->reg_obj);
+        k_reg_init<<<(n_nodes + REG_INIT_THREADS - 1) / REG_INIT_THREADS, REG_INIT_THREADS, 0, s>>>(
+            T_init, n_nodes, lam_c, t->stat, t->est, t->rblk, t->reg_acc, t->reg_T, t->reg_Rt, t->reg_bar, t->reg_obj);
     }
     // a large source that fits the tree's free point buffer is put into
     // spatial order there, with the CTAs' cell counts and the cells' totals in
@@ -952,8 +960,8 @@ int hgmm_register_descent_impl(hgmm_tree* t, const float4* src, int64_t n64, con
     const int n = int(n64);
     const int n_nodes = int(hgmm_node_count(t->depth));
     const float lam_c = d.lam_c >= 0.f ? d.lam_c : t->prm.lam_c;
-    k_reg_init<<<(n_nodes + 255) / 256, 256, 0, s>>>(T_init, n_nodes, lam_c, t->stat, t->est, t->rblk, t->reg_acc,
-                                                      t->reg_T, t->reg_Rt, t->reg_bar, t->reg_obj);
+    k_reg_init<<<(n_nodes + REG_INIT_THREADS - 1) / REG_INIT_THREADS, REG_INIT_THREADS, 0, s>>>(
+        T_init, n_nodes, lam_c, t->stat, t->est, nullptr, t->reg_acc, t->reg_T, t->reg_Rt, t->reg_bar, t->reg_obj);
     const int tgrid = (n_nodes + VAR_THREADS - 1) / VAR_THREADS;
     const int dgrid = std::max(1, std::min(4 * t->n_sm, (n + VAR_THREADS - 1) / VAR_THREADS));
     const bool full = d.full_eq7 != 0;

@@ -90,3 +90,23 @@ def test_scores_that_overflow(depth):
         tree.sync()
     except B.HgmmError as e:
         assert e.code == B.HGMM_EDEGENERATE
+
+
+def test_registrations_around_a_variant():
+    """A variant with another threshold between two registrations leaves no
+    trace: the blocks are those of the registration's own threshold."""
+    from paper_1807_02587_gb300 import binding as B
+    p = synth.primitive_pair(5, 20000)
+    tgt, _ = PT.device_cloud(p["tgt"])
+    src, _ = PT.device_cloud(p["src"])
+    want = {}
+    for lam_c in (-1.0, 0.0, 0.2):
+        tree = B.Tree(20000, 4)
+        tree.build(tgt, 4)
+        want[lam_c] = tree.register(src, iters=5, lam_c=lam_c).cpu().numpy()
+    tree = B.Tree(20000, 4)
+    tree.build(tgt, 4)
+    for lam_c, other in ((0.0, 0.2), (0.2, 0.0), (-1.0, 0.0), (0.0, -1.0)):
+        tree.register_descent(src, B.HGMM_DESCENT_MULTIPATH, tau=0.1, iters=2, lam_c=other)
+        assert np.array_equal(tree.register(src, iters=5, lam_c=lam_c).cpu().numpy(), want[lam_c])
+    tree.sync()
