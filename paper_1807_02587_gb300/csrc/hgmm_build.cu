@@ -288,6 +288,68 @@ k_estep(const float4* __restrict__ pts, const Item* __restrict__ items,
     flush_sets<COMP>(acc_s, acc_c, red, partials + int64_t(run) * NPART);
 }
 
+// The level-wide E-step of small clouds: chunks of at most ESTEP_SHORT_ITEMS
+// items, so that a run needs one compensated fold and no running pairs (the
+// arithmetic of estep_range, the same bits).  A few items per CTA are latency:
+// a quad of lanes per point, all of an item's points loaded at once and the next
+// item's behind them.  us per E-step (precision 1, depth 2; with the event
+// pair), k_estep / here: 1,000 points 8.0 / 6.1, 93,000 10.0 / 8.5, 409,000 (four
+// items per chunk, the last size it takes) 13.6 / 12.6.
+constexpr int ESTEP_SHORT_ITEMS = EST_FOLD * 64 / TILE;
+template <bool COMP>
+__global__ void __launch_bounds__(EST_THREADS, 3)
+k_estep_short(const float4* __restrict__ pts, const Item* __restrict__ items, const int* __restrict__ meta,
+              const NodeEst* __restrict__ est_lvl, float2* __restrict__ partials) {
+    constexpr int STEPS = TILE / 64;
+    __shared__ float2 red[EST_THREADS / 32][NPART];
+    const int n_items = meta[0], C = meta[1];
+    const int ib = blockIdx.x * C, ie = min(ib + C, n_items);
+    if (ib >= ie) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int q = warp * 8 + (lane >> 2), k = lane & 3;
+    float2 in[10];
+#pragma unroll
+    for (int v = 0; v < 10; ++v) in[v] = make_float2(0.f, 0.f);
+    auto flush = [&](int run) {
+        float s[20], c[20];
+#pragma unroll
+        for (int v = 0; v < 10; ++v) {
+            s[v] = in[v].x;
+            s[10 + v] = in[v].y;
+            c[v] = c[10 + v] = 0.f;
+            in[v] = make_float2(0.f, 0.f);
+        }
+        flush_warp<COMP>(s, c, warp, red);
+        flush_rows<COMP>(red, partials + int64_t(run) * NPART);
+    };
+    Item w = items[ib];
+    float4 z[STEPS];
+#pragma unroll
+    for (int u = 0; u < STEPS; ++u) z[u] = pts[w.start + min(64 * u + q, w.count - 1)];
+    int cur = -1, run = -1;
+    bool live = false;
+    ChildPair cp;
+    for (int it = ib; it < ie; ++it) {
+        if (w.parent != cur) {
+            if (cur >= 0) flush(run);
+            cur = w.parent;
+            run = it;
+            load_child_pair(est_lvl + 8 * cur + 2 * k, cp);
+            live = parent_has_live_child(cp);
+        }
+        const int count = w.count;
+        if (it + 1 < ie) w = items[it + 1];
+#pragma unroll
+        for (int u = 0; u < STEPS; ++u) {
+            const float4 p = z[u];
+            if (it + 1 < ie) z[u] = pts[w.start + min(64 * u + q, w.count - 1)];
+            // a parent without a live child: zero posteriors, nothing to add
+            if (live && 64 * u < count) estep_point_pair(cp, p, 64 * u + q < count, in);
+        }
+    }
+    flush(run);
+}
+
 // The level-wide M-step: CTA (p, j) reduces slice j of parent p's runs into
 // the slice buffer; the last of the parent's n_slices CTAs to finish
 // (arrival counter, reset by that CTA) combines the slices in order and runs
@@ -500,6 +562,20 @@ k_assign(const float4* __restrict__ pts, const Item* __restrict__ items, const i
     }
 }
 
+// The same with one CTA per item, while every item has its own (at most
+// n / TILE + parents <= the E-step's grid): a warp per item is then a chain of
+// eight steps on a few SMs.  us per level for the labels and for the partition,
+// a warp / a CTA per item: 10,000 points 9.6 + 6.8 / 8.3 + 6.2, 60,000 10.2 + 7.7 /
+// 8.5 + 6.0, 277,000 12.0 + 8.1 / 14.8 + 8.5.
+__global__ void __launch_bounds__(EST_THREADS)
+k_assign_cta(const float4* __restrict__ pts, const Item* __restrict__ items, const int* __restrict__ meta,
+             const NodeEst* __restrict__ est_lvl, uint32_t* __restrict__ codes, int* __restrict__ item_cnt) {
+    __shared__ AssignSmem as;
+    const int n_items = meta[0];
+    for (int it = blockIdx.x; it < n_items; it += gridDim.x)
+        assign_item(pts, items[it], it, est_lvl, codes, item_cnt, as);
+}
+
 // Slice j of the nsl slices of a parent's items [i0, i1).
 __device__ __forceinline__ void offset_slice(int i0, int i1, int nsl, int j, int& a, int& b) {
     const int per = (i1 - i0 + nsl - 1) / nsl;
@@ -616,6 +692,20 @@ __global__ void __launch_bounds__(256) k_scatter(const float4* __restrict__ pts_
             }
         }
     }
+}
+
+// The same with one CTA per item, for clouds of few items (see k_assign_cta).
+__global__ void __launch_bounds__(256) k_scatter_cta(const float4* __restrict__ pts_in,
+                                                     const int* __restrict__ perm_in,
+                                                     const Item* __restrict__ items,
+                                                     const int* __restrict__ meta,
+                                                     const uint32_t* __restrict__ codes,
+                                                     const int* __restrict__ item_off,
+                                                     float4* __restrict__ pts_out,
+                                                     int* __restrict__ perm_out) {
+    const int n_items = meta[0];
+    for (int it = blockIdx.x; it < n_items; it += gridDim.x)
+        scatter_item(pts_in, perm_in, items[it], it, codes, item_off, pts_out, perm_out, threadIdx.x, blockDim.x);
 }
 
 __global__ void k_finalize(int level, float lam_c, const RootDev* __restrict__ root,
@@ -807,6 +897,9 @@ int hgmm_build_impl(hgmm_tree* t, const float4* pts, int64_t n64, int depth,
                 l, n, n_par, t->seg_start, t->seg_count, t->item_range, t->meta, t->items);
         }
         HGMM_LAUNCH_CHECK();
+        // at most this many items (each parent's last may be ragged), G chunks of them
+        const int64_t items_most = (n64 + TILE - 1) / TILE + n_par;
+        const bool short_items = items_most <= int64_t(ESTEP_SHORT_ITEMS) * G, few_items = items_most <= G;
         const bool stop_here = p.debug_stop_level == l + 1;
         const int em_iters = stop_here ? p.debug_stop_iters : p.em_iters;
         const bool local_em = n_par >= LOCAL_EM_PARENTS && n64 <= LOCAL_EM_POINTS * n_par;
@@ -836,7 +929,13 @@ int hgmm_build_impl(hgmm_tree* t, const float4* pts, int64_t n64, int depth,
             }
         }
         for (int k = 0; k < (local_em || coop_em ? 0 : em_iters); ++k) {
-            {
+            if (short_items) {
+                ProfScope ps_(t, K_ESTEP, s);
+                if (comp)
+                    k_estep_short<true><<<G, EST_THREADS, 0, s>>>(cur, t->items, t->meta, est_lvl, t->partials);
+                else
+                    k_estep_short<false><<<G, EST_THREADS, 0, s>>>(cur, t->items, t->meta, est_lvl, t->partials);
+            } else {
                 ProfScope ps_(t, K_ESTEP, s);
                 if (comp)
                     k_estep<true><<<G, ESTEP_CTA, ESTEP_DYN_SMEM, s>>>(cur, t->items, t->meta, est_lvl, t->partials, t->status);
@@ -859,7 +958,11 @@ int hgmm_build_impl(hgmm_tree* t, const float4* pts, int64_t n64, int depth,
         if (stop_here) return HGMM_OK;  // checking aid: parameters after em_iters
         {
             ProfScope ps_(t, K_ASSIGN, s);
-            k_assign<<<t->n_sm * 2, ASSIGN_THREADS, 0, s>>>(cur, t->items, t->meta, est_lvl, t->codes, t->item_cnt);
+            if (few_items)
+                k_assign_cta<<<G, EST_THREADS, 0, s>>>(cur, t->items, t->meta, est_lvl, t->codes, t->item_cnt);
+            else
+                k_assign<<<t->n_sm * 2, ASSIGN_THREADS, 0, s>>>(cur, t->items, t->meta, est_lvl, t->codes,
+                                                                t->item_cnt);
         }
         {
             ProfScope ps_(t, K_OFFSETS, s);
@@ -877,8 +980,12 @@ int hgmm_build_impl(hgmm_tree* t, const float4* pts, int64_t n64, int depth,
         float4* out = t->pts[l & 1];
         {
             ProfScope ps_(t, K_SCATTER, s);
-            k_scatter<<<t->n_sm * 4, 256, 0, s>>>(cur, perm_prev, t->items, t->meta, t->codes, t->item_off,
-                                        out, t->perm[l]);
+            if (few_items)
+                k_scatter_cta<<<G, 256, 0, s>>>(cur, perm_prev, t->items, t->meta, t->codes, t->item_off, out,
+                                                t->perm[l]);
+            else
+                k_scatter<<<t->n_sm * 4, 256, 0, s>>>(cur, perm_prev, t->items, t->meta, t->codes, t->item_off, out,
+                                                      t->perm[l]);
         }
         const int m = int(level_size(l));
         {
