@@ -60,17 +60,56 @@ static_assert(GROUP == 32 && LSE_TILE % GROUP == 0, "whole groups");
 constexpr size_t GMAX_KEPT = size_t(1) << 26;
 constexpr int MOM_THREADS = 256; // one component per thread
 constexpr int MOM_STAGE = 2048;  // points staged per pass (a slice of an ordinary cloud)
+static_assert(MOM_STAGE % 32 == 0, "whole blocks of a warp");
+// A block of 16 points with at least this many for a warp is computed whole,
+// unrolled: the others add exact zeros.  Fewer are picked out two at a time, one
+// after the other, which the issue slots gain from and a lone warp's latency does
+// not: where every SM has at most one CTA, any point makes a block whole.
+// Registrations of 20 rounds, 90,000 points at depth 4 / 10,000 at depth 2, from
+// 7 / 10 / 13 / 16 points on: 5,682 / 5,640 / 5,684 / 5,722 us, 565 / 557 / 573 /
+// 597; 2,000 at depth 2: 476 us whole from the first point on, 495 from 16.
+constexpr int MOM_WHOLE = 10;
 constexpr int NMOM_MAX = 10;
 
 // ------------------------------------------------------------ from the tree
+// Component j from node g with path product w (`total`: the products' sum).
+__device__ __forceinline__ void write_component(const NodeStat* __restrict__ st, int g, int j, double w, double total,
+                                                double eps, FlatComp* __restrict__ comp, NodeEst* __restrict__ est,
+                                                float4* __restrict__ rterm, int* __restrict__ status) {
+    int l = 0;
+    while (g >= d_level_offset(l + 1)) ++l;
+    const NodeStat& s = st[g];
+    FlatComp& f = comp[j];
+    f.pi = w * (total > 0.0 ? 1.0 / total : 0.0);
+    for (int a = 0; a < 3; ++a) f.mu[a] = s.mu[a];
+    for (int v = 0; v < 6; ++v) f.S[v] = s.S[v];
+    for (int a = 0; a < 3; ++a) f.lam[a] = s.lam[a];
+    for (int v = 0; v < 9; ++v) f.V[v] = s.V[v];
+    for (int v = 0; v < 6; ++v) f.P[v] = s.P[v];
+    f.live = 1;
+    f.level = l;
+    f.index = int(g - d_level_offset(l));
+    if (!pack_est(f.pi, f.mu, f.S, eps, 0.f, est[j])) atomicOr(status, ST_CHOL);
+    const float4 a = est[j].a;
+    rterm[3 * j] = make_float4(float(s.P[0]), float(s.P[1]), float(s.P[2]), float(s.P[3]));
+    rterm[3 * j + 1] = make_float4(float(s.P[4]), float(s.P[5]), 0.f, 0.f);
+    rterm[3 * j + 2] = make_float4(float(s.mu[0] - double(a.x)), float(s.mu[1] - double(a.y)),
+                                   float(s.mu[2] - double(a.z)), 0.f);
+}
+
 // One CTA.  Candidates are the nodes of levels 0..L-1 (global id order);
 // thread t takes a contiguous run of them, so the block scan of the run
 // counts gives the components in (level, index) order.  slot[g] = component
 // of node g (-1: none), wt[g] = its path product, wtot = the products' sum.
+// WRITE: it writes the components too, one candidate per thread.
+constexpr int FROM_TREE_ONE = 128;
+template <bool WRITE>
 __global__ void __launch_bounds__(FROM_TREE_THREADS)
 k_flat_select(const NodeStat* __restrict__ st, const RootDev* __restrict__ root, int L, int n_cand,
               int* __restrict__ slot, double* __restrict__ wt, double* __restrict__ wtot, int* __restrict__ meta,
-              double* __restrict__ eps_out, int* __restrict__ status) {
+              double* __restrict__ eps_out, FlatComp* __restrict__ comp, NodeEst* __restrict__ est,
+              float4* __restrict__ rterm, int* __restrict__ status) {
+    __shared__ double total;
     __shared__ int wcount[FROM_TREE_THREADS / 32];
     __shared__ double wsum[FROM_TREE_THREADS / 32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -116,7 +155,7 @@ k_flat_select(const NodeStat* __restrict__ st, const RootDev* __restrict__ root,
             run += c;
             tot += wsum[w];
         }
-        *wtot = tot;
+        *wtot = total = tot;
         meta[0] = run;
         *eps_out = root->eps;
         if (!(tot > 0.0)) atomicOr(status, ST_DEGENERATE);
@@ -124,12 +163,16 @@ k_flat_select(const NodeStat* __restrict__ st, const RootDev* __restrict__ root,
     __syncthreads();
     const int first = wcount[warp] + incl - cnt;
     for (int g = g0; g < g1; ++g)
-        if (slot[g] >= 0) slot[g] += first;
+        if (slot[g] >= 0) {
+            slot[g] += first;
+            if (WRITE) write_component(st, g, slot[g], wt[g], total, root->eps, comp, est, rterm, status);
+        }
 }
 
 // The components, one thread per candidate (one CTA doing the selection and
 // the FP64 Cholesky factors of all of them took 170 us for 4,680 candidates;
-// the two launches 39).
+// the two launches 39; for the 584 of depth 3 36 and 23.5, for the 72 of depth 2
+// 20.3 and 22.5: up to FROM_TREE_ONE candidates k_flat_select writes them).
 __global__ void __launch_bounds__(64)
 k_flat_write(const NodeStat* __restrict__ st, int n_cand, const int* __restrict__ slot,
              const double* __restrict__ wt, const double* __restrict__ wtot, const double* __restrict__ eps_in,
@@ -137,28 +180,7 @@ k_flat_write(const NodeStat* __restrict__ st, int n_cand, const int* __restrict_
              int* __restrict__ status) {
     const int g = blockIdx.x * 64 + threadIdx.x;
     if (g >= n_cand) return;
-    const int j = slot[g];
-    if (j < 0) return;
-    int l = 0;
-    while (g >= d_level_offset(l + 1)) ++l;
-    const NodeStat& s = st[g];
-    const double total = *wtot;
-    FlatComp& f = comp[j];
-    f.pi = wt[g] * (total > 0.0 ? 1.0 / total : 0.0);
-    for (int a = 0; a < 3; ++a) f.mu[a] = s.mu[a];
-    for (int v = 0; v < 6; ++v) f.S[v] = s.S[v];
-    for (int a = 0; a < 3; ++a) f.lam[a] = s.lam[a];
-    for (int v = 0; v < 9; ++v) f.V[v] = s.V[v];
-    for (int v = 0; v < 6; ++v) f.P[v] = s.P[v];
-    f.live = 1;
-    f.level = l;
-    f.index = int(g - d_level_offset(l));
-    if (!pack_est(f.pi, f.mu, f.S, *eps_in, 0.f, est[j])) atomicOr(status, ST_CHOL);
-    const float4 a = est[j].a;
-    rterm[3 * j] = make_float4(float(s.P[0]), float(s.P[1]), float(s.P[2]), float(s.P[3]));
-    rterm[3 * j + 1] = make_float4(float(s.P[4]), float(s.P[5]), 0.f, 0.f);
-    rterm[3 * j + 2] = make_float4(float(s.mu[0] - double(a.x)), float(s.mu[1] - double(a.y)),
-                                   float(s.mu[2] - double(a.z)), 0.f);
+    if (slot[g] >= 0) write_component(st, g, slot[g], wt[g], *wtot, *eps_in, comp, est, rterm, status);
 }
 
 // ------------------------------------------------------------- E-step parts
@@ -383,7 +405,8 @@ __device__ __forceinline__ void fold_mom(float (&in)[NM], float (&s)[NM], float 
     }
 }
 
-// Partial moments of a tile of 256 components over the points of one slice; NM = 4 (gamma, gamma e) or 10 (and gamma e e^T), e = z' - mu32.
+// Partial moments of a tile of 256 components over the points of one slice;
+// NM = 4 (gamma, gamma e) or 10 (and gamma e e^T), e = z' - mu32.
 // Issue bounds it (22 instructions per 32 pairs at 79 % of the issue slots;
 // packing two components or points into FP32x2 instructions halves their
 // number and leaves the time as it was: 159 against 162 us), so the pairs
@@ -438,22 +461,28 @@ k_flat_moments(const float4* __restrict__ pts, int n, const float* __restrict__ 
             accum10(in, g, ex, ey, ez);
         }
     };
+    const int whole = pl.tiles * pl.slices <= gridDim.x / 4 ? 1 : MOM_WHOLE;  // gridDim: four CTAs per SM
     for (int b = i0; b < i1; b += MOM_STAGE) {
         const int cnt = min(MOM_STAGE, i1 - b);
+        // this warp's group maxima of the stage, two blocks of 32 points ahead
+        // (the first two are in flight while the stage is filled)
+        const float* gm = gmax && group * GROUP < J ? gmax + group * gstride + b : nullptr;
+        auto group_max = [&](int q) { return gm && q < cnt ? __ldg(gm + q) : CUDART_INF_F; };
+        float g0 = group_max(lane), g1 = group_max(32 + lane);
         __syncthreads();
         for (int q = threadIdx.x; q < cnt; q += MOM_THREADS) {
             float x, y, z;
             const bool fin = load_point<XF>(pts, b + q, r, x, y, z, nullptr);  // reported by k_flat_lse
             sp[q] = make_float4(x, y, z, fin ? __ldg(lse + b + q) : CUDART_INF_F);
         }
+        // the last block of 16 is filled up with points that add nothing
+        if (threadIdx.x < 16 && cnt + threadIdx.x < MOM_STAGE)
+            sp[cnt + threadIdx.x] = make_float4(0.f, 0.f, 0.f, CUDART_INF_F);
         __syncthreads();
         // this warp's points of the stage (a NaN keeps its point)
         if (group * GROUP >= J) continue;  // no component (after the block barriers: they come first in a stage)
         // plain FP32 sums over 16 points (a block without a point for this
         // warp leaves them and the fold unchanged), then one compensated fold
-        const float* gm = gmax ? gmax + group * gstride + b : nullptr;
-        auto group_max = [&](int q) { return gm && q < cnt ? __ldg(gm + q) : CUDART_INF_F; };
-        float g0 = group_max(lane), g1 = group_max(32 + lane);  // loaded two blocks of 32 ahead
         for (int w = 0; w < cnt; w += 32) {
             const float gc = g0;
             g0 = g1;
@@ -465,7 +494,7 @@ k_flat_moments(const float4* __restrict__ pts, int n, const float* __restrict__ 
                 unsigned mm = (live >> h) & 0xFFFFu;
                 if (mm == 0) continue;
                 const float4* z = sp + w + h;
-                if (mm == 0xFFFFu) {
+                if (__popc(mm) >= whole) {
 #pragma unroll
                     for (int u = 0; u < 16; ++u) pair(z[u]);
                 } else {
@@ -747,6 +776,7 @@ int moment_grid(const hgmm_flat* f) {
 
 // The table of group maxima for a call on n points, or null if it does not fit.
 float* group_maxima(const hgmm_flat* f, int64_t n) {
+    if (f->jcap <= GROUP) return nullptr;  // one group is never far from the likelihood it makes up
     return size_t(n) * size_t((f->jcap + GROUP - 1) / GROUP) <= f->gmax_cap ? f->gmax : nullptr;
 }
 
@@ -801,10 +831,13 @@ int hgmm_flat_from_tree(hgmm_flat* f, const hgmm_tree* t, int32_t level, void* s
     const int64_t n_cand = level_offset(L);
     if (n_cand > f->cap_comp) return HGMM_ECAPACITY;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    k_flat_select<<<1, FROM_TREE_THREADS, 0, s>>>(t->stat, t->root, L, int(n_cand), f->slot, f->wt,
-                                                 f->wt + f->cap_comp, f->meta, f->eps, f->status);
-    k_flat_write<<<int((n_cand + 63) / 64), 64, 0, s>>>(t->stat, int(n_cand), f->slot, f->wt, f->wt + f->cap_comp,
-                                                       f->eps, f->comp, f->est, f->rterm, f->status);
+    const auto select = n_cand <= FROM_TREE_ONE ? k_flat_select<true> : k_flat_select<false>;
+    select<<<1, FROM_TREE_THREADS, 0, s>>>(t->stat, t->root, L, int(n_cand), f->slot, f->wt, f->wt + f->cap_comp,
+                                           f->meta, f->eps, f->comp, f->est, f->rterm, f->status);
+    if (n_cand > FROM_TREE_ONE)
+        k_flat_write<<<int((n_cand + 63) / 64), 64, 0, s>>>(t->stat, int(n_cand), f->slot, f->wt,
+                                                           f->wt + f->cap_comp, f->eps, f->comp, f->est, f->rterm,
+                                                           f->status);
     f->jcap = int(n_cand);
     f->have = true;
     return launched();
