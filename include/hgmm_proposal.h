@@ -147,7 +147,13 @@ int hgmm_pose_select(int32_t n, const double* d_T_a, const double* d_obj_a, cons
  * n x 16 each; d_out may alias neither input). */
 int hgmm_pose_compose(int32_t n, const double* d_A, const double* d_B, double* d_out, void* stream);
 
-/* Checking entry point for the tensor-core GEMM the network runs on:
+/* Fallback check: while disabled (enable = 0), tensor maps count as
+ * unavailable and the network's passes run their products one by one, as they
+ * do where the driver cannot encode the maps. */
+int hgmm_debug_mlp_maps(hgmm_mlp* m, int32_t enable);
+
+/* Checking entry point for the tensor-core GEMM (the network's products where
+ * its passes are not fused):
  * d_out[m * N + n] = sum_k A[m][k] B[n][k] (float32, device) with BF16
  * operands A[m][k] = d_A[m * a_m + k * a_k], B[n][k] = d_B[n * b_n + k * b_k]
  * (element strides; for each operand either the k stride or the row stride

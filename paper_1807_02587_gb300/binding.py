@@ -120,6 +120,7 @@ def _load():
         "hgmm_mlp_adam": (ctypes.c_int, [vp, f32, vp]),
         "hgmm_mlp_train_step": (ctypes.c_int, [vp, vp, vp, vp, i32, i32, f32, f32, vp, vp]),
         "hgmm_mlp_sync": (ctypes.c_int, [vp, vp]),
+        "hgmm_debug_mlp_maps": (ctypes.c_int, [vp, i32]),
         "hgmm_tree_features": (ctypes.c_int, [vp, vp, vp, vp]),
         "hgmm_pose_decode": (ctypes.c_int, [vp, vp, i32, vp, vp]),
         "hgmm_pose_encode": (ctypes.c_int, [vp, vp, i32, vp, vp]),
@@ -609,6 +610,10 @@ def hgmm_mlp_train_step(h, x, labels, batch: int, index=None, w_t: float = 1.0, 
 
 def hgmm_mlp_sync(h, stream=None) -> None:
     _check(_lib.hgmm_mlp_sync(h, _stream_ptr(stream)), "hgmm_mlp_sync")
+
+
+def hgmm_debug_mlp_maps(h, enable: bool) -> None:
+    _check(_lib.hgmm_debug_mlp_maps(h, 1 if enable else 0), "hgmm_debug_mlp_maps")
 
 
 def hgmm_tree_features(h, feat, frame, stream=None):

@@ -539,6 +539,7 @@ struct hgmm_mlp {
     int* err = nullptr;
     float* ws = nullptr;      // K-slice partials of the weight gradients
     long long ws_cap = 0;     // floats
+    bool maps = true;         // tensor maps may be used (checking aid: hgmm_debug_mlp_maps)
     bf16* prop_x = nullptr;   // hgmm_propose: one pair's input (1280)
     double* prop_fr = nullptr;  // ... its frames (source, target: 32)
     float* prop_y = nullptr;  // ... the network's output (9)
@@ -616,10 +617,11 @@ int gemm_tma_launch(const GemmArgs& g, const CUtensorMap& ta, const CUtensorMap&
 // D = A B^T with the fused epilogue of g.  Both operands K-contiguous and
 // no K slices: the warp-specialised TMA kernel.  Otherwise the cp.async
 // kernel: N <= 16 runs 128 x 16 tiles, larger N 128 x 128 tiles; when the
-// tiles alone cannot fill the GPU and K is long (the weight gradients: K =
-// batch), K is cut into 64-multiple slices whose FP32 partials go to ws and
-// are summed in a fixed order.
-int gemm(GemmArgs g, cudaStream_t s, float* ws = nullptr, long long ws_cap = 0) {
+// tiles alone cannot fill the GPU, K is long and there is a workspace (the
+// weight gradients: K = batch), K is cut into 64-multiple slices whose FP32
+// partials go to ws and are summed in a fixed order.  maps: tensor maps may be
+// used.
+int gemm(GemmArgs g, cudaStream_t s, float* ws = nullptr, long long ws_cap = 0, bool maps = true) {
     if (g.M < 1 || g.N < 1 || g.K < 1 || !operand_ok(g.A, g.a_m, g.a_k, g.M, g.K) ||
         !operand_ok(g.B, g.b_n, g.b_k, g.N, g.K))
         return HGMM_EINVAL;
@@ -630,7 +632,7 @@ int gemm(GemmArgs g, cudaStream_t s, float* ws = nullptr, long long ws_cap = 0) 
     if (ws && g.epi == tc::EPI_F32 && tiles < 128) slices = std::min(std::min(MAX_SLICES, kt), (304 + tiles - 1) / tiles);
     g.k_split = ((kt + slices - 1) / slices) * tc::GEMM_BK;
     slices = (g.K + g.k_split - 1) / g.k_split;
-    if (slices <= 1 && g.a_k == 1 && g.b_k == 1) {
+    if (maps && slices <= 1 && g.a_k == 1 && g.b_k == 1) {
         // (operand_ok has checked 16-byte bases and row strides % 8 == 0)
         CUtensorMap ta, tb;
         if (encode_operand(&ta, g.A, g.a_m, g.M, g.K, tc::GEMM_BM) &&
@@ -681,6 +683,7 @@ GemmArgs gargs(const bf16* A, long long a_m, long long a_k, const bf16* B, long 
 // to m->H1 / m->H2 only when the backward pass needs them), or HGMM_ECUDA if
 // its tensor maps cannot be encoded (the caller then runs the three GEMMs).
 int forward_fused(hgmm_mlp* m, const bf16* X, int batch, float* Y, cudaStream_t s, bool keep_hidden) {
+    if (!m->maps) return HGMM_ECUDA;
     CUtensorMap tx, t1, t2, t3, h1 = {}, h2 = {};
     if (!encode_operand(&tx, X, IN, batch, IN, 128) || !encode_operand(&t1, m->W1, IN, HID, IN, HID) ||
         !encode_operand(&t2, m->W2, HID, HID, HID, HID) || !encode_operand(&t3, m->W3, HID, OUTP, HID, OUTP) ||
@@ -700,20 +703,53 @@ int forward_impl(hgmm_mlp* m, const bf16* X, int batch, float* Y, cudaStream_t s
     g.out_bf16 = m->H1;
     g.o_m = HID;
     g.o_n = 1;
-    if (int rc = gemm(g, s, m->ws, m->ws_cap)) return rc;
+    if (int rc = gemm(g, s, nullptr, 0, m->maps)) return rc;
     g = gargs(m->H1, HID, 1, m->W2, HID, 1, batch, HID, HID, tc::EPI_BIAS_RELU_BF16, m->err);
     g.bias = m->P + OFF_B2;
     g.out_bf16 = m->H2;
     g.o_m = HID;
     g.o_n = 1;
-    if (int rc = gemm(g, s, m->ws, m->ws_cap)) return rc;
+    if (int rc = gemm(g, s, nullptr, 0, m->maps)) return rc;
     g = gargs(m->H2, HID, 1, m->W3, HID, 1, batch, OUTP, HID, tc::EPI_BIAS_F32, m->err);
     g.bias = m->b3p;
     g.out_f32 = Y;
     g.o_m = OUT;
     g.o_n = 1;
     g.n_store = OUT;
-    return gemm(g, s);
+    return gemm(g, s, nullptr, 0, m->maps);
+}
+
+// The backward pass without tensor maps: the fused launches' products one by
+// one, the weight gradients into the first slice of ws (with their K slices
+// behind it).
+int backward_gemms(hgmm_mlp* m, const bf16* X, int batch, cudaStream_t s) {
+    float* const part = m->ws + WS_STRIDE;
+    const long long part_cap = m->ws_cap - WS_STRIDE;
+    // d = a b masked by act > 0, as BF16 (batch x HID)
+    auto activation = [&](const bf16* a, long long a_m, const bf16* b, int K, const bf16* act, bf16* d) {
+        GemmArgs g = gargs(a, a_m, 1, b, 1, HID, batch, HID, K, tc::EPI_MASK_BF16, m->err);
+        g.mask = act;
+        g.mask_m = HID;
+        g.out_bf16 = d;
+        g.o_m = HID;
+        g.o_n = 1;
+        return gemm(g, s, nullptr, 0, false);
+    };
+    // columns of a (M) times columns of b (N), summed over the batch
+    auto weights = [&](const bf16* a, const bf16* b, long long b_k, int N, int64_t off, long long o_m, long long o_n,
+                       int n_store) {
+        GemmArgs g = gargs(a, 1, HID, b, 1, b_k, HID, N, batch, tc::EPI_F32, m->err);
+        g.out_f32 = m->ws + off;
+        g.o_m = o_m;
+        g.o_n = o_n;
+        g.n_store = n_store;
+        return gemm(g, s, part, part_cap, false);
+    };
+    if (int rc = activation(m->dY, DY_STRIDE, m->W3, OUTP, m->H2, m->dZ2)) return rc;
+    if (int rc = activation(m->dZ2, HID, m->W2, HID, m->H1, m->dZ1)) return rc;
+    if (int rc = weights(m->H2, m->dY, DY_STRIDE, OUTP, OFF_W3, 1, HID, OUT)) return rc;
+    if (int rc = weights(m->dZ2, m->H1, HID, HID, OFF_W2, HID, 1, HID)) return rc;
+    return weights(m->dZ1, X, IN, IN, OFF_W1, IN, 1, IN);
 }
 
 bool set_gemm_smem() {
@@ -755,16 +791,17 @@ int gradients_impl(hgmm_mlp* m, const uint16_t* d_x, const float* d_labels, cons
     const float* L = d_labels;
     // tensor maps of the backward pass: K-major operands and the dZ tiles
     // (128-row boxes), and the weight gradients' operands (64-row boxes)
-    CUtensorMap bdy, bw3, bw2, bz2, bz1, gz1, gx, gz2, gh1, gh2, gdy;
+    CUtensorMap bdy = {}, bw3 = {}, bw2 = {}, bz2 = {}, bz1 = {}, gz1 = {}, gx = {}, gz2 = {}, gh1 = {}, gh2 = {},
+                gdy = {};
     const bf16* Xb = d_index ? m->Xg : X;
-    if (!encode_operand(&bdy, m->dY, DY_STRIDE, batch, DY_STRIDE, 128) ||
-        !encode_operand(&bw3, m->W3T, DY_STRIDE, HID, DY_STRIDE, HID) ||
-        !encode_operand(&bw2, m->W2T, HID, HID, HID, HID) || !encode_operand(&bz2, m->dZ2, HID, batch, HID, 128) ||
-        !encode_operand(&bz1, m->dZ1, HID, batch, HID, 128) || !encode_operand(&gz1, m->dZ1, HID, batch, HID, 64) ||
-        !encode_operand(&gx, Xb, IN, batch, IN, 64) || !encode_operand(&gz2, m->dZ2, HID, batch, HID, 64) ||
-        !encode_operand(&gh1, m->H1, HID, batch, HID, 64) || !encode_operand(&gh2, m->H2, HID, batch, HID, 64) ||
-        !encode_operand(&gdy, m->dY, DY_STRIDE, batch, DY_STRIDE, 64))
-        return HGMM_ECUDA;
+    const bool maps =
+        m->maps && encode_operand(&bdy, m->dY, DY_STRIDE, batch, DY_STRIDE, 128) &&
+        encode_operand(&bw3, m->W3T, DY_STRIDE, HID, DY_STRIDE, HID) &&
+        encode_operand(&bw2, m->W2T, HID, HID, HID, HID) && encode_operand(&bz2, m->dZ2, HID, batch, HID, 128) &&
+        encode_operand(&bz1, m->dZ1, HID, batch, HID, 128) && encode_operand(&gz1, m->dZ1, HID, batch, HID, 64) &&
+        encode_operand(&gx, Xb, IN, batch, IN, 64) && encode_operand(&gz2, m->dZ2, HID, batch, HID, 64) &&
+        encode_operand(&gh1, m->H1, HID, batch, HID, 64) && encode_operand(&gh2, m->H2, HID, batch, HID, 64) &&
+        encode_operand(&gdy, m->dY, DY_STRIDE, batch, DY_STRIDE, 64);
     if (d_index) {
         k_gather<<<batch, 160, 0, s>>>(X, d_labels, d_index, n_rows, m->Xg, m->Lg, m->err);
         X = m->Xg;
@@ -774,12 +811,17 @@ int gradients_impl(hgmm_mlp* m, const uint16_t* d_x, const float* d_labels, cons
     k_loss<<<(batch + LOSS_ROWS - 1) / LOSS_ROWS, LOSS_THREADS, 0, s>>>(m->Y, L, batch, w_t, m->dY, m->dYf,
                                                                        m->loss_part, m->loss_cnt,
                                                                        d_loss ? d_loss : m->loss);
-    k_mlp_backward<<<(batch + 127) / 128, BW_THREADS, BW_SMEM, s>>>(bdy, bw3, bw2, bz2, bz1, m->H1, m->H2, batch,
-                                                                   m->err);
-    const int slices = wg_slices(batch), nchunks = (batch + COLSUM_ROWS - 1) / COLSUM_ROWS;
-    k_mlp_wgrad<<<WG_TILES * slices + nchunks, WG_THREADS, WG_SMEM, s>>>(gz1, gx, gz2, gh1, gh2, gdy, batch, slices,
-                                                                        wg_chunks(batch), m->dZ1, m->dZ2, m->dYf,
-                                                                        m->ws, m->part, m->err);
+    const int nchunks = (batch + COLSUM_ROWS - 1) / COLSUM_ROWS;
+    const int slices = maps ? wg_slices(batch) : 1;
+    if (maps) {
+        k_mlp_backward<<<(batch + 127) / 128, BW_THREADS, BW_SMEM, s>>>(bdy, bw3, bw2, bz2, bz1, m->H1, m->H2, batch,
+                                                                       m->err);
+        k_mlp_wgrad<<<WG_TILES * slices + nchunks, WG_THREADS, WG_SMEM, s>>>(
+            gz1, gx, gz2, gh1, gh2, gdy, batch, slices, wg_chunks(batch), m->dZ1, m->dZ2, m->dYf, m->ws, m->part, m->err);
+    } else {
+        if (int rc = backward_gemms(m, X, batch, s)) return rc;
+        k_colsum<<<nchunks, WG_THREADS, 0, s>>>(m->dZ1, m->dZ2, m->dYf, batch, m->part);
+    }
     constexpr int ug = UPDATE_CTAS + UPDATE_BIAS_CTAS;
     if (lr) {
         m->step += 1;
@@ -824,7 +866,8 @@ int hgmm_mlp_create(int32_t max_batch, hgmm_mlp** out) {
                 malloc_into(m, &m->loss_part, (B + LOSS_ROWS - 1) / LOSS_ROWS) && malloc_into(m, &m->loss_cnt, 1) && malloc_into(m, &m->err, 1) &&
                 malloc_into(m, &m->prop_x, IN) && malloc_into(m, &m->prop_fr, 2 * HGMM_FRAME_DOUBLES) &&
                 malloc_into(m, &m->prop_y, 16);
-    m->ws_cap = (long long)WG_MAX_SLICES * WS_STRIDE;
+    // the fused launch's slices, or without tensor maps the gradients and dW1's 16 slices
+    m->ws_cap = std::max<long long>(WG_MAX_SLICES * WS_STRIDE, WS_STRIDE + 16ll * HID * IN);
     good = good && malloc_into(m, &m->ws, size_t(m->ws_cap));
     good = good && set_gemm_smem();
     if (!good) {
@@ -950,6 +993,12 @@ int hgmm_pose_encode(const double* d_T, const double* d_frames, int32_t n, float
     if (!d_T || !d_frames || !d_labels || n < 1) return HGMM_EINVAL;
     k_encode<<<(n + 127) / 128, 128, 0, static_cast<cudaStream_t>(stream)>>>(d_T, d_frames, n, d_labels);
     return cudaGetLastError() == cudaSuccess ? HGMM_OK : HGMM_ECUDA;
+}
+
+int hgmm_debug_mlp_maps(hgmm_mlp* m, int32_t enable) {
+    if (!m) return HGMM_EINVAL;
+    m->maps = enable != 0;
+    return HGMM_OK;
 }
 
 int hgmm_debug_gemm(const uint16_t* d_A, int64_t a_m, int64_t a_k, const uint16_t* d_B, int64_t b_n,

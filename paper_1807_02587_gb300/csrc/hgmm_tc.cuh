@@ -5,8 +5,7 @@
 // Two kernels compute a 128 x BN tile per CTA with the accumulator in
 // tensor memory (TMEM):
 //
-// k_gemm_tma (both operands stored with K contiguous: the forward pass):
-// warp-specialised.  One thread of warp 0 streams the operand tiles into a
+// k_gemm_tma (both operands stored with K contiguous): warp-specialised.  One thread of warp 0 streams the operand tiles into a
 // ring of shared-memory stages with TMA (cp.async.bulk.tensor, 128-byte
 // swizzle, completion counted on each stage's "full" mbarrier); one thread
 // of warp 1 waits for each full stage, issues the tcgen05.mma of its four
@@ -14,8 +13,7 @@
 // hands the stage back to the producer; after the last stage its commit on
 // the "done" mbarrier releases the four epilogue warps.
 //
-// k_gemm_bf16 (any operand layout: the weight gradients read activations
-// transposed, without a copy): all 128 threads stage operands with
+// k_gemm_bf16 (any operand layout, and K slices): all 128 threads stage operands with
 // cp.async into the canonical no-swizzle K-major layout (8-row x 16-byte
 // core matrices, adjacent along K 128 bytes apart, 8-row groups 1024 bytes
 // apart, 64 K-elements per stage) in a ring of GEMM_STAGES stages filled
@@ -27,6 +25,10 @@
 // MMAs in flight, frees its TMEM and returns.  The epilogue reads the
 // accumulator with tcgen05.ld (warp w owns TMEM lanes 32w..32w+31, i.e. tile
 // rows) and applies one of the fused epilogues below.
+//
+// The network's own passes are fused (k_mlp_forward, hgmm_train.cuh); these
+// kernels serve the checking entry point and, where tensor maps cannot be
+// encoded, the network's products one by one.
 #pragma once
 
 #include "hgmm_async.cuh"
@@ -167,6 +169,7 @@ enum Epilogue : int {
     EPI_F32 = 0,             // out_f32[m, n] = acc
     EPI_BIAS_F32 = 1,        // out_f32[m, n] = acc + bias[n]
     EPI_BIAS_RELU_BF16 = 2,  // out_bf16[m, n] = bf16(max(acc + bias[n], 0))
+    EPI_MASK_BF16 = 3,       // out_bf16[m, n] = bf16(mask[m, n] > 0 ? acc : 0)
 };
 
 struct GemmArgs {
@@ -180,6 +183,8 @@ struct GemmArgs {
     int n_store;          // columns n >= n_store are not written
     int epi;
     const float* bias;
+    const __nv_bfloat16* mask;
+    long long mask_m;
     float* out_f32;
     __nv_bfloat16* out_bf16;
     long long o_m, o_n;   // out[m * o_m + n * o_n]
@@ -257,6 +262,9 @@ __device__ __forceinline__ void epilogue16(const GemmArgs& g, float* outf, int m
         switch (g.epi) {
             case EPI_F32: outf[o] = x; break;
             case EPI_BIAS_F32: outf[o] = x + g.bias[n]; break;
+            case EPI_MASK_BF16:
+                g.out_bf16[o] = __float2bfloat16_rn(__bfloat162float(g.mask[m * g.mask_m + n]) > 0.f ? x : 0.f);
+                break;
             default:
                 x += g.bias[n];
                 g.out_bf16[o] = __float2bfloat16_rn(x > 0.f ? x : 0.f);
@@ -273,7 +281,7 @@ __device__ __forceinline__ void epilogue32(const GemmArgs& g, float* outf, int m
     const bool bf = g.epi == EPI_BIAS_RELU_BF16;
     const int lim = min(g.N, g.n_store);
     const long long o = m * g.o_m + n0c;
-    const bool vec = n0c + 32 <= lim && g.o_n == 1 &&
+    const bool vec = n0c + 32 <= lim && g.o_n == 1 && g.epi != EPI_MASK_BF16 &&
                      ((bf ? reinterpret_cast<uintptr_t>(g.out_bf16 + o) : reinterpret_cast<uintptr_t>(outf + o)) &
                       15u) == 0 &&
                      (g.epi == EPI_F32 || (reinterpret_cast<uintptr_t>(g.bias + n0c) & 15u) == 0);

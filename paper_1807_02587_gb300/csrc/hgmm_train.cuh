@@ -347,6 +347,13 @@ __device__ __forceinline__ void colsum_chunk(const bf16* __restrict__ dZ1, const
     p[2 * HID] = sy;
 }
 
+// The column sums alone (without tensor maps).
+__global__ void __launch_bounds__(WG_THREADS)
+k_colsum(const bf16* __restrict__ dZ1, const bf16* __restrict__ dZ2, const float* __restrict__ dYf, int batch,
+         float* __restrict__ part) {
+    colsum_chunk(dZ1, dZ2, dYf, batch, int(blockIdx.x), part);
+}
+
 __global__ void __launch_bounds__(WG_THREADS, 1)
 k_mlp_wgrad(const __grid_constant__ CUtensorMap tmZ1, const __grid_constant__ CUtensorMap tmX,
             const __grid_constant__ CUtensorMap tmZ2, const __grid_constant__ CUtensorMap tmH1,
