@@ -96,7 +96,10 @@ typedef struct hgmm_params {
  * in a fixed owner CTA) instead of separate E-step and M-step launches per
  * iteration.  The result is the same bit for bit; under a CUDA graph the
  * separate launches are faster on the bench workload, so this is off by
- * default. */
+ * default.  It has no effect on levels that hgmm_build builds in its one
+ * cooperative launch (precision 0, up to about 400,000 points, the first four
+ * levels), which launch nothing per iteration, nor on levels whose parents
+ * each run their EM in one CTA. */
 #define HGMM_FLAG_EM_COOPERATIVE 1
 
 /* Per-node record written by hgmm_tree_export: 16 float64 per node,
@@ -138,8 +141,8 @@ int hgmm_build(hgmm_tree* t, const float* d_points, int64_t n, int32_t depth,
  * The node moments are exact fixed-point sums of every point's moments, so
  * the result does not depend on the order of the source points, nor on how
  * many CTAs the launch has; a source of 2^20 points or more (up to
- * max_points) is sorted by its first-round nodes into the tree's free point
- * buffer for the remaining rounds, and one of 2^21 points or more runs with
+ * max_points) with more than one round is first put into spatial order in the
+ * tree's free point buffer, and one of 2^21 points or more runs with
  * three CTAs per SM instead of two (more warps for a throughput-bound
  * descent; the same bits).
  * Errors: HGMM_EINVAL, HGMM_ECUDA; singular normal equations are reported by
@@ -184,7 +187,7 @@ typedef struct hgmm_descent {
  * Eq. 9-16 solve (or the full Eq. 7 one, with second moments as well) and
  * T <- dT T.  One launch per round for the descent (a
  * warp-synchronous depth-first search per point with a bounded stack), one
- * for the node terms, one for the solve.  hgmm_register_objective and
+ * for the node terms, whose last CTA solves.  hgmm_register_objective and
  * hgmm_debug_reg_moments report on the last round.  Errors: as hgmm_register;
  * HGMM_EINVAL for an unknown mode or tau outside [0, 1]. */
 int hgmm_register_descent(hgmm_tree* t, const float* d_src, int64_t n, const double* d_T_init,
@@ -202,7 +205,7 @@ int hgmm_sync(hgmm_tree* t, void* stream);
  * host).  The first call of a shape (point counts, depth, parameters, rounds,
  * with or without h_T_init) captures the build and the registration into a
  * CUDA graph on a stream the tree owns; later calls of that shape replay it
- * (one launch instead of about 80); another shape replaces it.  Not while
+ * (one launch instead of 4 to about 90); another shape replaces it.  Not while
  * profiling or tracing.  Synchronous.  Errors: as hgmm_build, hgmm_register,
  * hgmm_sync. */
 int hgmm_register_pair_host(hgmm_tree* t, const float* h_tgt, int64_t n_tgt,

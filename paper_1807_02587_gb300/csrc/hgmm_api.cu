@@ -311,7 +311,7 @@ int hgmm_register_pair_host(hgmm_tree* t, const float* h_tgt, int64_t n_tgt, con
     // the build and the registration as one CUDA graph, captured for this
     // shape on the tree's own stream (the caller's may be the legacy default
     // stream, which cannot be captured) and replayed on the caller's stream:
-    // the ~80 kernels of a step cost one launch.  Not while profiling or
+    // the 4 to about 90 kernels of a step cost one launch.  Not while profiling or
     // tracing (their events and stamps are per launch).
     const int64_t key[5] = {n_tgt, n_src, depth, iters, h_T_init ? 1 : 0};
     bool use_graph = !t->prof_on && !t->trace_on && !t->pair_graph_failed;

@@ -1531,13 +1531,13 @@ __device__ __forceinline__ long long to_fix(float v) {
 // smallest unit it ever loads): per pair of children ten constants of both
 // (-mu_x, -mu_y, -mu_z, -C, W00, W10, W11, W20, W21, W22: the operands of
 // packed FP32x2 arithmetic) in five float4, then the children's stop flags as
-// a bit mask, and padding.  The shared-memory loads bound the descent of large
-// sources: each 16-byte load returns 512 bytes to a warp, four cycles of the
-// SM's 128-byte path, and node records of three float4 took 24 of them per
-// level (16.8M points: 3,450 warps per SM x 3.5 levels x 24 x 4 cycles = 560 us,
-// measured 567 us per round).  A block is 20 loads and one word.  Its stride of
-// 21 float4 puts the same constant of eight consecutive blocks on different
-// banks.
+// a bit mask, and padding: 20 loads and one word per block, where node records of
+// three float4 took 24, and packed arithmetic on what they return.  The stride
+// of 21 float4 puts the same constant of eight consecutive blocks on different
+// banks.  No single unit bounds the descent of large sources: 8M points keep the
+// load path 58 % busy (shared memory 47), the issue slots 55, ALU, FMA and FP64
+// pipes 34 / 31 / 29, with 24 warps per SM waiting mostly for the points and the
+// deeper levels' blocks (counters of the whole registration, 10 rounds).
 constexpr int STAGED_NODES = 584;  // levels 0..2 (8 + 64 + 512 nodes) live in shared memory
 constexpr int BLOCK_F4 = REG_BLOCK_F4;
 constexpr int STAGED_F4 = BLOCK_F4 * STAGED_NODES / 8;
@@ -1712,8 +1712,9 @@ __device__ __forceinline__ void add_moments(int chosen, long long (&q)[4], unsig
 // levels are where most points stop on large planar structures, so this
 // keeps thousands of warps from serialising on a few hot addresses.
 // Two points per lane that share a block's loads were tried: 16M points in
-// node order 459 us a round against 466, but 11.5 against 9.9 us at 4,000
-// points and 1,195 against 805 for a round in random order.
+// node order 459 us a round against 466 (the loads alone do not bound it), but
+// 11.5 against 9.9 us at 4,000 points and 1,195 against 805 for a round in random
+// order.
 // STAGED: a tree whose levels are all staged (up to depth 3).  Without it such
 // trees pay for the branch to the cached levels, where a small source's round
 // is one latency chain: 30 rounds at depth 2 take 1,000 / 10,000 / 100,000
