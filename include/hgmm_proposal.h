@@ -159,7 +159,7 @@ int hgmm_debug_mlp_maps(hgmm_mlp* m, int32_t enable);
  * (element strides; for each operand either the k stride or the row stride
  * is 1, the other a multiple of 8; a K stride of 1 needs K % 8 == 0, a row
  * stride of 1 needs the row count % 8 == 0; 16-byte aligned bases).  N <= 16
- * runs 128 x 16 tiles, larger N 128 x 256 tiles.  Errors: HGMM_EINVAL. */
+ * runs 128 x 16 tiles, larger N 128 x 128 tiles.  Errors: HGMM_EINVAL. */
 int hgmm_debug_gemm(const uint16_t* d_A, int64_t a_m, int64_t a_k, const uint16_t* d_B, int64_t b_n,
                     int64_t b_k, int32_t M, int32_t N, int32_t K, float* d_out, void* stream);
 
